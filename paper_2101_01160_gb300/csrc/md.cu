@@ -1057,10 +1057,10 @@ int observe(md_system *s, ObsArgs a) {
     a.complete = s->phase_half;
     const int nthr = 256;
     const int nblk = s->nslots / nthr;
-    if (s->prec == MD_FP64)
-        k_observe<double><<<nblk, nthr, 0, s->st>>>(s->sd, a);
-    else
-        k_observe<float><<<nblk, nthr, 0, s->st>>>(s->sd, a);
+    const bool pe = a.epart || a.fabs_sum;
+    const auto k = s->prec == MD_FP64 ? (pe ? k_observe<double, true> : k_observe<double, false>)
+                                      : (pe ? k_observe<float, true> : k_observe<float, false>);
+    k<<<nblk, nthr, 0, s->st>>>(s->sd, a);
     MD_CUDA_TRY(cudaGetLastError());
     s->phase_half = 0;
     return MD_OK;

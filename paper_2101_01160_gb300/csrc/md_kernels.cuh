@@ -1238,7 +1238,12 @@ struct ObsArgs {
     unsigned snap_mask;            // sampling slots whose snapshot is taken now
 };
 
-template <typename T>
+// kPE: the potential energy and the force magnitudes are wanted too (md_energy,
+// md_forces).  They are FP64 sums with a square root per pair on a pipe of 1/64
+// of the FP32 rate, so a call that only completes the half kick (state, raw and
+// snapshot readouts) leaves them out: 5.7M particles 3.86 -> about 0.1 ms, the force
+// bits the same (lj_pair_acc).
+template <typename T, bool kPE>
 __global__ void k_observe(SysDev S, ObsArgs A) {
     using V = typename V2<T>::type;
     const int set = S.ctl->set, cur = S.ctl->cur;
@@ -1258,7 +1263,7 @@ __global__ void k_observe(SysDev S, ObsArgs A) {
             // force readout, the potential energy); a snapshot or state
             // readout needs none
             if (A.complete || A.fx || A.epart)
-                lj_stencil<T, true>(R, pos, S.cell_start, cpk, oi, slot, fx, fy, pe, fa);
+                lj_stencil<T, kPE>(R, pos, S.cell_start, cpk, oi, slot, fx, fy, pe, fa);
             if (A.complete) {
                 const T hk = rd<T>(R.hk, R.hkf);
                 v.x = axpyT(v.x, hk, fx);
