@@ -380,10 +380,10 @@ int mdlg_bin(const md_snapshot *t0, const md_snapshot *t1, int64_t n, int32_t lx
  * same results bit for bit (same launch shape).  The per-CTA moment
  * partials go to one fixed 32 KiB device array inside the library (every
  * GPU that loads the library holds it until the process exits), room for
- * 2048 CTAs; the grid is
- * min(ceil(n/256), 8 x SM count), 1216 CTAs on a 152-SM GPU, and a call
- * that would need more returns MD_E_LIMIT.  The outputs are cleared with
- * cudaMemsetAsync on `stream`; the array needs no clearing.  The array is
+ * 2048 CTAs; the grid is one wave of resident CTAs, at most 8 per SM (1216
+ * on a 152-SM GPU), and a call that would need more returns MD_E_LIMIT.  Up
+ * to 32768 particles take a single cluster and no scratch.  The outputs are
+ * cleared by a kernel on `stream`; the array needs no clearing.  The array is
  * shared by every call on a device: calls that may run at the same time on
  * the device (other streams, other host threads, without ordering between
  * them) race on it and can return wrong moments, so order them.  The first

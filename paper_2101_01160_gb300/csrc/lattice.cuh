@@ -24,31 +24,6 @@ __device__ __forceinline__ long long lattice_cell(double x, double dxl, int lx) 
     return l;
 }
 
-// The same lattice cell, floor(RN(x / dxl)) mod lx, with the division
-// replaced by a product with inv = RN(1 / dxl) wherever that cannot change
-// the result.  q = RN(x * inv) and RN(x / dxl) both lie within |q| 2^-51 of
-// the exact quotient x / dxl (each is one or two roundings of relative size
-// 2^-53 away from it), so when q is more than |q| 2^-50 from the nearest
-// integer no integer separates them and floor(q) is the answer; otherwise
-// (points on or next to a lattice line, x = 0, and |q| < 2^-900, where
-// underflow would void the relative bounds) the division is done.
-// Bit-identical to lattice_cell for every finite x; one FP64 product, a rint
-// and a compare in place of a division on all but those cases.
-__device__ __forceinline__ long long lattice_cell_mul(double x, double dxl, double inv, int lx) {
-    const double q = __dmul_rn(x, inv);
-    const double t = rint(q);
-    const double fq = fabs(q);
-    double f;
-    if (fq > 0x1p-900 && fabs(__dsub_rn(q, t)) > __dmul_rn(fq, 0x1p-50))
-        f = floor(q);
-    else
-        f = floor(__ddiv_rn(x, dxl));
-    long long l = (long long)f;
-    l %= lx;
-    if (l < 0) l += lx;
-    return l;
-}
-
 // The lattice cell of the position encoded as (cell coordinate c, offset
 // off), floor(RN(RN(c*h + off) / dxl)) mod lx as lattice_cell computes it,
 // decided in FP32 wherever FP32 provably gives the same cell.  With a =
@@ -70,43 +45,65 @@ static __device__ __noinline__ int lattice_cell_slow(int c, double off, double h
     return (int)lattice_cell(cell_position(c, h, off), dxl, lx);
 }
 
+// (float)c for 0 <= c < 2^23, from the float bits of 2^23 + c: two ordinary
+// operations in place of a conversion (conversions, like rint and floor, run
+// on the special-function pipe at a quarter of the rate).
+__device__ __forceinline__ float small_int_to_float(int c) {
+    return __fsub_rn(__int_as_float(0x4b000000 | c), 8388608.0f);
+}
+
+// The decision of lattice_cell_f32 without the reduction modulo lx: the
+// quotient's floor where FP32 decides it, else the FP64 cell (already
+// reduced; callers reduce either).  0 <= c < 2^23.  Adding 1.5 * 2^23 rounds
+// |q| < 2^22 to the nearest integer in its low bits.
 template <typename T>
-__device__ __forceinline__ int lattice_cell_f32(int c, T off, double h, float hf, double dxl, float invf,
-                                                int lx) {
-    const float a = __fmul_rn((float)c, hf);
+__device__ __forceinline__ int lattice_floor_f32(int c, T off, double h, float hf, double dxl, float invf,
+                                                 int lx) {
+    const float a = __fmul_rn(small_int_to_float(c), hf);
     const float o = (float)off;
     const float q = __fmul_rn(__fadd_rn(a, o), invf);
     const float S = __fmul_rn(__fadd_rn(fabsf(a), fabsf(o)), invf);
-    if (S < 0x1p22f && fabsf(__fsub_rn(q, rintf(q))) > __fmul_rn(S, 0x1p-20f)) {
-        int l = __float2int_rd(q);   // |q| < 2^22: floor in one 32-bit conversion
-        // positions within a box edge of the box need one wrap; others the
-        // general reduction
-        if (l < 0) l += lx;
-        else if (l >= lx) l -= lx;
-        if (l < 0 || l >= lx) {
-            l %= lx;
-            if (l < 0) l += lx;
-        }
-        return l;
-    }
+    const float big = __fadd_rn(q, 12582912.0f);
+    const float d = __fsub_rn(q, __fsub_rn(big, 12582912.0f));   // q - rint(q), exact
+    if (S < 0x1p22f && fabsf(d) > __fmul_rn(S, 0x1p-20f))
+        return __float_as_int(big) - 0x4b400000 - (d < 0.0f ? 1 : 0);
     return lattice_cell_slow(c, (double)off, h, dxl, lx);
 }
 
-// Splits a linear cell index c = cy * ncell + cx (0 <= cx, cy < ncell,
-// ncell^2 < 2^31) without an integer division: the float estimate of
-// c / ncell (< 46341) carries a relative error below 2^-22, so it is off by
-// at most one, and one multiply-subtract with a fix-up makes it exact.
-__device__ __forceinline__ void split_cell(int c, int ncell, float inv_ncell, int &cx, int &cy) {
-    int y = (int)__fmul_rz((float)c, inv_ncell);
-    int x = c - y * ncell;
-    if (x < 0) {
-        --y;
-        x += ncell;
-    } else if (x >= ncell) {
-        ++y;
-        x -= ncell;
+template <typename T>
+__device__ __forceinline__ int lattice_cell_f32(int c, T off, double h, float hf, double dxl, float invf,
+                                                int lx) {
+    int l = lattice_floor_f32<T>(c, off, h, hf, dxl, invf, lx);
+    // positions within a box edge of the box need one wrap; others the
+    // general reduction
+    if (l < 0) l += lx;
+    else if (l >= lx) l -= lx;
+    if (l < 0 || l >= lx) {
+        l %= lx;
+        if (l < 0) l += lx;
     }
-    cx = x;
+    return l;
+}
+
+// Division of 0 <= c < 2^31 by an invariant ncell >= 1 as one high product
+// and a shift (Granlund and Montgomery 1994): with s = ceil(log2 ncell) and
+// m = floor(2^(31+s) / ncell) + 1 < 2^32 + 1, c m / 2^(31+s) exceeds c /
+// ncell by less than c / 2^(31+s) < 1 / ncell, so the floors agree.
+struct CellDiv {
+    uint32_t mul;
+    int32_t shift;     // of the high 32 bits of c * mul; -1: ncell = 1
+};
+inline CellDiv cell_div(int ncell) {
+    int s = 0;
+    while ((1ll << s) < ncell) ++s;
+    if (s == 0) return CellDiv{0u, -1};
+    return CellDiv{(uint32_t)((1ull << (31 + s)) / (uint64_t)ncell + 1ull), s - 1};
+}
+
+// Splits a linear cell index c = cy * ncell + cx, 0 <= c < 2^31.
+__device__ __forceinline__ void split_cell(int c, int ncell, CellDiv D, int &cx, int &cy) {
+    const int y = D.shift < 0 ? c : (int)(__umulhi((uint32_t)c, D.mul) >> D.shift);
+    cx = c - y * ncell;
     cy = y;
 }
 
@@ -120,11 +117,20 @@ __device__ __forceinline__ int lattice_shift_near(int d, int lx) {
 
 // Lattice displacement reduced to the nearest periodic image, in
 // (-lx/2, lx/2].
-__device__ __forceinline__ long long lattice_shift(long long d, int lx) {
+static __device__ __noinline__ int lattice_shift(int d, int lx) {
     d %= lx;
     if (d < 0) d += lx;
     if (d > lx / 2) d -= lx;
     return d;
+}
+
+// Nearest image of the difference d of two lattice_floor_f32 values: one wrap
+// for positions within a box edge of the box, the general reduction else.
+__device__ __forceinline__ int lattice_shift_floors(int d, int lx) {
+    const int half = lx / 2, low = half + 1 - lx;   // (-lx/2, lx/2] as integers
+    if (d > half) d -= lx;
+    if (d < low) d += lx;
+    return d > half || d < low ? lattice_shift(d, lx) : d;
 }
 
 __device__ __forceinline__ double nearest_image(double d, double L) {

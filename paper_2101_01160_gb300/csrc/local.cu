@@ -28,7 +28,8 @@ struct LocSnap {
 
 struct OccParams {
     int ncell, lx, W;
-    float inv_ncell, hf, invf;
+    CellDiv div;
+    float hf, invf;
     double h, dxl;
 };
 
@@ -38,8 +39,8 @@ template <typename T>
 __device__ __forceinline__ int occ_index(const OccParams &P, int c0, T ox0, T oy0, int c1, T ox1, T oy1,
                                          int &oi) {
     int cx0, cy0, cx1, cy1;
-    split_cell(c0, P.ncell, P.inv_ncell, cx0, cy0);
-    split_cell(c1, P.ncell, P.inv_ncell, cx1, cy1);
+    split_cell(c0, P.ncell, P.div, cx0, cy0);
+    split_cell(c1, P.ncell, P.div, cx1, cy1);
     const int sx1 = lattice_cell_f32<T>(cx1, ox1, P.h, P.hf, P.dxl, P.invf, P.lx);
     const int sy1 = lattice_cell_f32<T>(cy1, oy1, P.h, P.hf, P.dxl, P.invf, P.lx);
     const int vx = lattice_shift_near(sx1 - lattice_cell_f32<T>(cx0, ox0, P.h, P.hf, P.dxl, P.invf, P.lx), P.lx);
@@ -243,7 +244,7 @@ extern "C" int mdlg_site_occupation(const md_snapshot *t0, const md_snapshot *t1
     P.W = W;
     P.h = t0->h;
     P.dxl = (double)t0->ncell * t0->h / (double)lx;
-    P.inv_ncell = 1.0f / (float)t0->ncell;
+    P.div = cell_div(t0->ncell);
     P.hf = (float)t0->h;
     P.invf = (float)(1.0 / P.dxl);
     auto al16 = [](const void *p) { return ((uintptr_t)p & 15u) == 0; };

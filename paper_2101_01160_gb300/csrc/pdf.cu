@@ -82,7 +82,8 @@ template <> struct PdfVec4<double> {
 
 struct DispParams {
     int ncell, nbins;
-    float inv_ncell, hf, invwf;
+    CellDiv div;
+    float hf, invwf;
     double h, w;
 };
 
@@ -91,8 +92,8 @@ template <typename T>
 __device__ __forceinline__ void disp_count(const DispParams &P, int c0, int c1, T x0, T y0, T x1, T y1,
                                            unsigned *sh_bins, unsigned &my_out) {
     int cc0[2], cc1[2];
-    split_cell(c0, P.ncell, P.inv_ncell, cc0[0], cc0[1]);
-    split_cell(c1, P.ncell, P.inv_ncell, cc1[0], cc1[1]);
+    split_cell(c0, P.ncell, P.div, cc0[0], cc0[1]);
+    split_cell(c1, P.ncell, P.div, cc1[0], cc1[1]);
     const T o0[2] = {x0, y0}, o1[2] = {x1, y1};
     const long long lo = -(long long)(P.nbins / 2), hi = (long long)P.nbins - P.nbins / 2;
 #pragma unroll
@@ -215,7 +216,7 @@ extern "C" int mdlg_disp_hist(const md_snapshot *t0, const md_snapshot *t1, int6
     P.w = width;
     P.hf = (float)t0->h;
     P.invwf = (float)(1.0 / width);
-    P.inv_ncell = 1.0f / (float)t0->ncell;
+    P.div = cell_div(t0->ncell);
     const size_t smem = sizeof(unsigned) * nbins;
     auto al16 = [](const void *p) { return ((uintptr_t)p & 15u) == 0; };
     const bool vec = al16(a.cell) && al16(a.ox) && al16(a.oy) && al16(b.cell) && al16(b.ox) && al16(b.oy);
