@@ -33,20 +33,21 @@ __global__ void k_feq_gaussian(double a2, double ux, double uy, int W, double *P
 }
 
 // One CTA per lattice velocity; its threads share the Poisson terms
-// c = cmin..cmax (terms outside the window weigh < 1e-16 in total: the
-// Poisson tails beyond 12 sqrt(lambda) + 20 of the mean).  Fixed-order
-// reduction, so the result is reproducible.
+// c = cmin, cmin + stride, .. (wsg_terms; terms outside the window weigh <
+// 1e-16 in total: the Poisson tails beyond 12 sqrt(lambda) + 20 of the mean).
+// Fixed-order reduction, so the result is reproducible.
 constexpr int WSG_THREADS = 128;
 
 __global__ void __launch_bounds__(WSG_THREADS) k_feq_wsg(double a2, double lam, double ux, double uy,
-                                                         int W, int cmin, int cmax, double *P) {
+                                                         int W, int cmin, int stride, int terms, double *P) {
     __shared__ double red[WSG_THREADS];
     const int side = 2 * W + 1;
     const int i = blockIdx.x;
     const double vx = (double)(i % side - W) - ux, vy = (double)(i / side - W) - uy;
     double acc = 0.0;
-    for (int c = cmin + (int)threadIdx.x; c <= cmax; c += WSG_THREADS) {
-        const double w = poisson_weight(c, lam);
+    for (int j = (int)threadIdx.x; j < terms; j += WSG_THREADS) {
+        const int c = cmin + j * stride;
+        const double w = (double)stride * poisson_weight(c, lam);
         const double var = a2 * ((double)c + 1.0) / (lam + 1.0);
         acc += w * (cell_gauss_1d(vx, var) * cell_gauss_1d(vy, var));
     }
@@ -124,7 +125,7 @@ int feq_wsg(double a2, double lambda, double ux, double uy, int32_t W, double *P
     if (!P_out) return fail(MD_E_ARG, "feq_wsg: P_out is NULL");
     const int nb = (2 * W + 1) * (2 * W + 1);
     k_feq_wsg<<<nb, WSG_THREADS, 0, (cudaStream_t)stream>>>(a2, lambda, ux, uy, W, wsg_cmin(lambda),
-                                                            wsg_cmax(lambda), P_out);
+                                                            wsg_stride(lambda), wsg_terms(lambda), P_out);
     MD_CUDA_TRY(cudaGetLastError());
     return MD_OK;
 }

@@ -96,25 +96,25 @@ struct FeqArgs {
 // Normalised measured equilibrium (Eq. theory_feq per particle), batch-means
 // error bars over blocks of windows, optional symmetric-set averaging
 // (Sec. 5), moments mu2, mu4 and a^2 (Eq. a2_n_ua).  One CTA.
-constexpr int FEQ_THREADS = 128;
+constexpr int FEQ_THREADS = 256;
+
+// Sums of the moment partials of groups [g0, g1), in thread 0 (both f_eq
+// kernels: the same threads, strides and tree, so the same bits).
+__device__ __forceinline__ void feq_moments(const double *mom, int g0, int g1, int n_lg, int lg, double &m2, double &m4) {
+    const double2 *p = reinterpret_cast<const double2 *>(mom) + lg;
+    m2 = m4 = 0.0;
+#pragma unroll 8
+    for (int g = g0 + (int)threadIdx.x; g < g1; g += FEQ_THREADS) {
+        const double2 m = p[(long long)g * n_lg];
+        m2 += m.x;
+        m4 += m.y;
+    }
+    block_sum2(m2, m4);
+}
 
 __global__ void __launch_bounds__(FEQ_THREADS) k_feq_measured(FeqArgs A) {
-    __shared__ double s2[FEQ_THREADS], s4[FEQ_THREADS];
-    double m2 = 0.0, m4 = 0.0;
-    for (int g = A.g0 + threadIdx.x; g < A.g1; g += blockDim.x) {
-        m2 += A.mom[((long long)g * A.n_lg + A.lg) * 2];
-        m4 += A.mom[((long long)g * A.n_lg + A.lg) * 2 + 1];
-    }
-    s2[threadIdx.x] = m2;
-    s4[threadIdx.x] = m4;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) {
-            s2[threadIdx.x] += s2[threadIdx.x + o];
-            s4[threadIdx.x] += s4[threadIdx.x + o];
-        }
-        __syncthreads();
-    }
+    double m2, m4;
+    feq_moments(A.mom, A.g0, A.g1, A.n_lg, A.lg, m2, m4);
     const double samples = A.n * (double)A.nwin;
     const int side = 2 * A.W + 1;
     for (int i = threadIdx.x; i < A.nb; i += blockDim.x) {
@@ -153,8 +153,8 @@ __global__ void __launch_bounds__(FEQ_THREADS) k_feq_measured(FeqArgs A) {
     }
     if (threadIdx.x == 0) {
         double *st = A.out + 2 * A.nb;
-        const double mu2 = samples > 0 ? s2[0] / (2.0 * samples) : 0.0;
-        const double mu4 = samples > 0 ? s4[0] / (2.0 * samples) : 0.0;
+        const double mu2 = samples > 0 ? m2 / (2.0 * samples) : 0.0;
+        const double mu4 = samples > 0 ? m4 / (2.0 * samples) : 0.0;
         st[0] = mu2;
         st[1] = mu4;
         st[2] = mu2 / (A.dx_eff * A.dx_eff);
@@ -197,16 +197,24 @@ __global__ void k_nc_of_id(SysDev S, int32_t *nc_of_id) {
 
 
 // ---------------------------------------------------------------- batched f_eq stage
-// For every replica, on the device (k_feq_params: the moments and lambda;
-// k_feq_terms: the WSG sums over the Poisson window, split over CTAs;
-// k_feq_batch: one CTA per replica for the rest): the measured equilibrium
+// For every replica, on the device, one CTA each: the measured equilibrium
 // (Eq. theory_feq per particle, optionally averaged over symmetric sets),
 // the moments mu2, mu4 and a^2 (Eq. a2_n_ua), lambda from Eq. (lambda_eq)
 // (root 2), the Gaussian (Eq. feq_gaussian) and WSG (Eq. f_eq_wsg)
 // equilibria at that a^2 and lambda, and their distance to the measured one
 // (max |difference| and Eq. kullback_leibler).
-constexpr int FEQB_THREADS = 128;
+//
+// What bounds it is the FP64 pipe (a warp instruction every 15 clocks of an
+// SM) and, for few replicas, the chain of its phases.  So the WSG sum takes
+// the strided window (at most 137 terms, wsg_stride), a term's exponentials
+// and error functions are evaluated at |v| = 1 .. W+1 only (u = 0: both
+// equilibria depend on |vx|, |vy|), one (term, point) per thread, the 2D
+// products are summed once per symmetric set {|vx|, |vy|}, and the Gaussian
+// is one more row of the table.  Measured: 256 replicas 291 -> 57 us, one
+// replica of 262,144 particles 123 -> 25 us (three kernels before).
+constexpr int FEQB_THREADS = FEQ_THREADS;
 constexpr int FEQB_STATS = 16;
+constexpr int FEQB_SPLIT = 8;     // partial sums over the terms per symmetric set
 
 struct FeqBatchArgs {
     const RepDev *reps;
@@ -218,44 +226,48 @@ struct FeqBatchArgs {
     double *out;                   // [nrep][3 nb + FEQB_STATS]
 };
 
-// The WSG sum of one replica is spread over up to FEQB_SPLIT CTAs of
-// FEQB_SPLIT_TERMS Poisson terms each (the last takes any remainder): with
-// lambda capped at 1e5 the window holds at most 7,631 terms, and a single
-// CTA would carry them all on one SM's FP64 pipe.
-constexpr int FEQB_SPLIT = 64;
-constexpr int FEQB_SPLIT_TERMS = FEQB_THREADS;
-
-// Splits that hold terms for lambda (the others add nothing).
-__device__ inline int feqb_splits_used(double lam) {
-    const int n = wsg_cmax(lam) - wsg_cmin(lam) + 1;
-    return min(FEQB_SPLIT, (n + FEQB_SPLIT_TERMS - 1) / FEQB_SPLIT_TERMS);
+// Sums of a and b over the CTA (fixed tree), in every thread.
+__device__ __forceinline__ void feqb_sum2(double &a, double &b, double *s_r) {
+    block_sum2(a, b);
+    if (threadIdx.x == 0) {
+        s_r[0] = a;
+        s_r[1] = b;
+    }
+    __syncthreads();
+    a = s_r[0];
+    b = s_r[1];
+    __syncthreads();
 }
 
-// Moments, a^2 and lambda of replica r into s_par = {mu2, a^2, lambda}
-// (every thread calls it; s_a, s_b: FEQB_THREADS doubles of scratch); with
-// out != nullptr thread 0 also writes the replica's statistics.
-__device__ void feqb_params(const FeqBatchArgs &A, const RepDev &R, int r, double *s_a, double *s_b,
-                            double *s_par, double *out) {
-    const int tid = threadIdx.x;
+__global__ void __launch_bounds__(FEQB_THREADS) k_feq_batch(FeqBatchArgs A) {
+    constexpr int ROWS = WSG_MAX_TERMS + 1;             // terms of a chunk and the Gaussian
+    constexpr int PTS = MD_MAX_W + 2;                   // |v| = 0 .. W + 1
+    constexpr int SETS = (MD_MAX_W + 1) * (MD_MAX_W + 2) / 2;
+    __shared__ double s_var[ROWS], s_w[ROWS], s_E[ROWS][PTS], s_R[ROWS][PTS];
+    __shared__ double s_part[SETS * FEQB_SPLIT], s_wsg[SETS], s_G[MD_MAX_W + 1], s_par[4], s_r[2];
+    __shared__ long long s_tot[(2 * MD_MAX_W + 1) * (2 * MD_MAX_W + 1)];
+    const int r = blockIdx.x, tid = threadIdx.x;
+    const RepDev &R = A.reps[r];
+    double *out = A.out + (long long)r * (3 * A.nb + FEQB_STATS);
+    const int32_t *hist = A.hist + ((((long long)r * A.n_lg + A.lg) * A.n_dx + A.dxi) * MD_NBLK) * A.nb;
     const double samples = (double)R.n * (double)A.nwin;
-    double m2 = 0.0, m4 = 0.0;
-    for (int g = R.pbase / 32 + tid; g < (R.pbase + R.cap) / 32; g += FEQB_THREADS) {
-        m2 += A.mom[((long long)g * A.n_lg + A.lg) * 2];
-        m4 += A.mom[((long long)g * A.n_lg + A.lg) * 2 + 1];
+    const int side = 2 * A.W + 1, W = A.W;
+    // counts of every class over the blocks, requested before the moments
+    for (int i = tid; i < A.nb; i += FEQB_THREADS) {
+        int v[MD_NBLK];
+#pragma unroll
+        for (int b = 0; b < MD_NBLK; ++b) v[b] = hist[b * A.nb + i];
+        long long t = 0;
+#pragma unroll
+        for (int b = 0; b < MD_NBLK; ++b) t += v[b];
+        s_tot[i] = t;
     }
-    s_a[tid] = m2;
-    s_b[tid] = m4;
-    __syncthreads();
-    for (int o = FEQB_THREADS / 2; o > 0; o >>= 1) {
-        if (tid < o) {
-            s_a[tid] += s_a[tid + o];
-            s_b[tid] += s_b[tid + o];
-        }
-        __syncthreads();
-    }
+    // moments, a^2, lambda
+    double m2, m4;
+    feq_moments(A.mom, R.pbase / 32, (R.pbase + R.cap) / 32, A.n_lg, A.lg, m2, m4);
     if (tid == 0) {
-        const double mu2 = samples > 0 ? s_a[0] / (2.0 * samples) : 0.0;
-        const double mu4 = samples > 0 ? s_b[0] / (2.0 * samples) : 0.0;
+        const double mu2 = samples > 0 ? m2 / (2.0 * samples) : 0.0;
+        const double mu4 = samples > 0 ? m4 / (2.0 * samples) : 0.0;
         const double dx = R.dxl[A.dxi];
         double lam = 0.0, st = 0.0;
         const double k = mu2 > 0 ? mu4 / (mu2 * mu2) : 0.0;
@@ -271,134 +283,103 @@ __device__ void feqb_params(const FeqBatchArgs &A, const RepDev &R, int r, doubl
                 st = 3.0;
             }
         }
-        s_par[0] = mu2;
         s_par[1] = mu2 / (dx * dx);
         s_par[2] = lam;
-        if (out) {
-            out[3 * A.nb + 0] = mu2;
-            out[3 * A.nb + 1] = mu4;
-            out[3 * A.nb + 2] = s_par[1];
-            out[3 * A.nb + 3] = lam;
-            out[3 * A.nb + 8] = (double)A.nwin;
-            out[3 * A.nb + 9] = samples;
-            out[3 * A.nb + 10] = (double)A.ovf[((long long)r * A.n_lg + A.lg) * A.n_dx + A.dxi];
-            out[3 * A.nb + 11] = dx;
-            out[3 * A.nb + 12] = st;
-        }
+        out[3 * A.nb + 0] = mu2;
+        out[3 * A.nb + 1] = mu4;
+        out[3 * A.nb + 2] = s_par[1];
+        out[3 * A.nb + 3] = lam;
+        out[3 * A.nb + 8] = (double)A.nwin;
+        out[3 * A.nb + 9] = samples;
+        out[3 * A.nb + 10] = (double)A.ovf[((long long)r * A.n_lg + A.lg) * A.n_dx + A.dxi];
+        out[3 * A.nb + 11] = dx;
+        out[3 * A.nb + 12] = st;
     }
     __syncthreads();
-}
-
-constexpr int FEQB_CPT = ((2 * MD_MAX_W + 1) * (2 * MD_MAX_W + 1) + FEQB_THREADS - 1) / FEQB_THREADS;
-
-// One CTA per replica: par[4 r + {0, 1, 2}] = mu2, a^2, lambda.
-__global__ void __launch_bounds__(FEQB_THREADS) k_feq_params(FeqBatchArgs A, double *par) {
-    __shared__ double s_a[FEQB_THREADS], s_b[FEQB_THREADS], s_par[4];
-    const int r = blockIdx.x;
-    feqb_params(A, A.reps[r], r, s_a, s_b, s_par, nullptr);
-    if (threadIdx.x < 3) par[4 * r + threadIdx.x] = s_par[threadIdx.x];
-}
-
-// Grid (replica, split): the split's Poisson terms c, one per thread in
-// chunks of FEQB_THREADS; the 1D factors of one term are evaluated once for
-// the 2W+1 displacements and shared by all classes (the 2D value is their
-// outer product); each class sums the chunk's terms in increasing c.
-// part[(r * FEQB_SPLIT + split) * nb + i] = the split's partial sum, written
-// by the splits that hold terms (feqb_splits_used); the others return at
-// once.
-__global__ void __launch_bounds__(FEQB_THREADS) k_feq_terms(FeqBatchArgs A, const double *par,
-                                                            double *part) {
-    __shared__ double s_w[FEQB_THREADS];
-    __shared__ double s_F[FEQB_THREADS][2 * MD_MAX_W + 1];
-    const int r = blockIdx.x, split = blockIdx.y, tid = threadIdx.x;
-    const double a2 = par[4 * r + 1], lam = par[4 * r + 2];
-    if (split >= feqb_splits_used(lam)) return;
-    const int side = 2 * A.W + 1;
-    double accW[FEQB_CPT];
-#pragma unroll
-    for (int q = 0; q < FEQB_CPT; ++q) accW[q] = 0.0;
-    const int cmin = wsg_cmin(lam), cmax = wsg_cmax(lam);
-    const int lo = cmin + split * FEQB_SPLIT_TERMS;
-    const int hi = split == FEQB_SPLIT - 1 ? cmax : min(cmax, lo + FEQB_SPLIT_TERMS - 1);
-    for (int c0 = lo; c0 <= hi && a2 > 0; c0 += FEQB_THREADS) {
-        const int c = c0 + tid;
-        if (c <= hi) {
-            s_w[tid] = poisson_weight(c, lam);
-            cell_gauss_row(a2 * ((double)c + 1.0) / (lam + 1.0), A.W, s_F[tid]);
+    const double a2 = s_par[1], lam = s_par[2];
+    const int nsets = (W + 1) * (W + 2) / 2;             // (lo <= hi): index hi (hi + 1) / 2 + lo
+    const int terms = wsg_terms(lam), cmin = wsg_cmin(lam), dc = wsg_stride(lam);
+    for (int e = tid; e < nsets; e += FEQB_THREADS) s_wsg[e] = 0.0;
+    for (int j0 = 0; j0 < terms && a2 > 0; j0 += WSG_MAX_TERMS) {
+        // rows 0 .. nt-1: terms of the chunk; row nt: the Gaussian
+        const int nt = min(WSG_MAX_TERMS, terms - j0);
+        for (int t = tid; t <= nt; t += FEQB_THREADS) {
+            const int c = cmin + (j0 + t) * dc;
+            s_w[t] = t < nt ? (double)dc * poisson_weight(c, lam) : 0.0;
+            s_var[t] = t < nt ? a2 * ((double)c + 1.0) / (lam + 1.0) : a2;
+            s_E[t][0] = 1.0;
+            s_R[t][0] = 0.0;
         }
         __syncthreads();
-        const int nterm = min(FEQB_THREADS, hi - c0 + 1);
+        for (int e = tid; e < (nt + 1) * (W + 1); e += FEQB_THREADS) {
+            const int t = e / (W + 1), q = e % (W + 1) + 1;
+            const double p = (double)q, var2 = 2.0 * s_var[t];
+            s_E[t][q] = exp(-(p * p) / var2);
+            s_R[t][q] = erf(p / sqrt(var2));
+        }
+        __syncthreads();
+        // 1D factors (cell_gauss_1d) of |v| = 0 .. W, in place over E: a pass
+        // to registers, then the write
+        constexpr int FPT = (ROWS * (MD_MAX_W + 1) + FEQB_THREADS - 1) / FEQB_THREADS;
+        double f[FPT];
 #pragma unroll
-        for (int q = 0; q < FEQB_CPT; ++q) {
-            const int i = tid + q * FEQB_THREADS;
-            if (i < A.nb) {
-                const int ix = i % side, iy = i / side;
-                double acc = accW[q];
-                for (int t = 0; t < nterm; ++t) acc += s_w[t] * (s_F[t][ix] * s_F[t][iy]);
-                accW[q] = acc;
+        for (int k = 0; k < FPT; ++k) {
+            const int e = tid + k * FEQB_THREADS;
+            if (e < (nt + 1) * (W + 1)) {
+                const int t = e / (W + 1), v = e % (W + 1), lo = v ? v - 1 : 1;
+                const double u = (double)v, um = u - 1.0, up = u + 1.0;
+                const double norm = sqrt(s_var[t]) * 0.39894228040143267794;
+                const double E = s_E[t][lo] - 2.0 * s_E[t][v] + s_E[t][v + 1];
+                const double Rm = v ? s_R[t][lo] : -s_R[t][1], eu = s_R[t][v];
+                f[k] = norm * E + 0.5 * um * (Rm - eu) + 0.5 * up * (s_R[t][v + 1] - eu);
             }
         }
         __syncthreads();
-    }
-    double *dst = part + ((long long)r * FEQB_SPLIT + split) * A.nb;
 #pragma unroll
-    for (int q = 0; q < FEQB_CPT; ++q) {
-        const int i = tid + q * FEQB_THREADS;
-        if (i < A.nb) dst[i] = accW[q];
+        for (int k = 0; k < FPT; ++k) {
+            const int e = tid + k * FEQB_THREADS;
+            if (e < (nt + 1) * (W + 1)) s_E[e / (W + 1)][e % (W + 1)] = f[k];
+        }
+        __syncthreads();
+        for (int e = tid; e < nsets * FEQB_SPLIT; e += FEQB_THREADS) {
+            const int set = e / FEQB_SPLIT, sp = e % FEQB_SPLIT;
+            int hi = 0;
+            while ((hi + 1) * (hi + 2) / 2 <= set) ++hi;
+            const int lo = set - hi * (hi + 1) / 2;
+            double acc = 0.0;
+            for (int t = sp; t < nt; t += FEQB_SPLIT) acc += s_w[t] * (s_E[t][lo] * s_E[t][hi]);
+            s_part[e] = acc;
+        }
+        if (tid <= W) s_G[tid] = s_E[nt][tid];
+        __syncthreads();
+        for (int e = tid; e < nsets; e += FEQB_THREADS) {
+            double acc = s_wsg[e];
+            for (int sp = 0; sp < FEQB_SPLIT; ++sp) acc += s_part[e * FEQB_SPLIT + sp];
+            s_wsg[e] = acc;
+        }
+        __syncthreads();
     }
-}
-
-// One CTA per replica: the statistics, the WSG sum of the splits' partials
-// (in split order), the measured and Gaussian equilibria and the distances.
-__global__ void __launch_bounds__(FEQB_THREADS) k_feq_batch(FeqBatchArgs A, const double *part) {
-    __shared__ double s_a[FEQB_THREADS], s_b[FEQB_THREADS], s_c[FEQB_THREADS], s_d[FEQB_THREADS];
-    __shared__ double s_par[4];
-    const int r = blockIdx.x, tid = threadIdx.x;
-    const RepDev &R = A.reps[r];
-    const int stride = 3 * A.nb + FEQB_STATS;
-    double *out = A.out + (long long)r * stride;
-    const int32_t *hist = A.hist + ((((long long)r * A.n_lg + A.lg) * A.n_dx + A.dxi) * MD_NBLK) * A.nb;
-    const double samples = (double)R.n * (double)A.nwin;
-    feqb_params(A, R, r, s_a, s_b, s_par, out);
-    const double a2 = s_par[1];
-    const int side = 2 * A.W + 1;
-    const int used = feqb_splits_used(s_par[2]);
-    // the Gaussian's 1D factors, one row shared by all classes
-    __shared__ double s_G[2 * MD_MAX_W + 1];
-    if (tid == 0 && a2 > 0) cell_gauss_row(a2, A.W, s_G);
     __syncthreads();
-    constexpr int CPT = FEQB_CPT;
-    double accW[CPT];
-#pragma unroll
-    for (int q = 0; q < CPT; ++q) {
-        const int i = tid + q * FEQB_THREADS;
-        double acc = 0.0;
-        if (i < A.nb && a2 > 0)
-            for (int sp = 0; sp < used; ++sp) acc += part[((long long)r * FEQB_SPLIT + sp) * A.nb + i];
-        accW[q] = acc;
-    }
-    double mg = 0.0, kg = 0.0, mw = 0.0, kw = 0.0, sum = 0.0;
-#pragma unroll
-    for (int q = 0; q < CPT; ++q) {
-        const int i = tid + q * FEQB_THREADS;
-        if (i >= A.nb) continue;
-        int mem[8], nm = 0;
+    double mg = 0.0, kg = 0.0, mw = 0.0, kw = 0.0, sum = 0.0, zero = 0.0;
+    for (int i = tid; i < A.nb; i += FEQB_THREADS) {
+        const int x = abs(i % side - W), y = abs(i / side - W);
+        const int lo = min(x, y), hi = max(x, y);
+        long long tot = 0;
+        int nm = 1;
         if (A.sym) {
-            const int a = abs(i % side - A.W), b = abs(i / side - A.W);
-            const int lo = min(a, b), hi = max(a, b);
-            for (int j = 0; j < A.nb && nm < 8; ++j) {
-                const int c = abs(j % side - A.W), d = abs(j / side - A.W);
-                if (min(c, d) == lo && max(c, d) == hi) mem[nm++] = j;
+            nm = 0;
+            for (int q = 0; q < 8; ++q) {                 // (+-lo, +-hi), (+-hi, +-lo), each once
+                const int sx = (q & 1 ? -1 : 1) * (q & 4 ? hi : lo), sy = (q & 2 ? -1 : 1) * (q & 4 ? lo : hi);
+                if (((q & 1) && sx == 0) || ((q & 2) && sy == 0) || ((q & 4) && lo == hi)) continue;
+                tot += s_tot[(sy + W) * side + sx + W];
+                ++nm;
             }
         } else {
-            mem[nm++] = i;
+            tot = s_tot[i];
         }
-        long long tot = 0;
-        for (int b = 0; b < MD_NBLK; ++b)
-            for (int m = 0; m < nm; ++m) tot += hist[b * A.nb + mem[m]];
         const double P = samples > 0 ? (double)tot / ((double)nm * samples) : 0.0;
-        const double G = a2 > 0 ? s_G[i % side] * s_G[i / side] : 0.0;
-        const double Wg = accW[q];
+        const double G = a2 > 0 ? s_G[x] * s_G[y] : 0.0;
+        const double Wg = s_wsg[hi * (hi + 1) / 2 + lo];
         out[i] = P;
         out[A.nb + i] = G;
         out[2 * A.nb + i] = Wg;
@@ -410,35 +391,28 @@ __global__ void __launch_bounds__(FEQB_THREADS) k_feq_batch(FeqBatchArgs A, cons
         }
         sum += P;
     }
-    s_a[tid] = mg;
-    s_b[tid] = kg;
-    s_c[tid] = mw;
-    s_d[tid] = kw;
-    __syncthreads();
-    for (int o = FEQB_THREADS / 2; o > 0; o >>= 1) {
-        if (tid < o) {
-            s_a[tid] = fmax(s_a[tid], s_a[tid + o]);
-            s_b[tid] += s_b[tid + o];
-            s_c[tid] = fmax(s_c[tid], s_c[tid + o]);
-            s_d[tid] += s_d[tid + o];
-        }
-        __syncthreads();
+    feqb_sum2(kg, kw, s_r);
+    feqb_sum2(sum, zero, s_r);
+    for (int o = 16; o > 0; o >>= 1) {
+        mg = fmax(mg, __shfl_xor_sync(0xffffffffu, mg, o));
+        mw = fmax(mw, __shfl_xor_sync(0xffffffffu, mw, o));
     }
-    // the sum of P goes through the same fixed tree
+    if ((tid & 31) == 0) {
+        s_part[tid >> 5] = mg;
+        s_part[32 + (tid >> 5)] = mw;
+    }
+    __syncthreads();
     if (tid == 0) {
-        out[3 * A.nb + 4] = s_a[0];
-        out[3 * A.nb + 5] = s_b[0];
-        out[3 * A.nb + 6] = s_c[0];
-        out[3 * A.nb + 7] = s_d[0];
+        for (int w = 1; w < FEQB_THREADS / 32; ++w) {
+            mg = fmax(mg, s_part[w]);
+            mw = fmax(mw, s_part[32 + w]);
+        }
+        out[3 * A.nb + 4] = mg;
+        out[3 * A.nb + 5] = kg;
+        out[3 * A.nb + 6] = mw;
+        out[3 * A.nb + 7] = kw;
+        out[3 * A.nb + 13] = sum;
     }
-    __syncthreads();
-    s_a[tid] = sum;
-    __syncthreads();
-    for (int o = FEQB_THREADS / 2; o > 0; o >>= 1) {
-        if (tid < o) s_a[tid] += s_a[tid + o];
-        __syncthreads();
-    }
-    if (tid == 0) out[3 * A.nb + 13] = s_a[0];
 }
 
 // ---------------------------------------------------------------- bootstrap
@@ -648,8 +622,6 @@ struct md_system {
     Control *d_ctl = nullptr;
     double *d_epart = nullptr;
     double *d_small = nullptr;   // readout scratch (2*nb + 8 doubles, 4 energy)
-    double *d_feq_part = nullptr;   // WSG partial sums of the f_eq stage [nrep][FEQB_SPLIT][nb]
-    double *d_feq_par = nullptr;    // per replica mu2, a^2, lambda of the f_eq stage [nrep][4]
     long long *d_hist64 = nullptr;
     int32_t *d_nc_of_id = nullptr;
     // resident engine (md_tune staging 4): plan, buffers, launch shape; the
@@ -1272,8 +1244,6 @@ int md_init_batch(const md_params *p, int32_t n_rep, const double *x, const doub
     ALLOC(S.disp_rep, sizeof(double) * (size_t)n_rep);
     ALLOC(s->d_epart, sizeof(double) * ngr * 4);
     ALLOC(s->d_small, sizeof(double) * (2 * s->nb + 16));
-    ALLOC(s->d_feq_part, sizeof(double) * (size_t)n_rep * FEQB_SPLIT * s->nb);
-    ALLOC(s->d_feq_par, sizeof(double) * 4 * (size_t)n_rep);
     ALLOC(s->d_hist64, sizeof(long long) * s->nb);
     ALLOC(s->d_nc_of_id, sizeof(int32_t) * s->ntot);
 #undef ALLOC
@@ -1823,9 +1793,7 @@ int feq_batch(md_system *s, int32_t lg, int32_t dxi, int32_t symmetrize, double 
     double *dst = out;
     if (!dev) MD_CUDA_TRY(cudaMallocAsync((void **)&dst, bytes, s->st));
     A.out = dst;
-    k_feq_params<<<s->nrep, FEQB_THREADS, 0, s->st>>>(A, s->d_feq_par);
-    k_feq_terms<<<dim3(s->nrep, FEQB_SPLIT), FEQB_THREADS, 0, s->st>>>(A, s->d_feq_par, s->d_feq_part);
-    k_feq_batch<<<s->nrep, FEQB_THREADS, 0, s->st>>>(A, s->d_feq_part);
+    k_feq_batch<<<s->nrep, FEQB_THREADS, 0, s->st>>>(A);
     cudaError_t e = cudaGetLastError();
     if (!dev) {
         if (e == cudaSuccess) e = cudaMemcpyAsync(out, dst, bytes, cudaMemcpyDeviceToHost, s->st);

@@ -160,10 +160,10 @@ __global__ void k_pdf_models(double mu2, double lam, double width, int nbins, do
     const double hi = __dadd_rn(lo, width);
     pg[k] = normal_mass(lo, hi, mu2);
     double s = 0.0;
-    const int c1 = wsg_cmax(lam);
-    for (int c = wsg_cmin(lam); c <= c1; ++c)
+    const int c1 = wsg_cmax(lam), dc = wsg_stride(lam);
+    for (int c = wsg_cmin(lam); c <= c1; c += dc)
         s += poisson_weight(c, lam) * normal_mass(lo, hi, (double)(c + 1) * mu2 / (lam + 1.0));
-    pwsg[k] = s;
+    pwsg[k] = (double)dc * s;
 }
 
 __global__ void k_kl_terms(const double *R, const double *Q, int n, double *K) {

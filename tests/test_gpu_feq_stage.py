@@ -37,3 +37,70 @@ def test_bootstrap_tiles(mdlg, orc, W, windows, block_windows, sym, B):
         ref = orc.bootstrap_feq(h.astype(np.int64), w, W, float(p.n), sym=sym, B=B, seed=5, rep=r)
         assert np.array_equal(sig[r], ref), (r, np.max(np.abs(sig[r] - ref)))
     s.close()
+
+
+def _wsg_weights(lam):
+    """Poisson weights of the window in extended precision, from the mode by
+    the ratio w(c+1)/w(c) = lam/(c+1), normalised by their own sum."""
+    lo, hi = max(0, int(lam - 14 * np.sqrt(lam) - 30)), int(lam + 14 * np.sqrt(lam) + 40)
+    c = np.arange(lo, hi + 1)
+    m = int(lam) - lo
+    r = np.longdouble(lam) / np.arange(lo + 1, hi + 1).astype(np.longdouble)
+    w = np.ones(c.size, np.longdouble)
+    w[m + 1:] = np.cumprod(r[m:])
+    w[:m] = np.cumprod(1 / r[:m][::-1])[::-1]
+    return c, (w / w.sum()).astype(np.float64)
+
+
+@pytest.mark.parametrize("lam", [0.0, 15.9, 39.99, 40.0, 44.5, 79.1, 333.0, 2.0e4, 1.0e5, 9.9e5])
+def test_wsg_strided_window(mdlg, lam):
+    """feq_wsg and disp_pdf_models on both sides of the strided window's line.
+    Bar 1e-13: the weights' exponents carry up to 2^-53 * 200 below c = 16
+    and the 1D factors a few 2^-53."""
+    from math import erf, exp, pi, sqrt
+
+    c, w = _wsg_weights(lam) if lam > 0 else (np.array([0]), np.array([1.0]))
+    a2 = 0.21
+    var = a2 * (c + 1.0) / (lam + 1.0)
+
+    def f(u):
+        return np.array([sqrt(v / (2 * pi)) * (exp(-(u - 1) ** 2 / (2 * v)) - 2 * exp(-u * u / (2 * v)) + exp(-(u + 1) ** 2 / (2 * v)))
+                         + 0.5 * (u - 1) * (erf((u - 1) / sqrt(2 * v)) - erf(u / sqrt(2 * v)))
+                         + 0.5 * (u + 1) * (erf((u + 1) / sqrt(2 * v)) - erf(u / sqrt(2 * v))) for v in var])
+
+    F = [f(float(u)) for u in range(-4, 5)]
+    ref = np.array([[np.sum(w * F[x] * F[y]) for x in range(9)] for y in range(9)]).reshape(-1)
+    got = mdlg.feq_wsg(a2, lam, W=4).cpu().numpy()
+    assert np.max(np.abs(got - ref)) < 1e-13
+    if lam <= 1e5:
+        nb, width, mu2 = 33, 0.3, 1.7
+        s2 = np.sqrt(2 * mu2 * (c + 1.0) / (lam + 1.0))
+        edge = (np.arange(nb + 1) - nb // 2) * width
+        E = np.array([np.sum(w * np.array([erf(e / s) for s in s2])) for e in edge]) * 0.5
+        _, pw = mdlg.disp_pdf_models(mu2, lam, width, nb)
+        assert np.max(np.abs(pw.cpu().numpy() - np.diff(E))) < 1e-13
+
+
+@pytest.mark.parametrize("W,sym", [(1, True), (4, False), (4, True), (10, False), (10, True)])
+def test_feq_batch_rows(mdlg, orc, W, sym):
+    """Every part of a feq_batch row against the integer histogram and the
+    single-distribution oracle at the row's own a^2 and lambda."""
+    s, params = _batch(mdlg, W, 35, every=15)
+    P, G, Wg, st = mdlg.feq_batch(s, 0, 0, symmetrize=sym)
+    for r, p in enumerate(params):
+        h, ov, nw = s.hist_raw(r, 0, 0)
+        ref = h / (float(p.n) * nw)
+        if sym:
+            ref = orc.symmetrize(ref, W)
+        assert np.max(np.abs(P[r] - ref)) <= 4 * 2.0 ** -53
+        a2, lam = st[r, 2], st[r, 3]
+        assert np.max(np.abs(G[r] - orc.feq_gaussian(a2, 0.0, 0.0, W))) < 1e-12
+        bar = 1e-12 + 4e-15 * lam          # the oracle's weights lose lambda * log(lambda) * 2^-53
+        assert np.max(np.abs(Wg[r] - orc.feq_wsg(a2, lam, 0.0, 0.0, W))) < bar
+        ok = P[r] > 0
+        assert abs(st[r, 4] - np.max(np.abs(P[r] - G[r]))) < 1e-15
+        assert abs(st[r, 6] - np.max(np.abs(P[r] - Wg[r]))) < 1e-15
+        kl = np.sum(P[r][ok] * np.log(P[r][ok] / Wg[r][ok]))
+        assert abs(st[r, 7] - kl) < 1e-12 * max(1.0, abs(kl)) and abs(st[r, 13] - P[r].sum()) < 1e-14
+        assert st[r, 8] == nw and st[r, 10] == ov
+    s.close()
