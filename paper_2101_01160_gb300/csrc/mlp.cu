@@ -2,9 +2,10 @@
 // the state point (phi, T, Delta t_LG, Delta x) to the probabilities of the
 // (2W+1)^2 = 81 displacement classes, trained on histograms measured by the
 // MD of this library.  Hidden layers are BF16 GEMMs on the tensor cores
-// (tcgen05.mma, FP32 accumulation in TMEM, fused bias/activation epilogues);
-// the 4-input first layer, softmax, loss, transposes, bias gradients and
-// Adam are CUDA-core kernels.
+// (tcgen05.mma, FP32 accumulation in TMEM).  A training step is three
+// launches: the forward and backward chain of each 128-row tile on one
+// thread-block cluster (k_train_chain), the weight gradients' partial sums
+// (k_train_grads), and their sum with the Adam update (k_train_update).
 //
 // Model: x_f = (x - shift)/scale; h_1 = silu(W_1 x_f + b_1) (CUDA cores);
 // h_l = silu(W_l h_{l-1} + b_l), l = 2..L-1 (tensor cores); logits =
@@ -26,23 +27,16 @@ using bf16 = __nv_bfloat16;
 
 constexpr int GBM = 128;   // GEMM tile rows (TMEM lanes)
 constexpr int GBK = 64;    // K per pipeline stage
-constexpr int GRAD_MAX_SPLIT = 64;   // K splits of a weight-gradient GEMM (K = the batch)
+constexpr int GRAD_MAX_SPLIT = 64;   // splits of a weight gradient over the batch
+constexpr int GRAD_ROWS = 128;       // rows of one partial bias or first-layer gradient
 constexpr uint64_t GEMM_WAIT_NS = 2000000000ull;
-
-enum Epi { EPI_F32 = 0, EPI_BIAS_F32 = 1, EPI_BIAS_SILU = 2, EPI_DSILU = 3 };
 
 struct GemmArgs {
     const bf16 *A;      // [M][K] row-major (K contiguous)
     const bf16 *B;      // [N][K] row-major
     int lda, ldb, M, N, K;
-    float *C;           // FP32 output (EPI_F32 / EPI_BIAS_F32; pre-activation for EPI_BIAS_SILU)
+    float *C;           // [M][ldc] FP32
     int ldc;
-    long long c_split;  // EPI_F32 split over K (grid.y = z): K range z of length K, tile at C + z c_split
-    bf16 *H;            // BF16 output (activation or gradient)
-    int ldh;
-    const float *bias;  // [N]
-    const float *Zp;    // EPI_DSILU: pre-activation, [M][ldz]
-    int ldz;
     int *status;
     uint64_t wait_ns;   // limit of every mbarrier wait (0: GEMM_WAIT_NS)
     int dbg_skip_commit;   // bf16_gemm_selftest: CTA 0 does not signal stage dbg_skip_commit - 1 (0: never)
@@ -66,7 +60,6 @@ __device__ __forceinline__ int tile_off(int r, int k8) { return (r >> 3) * 1024 
 // C = A * B^T on the tensor cores; one CTA computes a 128 x N tile (N <= 256,
 // a multiple of 16) with the accumulator in N TMEM columns.  K is consumed
 // in stages of 64: the loads of stage k+1 overlap the MMAs of stage k.
-template <int EPI>
 __global__ void __launch_bounds__(128) k_gemm(GemmArgs g) {
     extern __shared__ __align__(1024) unsigned char sm[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -92,8 +85,7 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs g) {
     const uint32_t tmem = *s_tmem;
     const int m0 = blockIdx.x * GBM;
     const int nk = g.K / GBK;
-    const int kb = (int)blockIdx.y * nk;   // first stage of this CTA's K range
-    const int n0 = (int)blockIdx.z * N;    // first output column of this CTA (N split)
+    const int n0 = (int)blockIdx.y * N;    // first output column of this CTA (N split)
     const uint32_t idesc = umma::idesc_bf16(GBM, N);
     for (int kt = 0; kt < nk; ++kt) {
         const int s = kt & 1;
@@ -104,11 +96,11 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs g) {
         if (!s_ok) break;
         for (int c = tid; c < GBM * 8; c += 128) {
             const int r = c >> 3, k8 = c & 7;
-            cpa16(sa + tile_off(r, k8), g.A + (size_t)(m0 + r) * g.lda + (kb + kt) * GBK + k8 * 8);
+            cpa16(sa + tile_off(r, k8), g.A + (size_t)(m0 + r) * g.lda + kt * GBK + k8 * 8);
         }
         for (int c = tid; c < N * 8; c += 128) {
             const int r = c >> 3, k8 = c & 7;
-            cpa16(sb + tile_off(r, k8), g.B + (size_t)(n0 + r) * g.ldb + (kb + kt) * GBK + k8 * 8);
+            cpa16(sb + tile_off(r, k8), g.B + (size_t)(n0 + r) * g.ldb + kt * GBK + k8 * 8);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
         asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -142,36 +134,9 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs g) {
         for (int cl = 0; cl < N; cl += 16) {
             float v[16];
             umma::ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)cl, v);
-            const int c0 = n0 + cl;   // output column
-            if (EPI == EPI_F32 || EPI == EPI_BIAS_F32) {
-                float4 *dst = reinterpret_cast<float4 *>(g.C + (size_t)blockIdx.y * g.c_split + (size_t)row * g.ldc + c0);
+            float4 *dst = reinterpret_cast<float4 *>(g.C + (size_t)row * g.ldc + n0 + cl);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    float4 o;
-                    o.x = v[4 * q + 0] + (EPI == EPI_BIAS_F32 ? g.bias[c0 + 4 * q + 0] : 0.0f);
-                    o.y = v[4 * q + 1] + (EPI == EPI_BIAS_F32 ? g.bias[c0 + 4 * q + 1] : 0.0f);
-                    o.z = v[4 * q + 2] + (EPI == EPI_BIAS_F32 ? g.bias[c0 + 4 * q + 2] : 0.0f);
-                    o.w = v[4 * q + 3] + (EPI == EPI_BIAS_F32 ? g.bias[c0 + 4 * q + 3] : 0.0f);
-                    dst[q] = o;
-                }
-            } else {
-                __align__(16) bf16 hb[16];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    float o;
-                    if (EPI == EPI_BIAS_SILU) {
-                        const float z = v[i] + g.bias[c0 + i];
-                        if (g.C) g.C[(size_t)row * g.ldc + c0 + i] = z;
-                        o = silu(z);
-                    } else {
-                        o = v[i] * silu_grad(g.Zp[(size_t)row * g.ldz + c0 + i]);
-                    }
-                    hb[i] = __float2bfloat16_rn(o);
-                }
-                uint4 *dst = reinterpret_cast<uint4 *>(g.H + (size_t)row * g.ldh + c0);
-                dst[0] = reinterpret_cast<const uint4 *>(hb)[0];
-                dst[1] = reinterpret_cast<const uint4 *>(hb)[1];
-            }
+            for (int q = 0; q < 4; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
         }
     } else if (tid == 0) {
         atomicOr(g.status, 1);
@@ -183,188 +148,24 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs g) {
 
 size_t gemm_smem(int N) { return 2 * (size_t)(GBM * GBK * 2 + N * GBK * 2) + 32; }
 
-// ksplit > 1 (EPI_F32 only): g.K is one split's K; split z writes its
-// partial tile to C + z c_split, to be summed in split order.  A GEMM with
-// fewer 128-row tiles than the device has SMs is also split over N into two
-// column blocks of N/2 (grid.z), each CTA with its own accumulator; the
-// arithmetic of every output is the same.
-template <int EPI>
-int gemm_launch(const GemmArgs &g, cudaStream_t st, int ksplit = 1) {
+// A GEMM with fewer 128-row tiles than the device has SMs is split over N
+// into two column blocks of N/2 (grid.y), each CTA with its own accumulator;
+// the arithmetic of every output is the same.
+int gemm_launch(const GemmArgs &g, cudaStream_t st) {
     if (g.M % GBM || g.K % GBK || g.N % 16 || g.N < 16 || g.N > 256 || g.lda % 8 || g.ldb % 8)
         return fail(MD_E_ARG, "gemm: M %% 128, K %% 64, N %% 16 in [16,256], lda/ldb %% 8 required");
-    if (ksplit < 1 || (ksplit > 1 && EPI != EPI_F32)) return fail(MD_E_ARG, "gemm: K split only for EPI_F32");
     int dev = 0, nsm = 0;
     MD_CUDA_TRY(cudaGetDevice(&dev));
     MD_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    const int nsplit = (g.N % 32 == 0 && (long long)(g.M / GBM) * ksplit < nsm) ? 2 : 1;
+    const int nsplit = (g.N % 32 == 0 && g.M / GBM < nsm) ? 2 : 1;
     GemmArgs gg = g;
     gg.N = g.N / nsplit;
     const size_t smem = gemm_smem(gg.N);
-    MD_CUDA_TRY(cudaFuncSetAttribute(k_gemm<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_gemm<EPI><<<dim3(g.M / GBM, ksplit, nsplit), 128, smem, st>>>(gg);
+    MD_CUDA_TRY(cudaFuncSetAttribute(k_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_gemm<<<dim3(g.M / GBM, nsplit), 128, smem, st>>>(gg);
     MD_CUDA_TRY(cudaGetLastError());
     return MD_OK;
 }
-
-// ---------------------------------------------------------------- CUDA-core kernels
-// First layer (4 inputs): features, pre-activation (optional) and BF16
-// activation; rows >= M (padding) get zero features.
-__global__ void k_layer1(const float *X, int M, int Mpad, const float *W, const float *b,
-                         const float4 shift, const float4 scale, int width, float *xf, float *Z,
-                         bf16 *H) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)Mpad * width) return;
-    const int m = (int)(i / width), o = (int)(i % width);
-    float f0 = 0.f, f1 = 0.f, f2 = 0.f, f3 = 0.f;
-    if (m < M) {
-        f0 = (X[4 * m + 0] - shift.x) / scale.x;
-        f1 = (X[4 * m + 1] - shift.y) / scale.y;
-        f2 = (X[4 * m + 2] - shift.z) / scale.z;
-        f3 = (X[4 * m + 3] - shift.w) / scale.w;
-    }
-    if (xf && o == 0) {
-        xf[4 * m + 0] = f0;
-        xf[4 * m + 1] = f1;
-        xf[4 * m + 2] = f2;
-        xf[4 * m + 3] = f3;
-    }
-    const float z = b[o] + W[4 * o + 0] * f0 + W[4 * o + 1] * f1 + W[4 * o + 2] * f2 + W[4 * o + 3] * f3;
-    if (Z) Z[i] = z;
-    H[i] = __float2bfloat16_rn(silu(z));
-}
-
-// Softmax over the first ncls logits of each row; with targets, also the
-// row's share of the mean KL loss and d loss / d logits = (p sum(t) - t) / Mb
-// as BF16 (zero in the padding columns).
-__global__ void k_softmax(const float *logits, int ldl, int M, int ncls, float *P, const float *T,
-                          float *rowloss, bf16 *dlog, int ldd, float inv_batch) {
-    const int m = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (m >= M) return;
-    const float *l = logits + (size_t)m * ldl;
-    float mx = -INFINITY;
-    for (int c = lane; c < ncls; c += 32) mx = fmaxf(mx, l[c]);
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    float s = 0.f;
-    for (int c = lane; c < ncls; c += 32) s += __expf(l[c] - mx);
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    const float inv = 1.0f / s;
-    float ts = 0.f, loss = 0.f;
-    if (T)
-        for (int c = lane; c < ncls; c += 32) ts += T[(size_t)m * ncls + c];
-    for (int o = 16; o > 0; o >>= 1) ts += __shfl_xor_sync(0xffffffffu, ts, o);
-    for (int c = lane; c < ldd || c < ncls; c += 32) {
-        if (c < ncls) {
-            const float p = __expf(l[c] - mx) * inv;
-            if (P) P[(size_t)m * ncls + c] = p;
-            if (T) {
-                const float t = T[(size_t)m * ncls + c];
-                if (t > 0.f) loss += t * (__logf(t) - __logf(p));
-                if (dlog) dlog[(size_t)m * ldd + c] = __float2bfloat16_rn((p * ts - t) * inv_batch);
-            }
-        } else if (dlog && c < ldd) {
-            dlog[(size_t)m * ldd + c] = __float2bfloat16_rn(0.f);
-        }
-    }
-    if (rowloss) {
-        for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
-        if (lane == 0) rowloss[m] = loss * inv_batch;
-    }
-}
-
-// BF16 transpose [R][C] -> [C][R] through a 32x33 shared tile.
-__global__ void k_transpose(const bf16 *in, int R, int C, bf16 *out) {
-    __shared__ bf16 t[32][33];
-    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    for (int y = threadIdx.y; y < 32; y += blockDim.y) {
-        const int r = r0 + y, c = c0 + threadIdx.x;
-        t[y][threadIdx.x] = (r < R && c < C) ? in[(size_t)r * C + c] : __float2bfloat16_rn(0.f);
-    }
-    __syncthreads();
-    for (int y = threadIdx.y; y < 32; y += blockDim.y) {
-        const int c = c0 + y, r = r0 + threadIdx.x;
-        if (c < C && r < R) out[(size_t)c * R + r] = t[threadIdx.x][y];
-    }
-}
-
-// Column sums of a BF16 [M][N] matrix in FP32 (fixed order), into out[n].
-// Reductions over the batch in two passes with a fixed order: partial sums
-// over chunks of GRAD_ROWS rows (grid.y = chunk), then the chunks summed in
-// chunk order (k_sum_parts), so that the batch is spread over many CTAs and
-// the result does not depend on the launch.
-constexpr int GRAD_ROWS = 128;
-
-// part[chunk][n] = sum of column n of a [M][ld] BF16 matrix over the chunk.
-__global__ void k_colsum_part(const bf16 *a, int M, int N, int ld, float *part) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    const int m0 = blockIdx.y * GRAD_ROWS, m1 = min(M, m0 + GRAD_ROWS);
-    float s = 0.f;
-    for (int m = m0; m < m1; ++m) s += __bfloat162float(a[(size_t)m * ld + n]);
-    part[(size_t)blockIdx.y * N + n] = s;
-}
-
-// dW_1 = dZ_1^T x_f (4 inputs): part[chunk][o * 4 + k] over the chunk's rows.
-__global__ void k_grad_layer1_part(const bf16 *dZ, int M, int width, const float *xf, float *part) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= width * 4) return;
-    const int o = i / 4, k = i % 4;
-    const int m0 = blockIdx.y * GRAD_ROWS, m1 = min(M, m0 + GRAD_ROWS);
-    float s = 0.f;
-    for (int m = m0; m < m1; ++m) s += __bfloat162float(dZ[(size_t)m * width + o]) * xf[4 * m + k];
-    part[(size_t)blockIdx.y * width * 4 + i] = s;
-}
-
-// out[r][c] = sum over z = 0 .. nz-1, in z order, of part[z stride + r ldp + c].
-__global__ void k_sum_parts(const float *part, int nz, long long stride, int rows, int cols, int ldp,
-                            float *out, int ldo) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)rows * cols) return;
-    const int r = (int)(i / cols), c = (int)(i % cols);
-    float s = 0.f;
-    for (int z = 0; z < nz; ++z) s += part[z * stride + (long long)r * ldp + c];
-    out[(long long)r * ldo + c] = s;
-}
-
-// Adam on FP32 master parameters; refreshes the BF16 copy (and its
-// transpose) used by the tensor cores.  rows x cols block of a parameter with
-// leading dimension ld; master/m/v/g share that layout.
-__global__ void k_adam(float *w, float *mom, float *var, const float *g, int rows, int cols, int ld,
-                       float lr, float b1, float b2, float c1, float c2, float eps, bf16 *wb,
-                       bf16 *wt, int ldt) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows * cols) return;
-    const int r = i / cols, c = i % cols;
-    const size_t k = (size_t)r * ld + c;
-    const float gr = g[k];
-    const float m = b1 * mom[k] + (1.f - b1) * gr;
-    const float v = b2 * var[k] + (1.f - b2) * gr * gr;
-    mom[k] = m;
-    var[k] = v;
-    const float nw = w[k] - lr * (m / c1) / (sqrtf(v / c2) + eps);
-    w[k] = nw;
-    if (wb) wb[k] = __float2bfloat16_rn(nw);
-    if (wt) wt[(size_t)c * ldt + r] = __float2bfloat16_rn(nw);
-}
-
-__global__ void k_to_bf16(const float *w, int n, bf16 *out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = __float2bfloat16_rn(w[i]);
-}
-
-__global__ void k_sum(const float *a, int n, float *out) {
-    __shared__ float s[256];
-    float acc = 0.f;
-    for (int i = threadIdx.x; i < n; i += 256) acc += a[i];
-    s[threadIdx.x] = acc;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *out = s[0];
-}
-
 
 // ---------------------------------------------------------------- fused inference
 // Whole forward pass in one persistent, warp-specialised kernel over 128-row
@@ -744,23 +545,606 @@ __global__ void k_pack0(const float *W, const float *b, float sc, bf16 *out) {
     out[(n >> 3) * (F_SBO_B0 / 2) + (k >> 3) * 64 + (n & 7) * 8 + (k & 7)] = __float2bfloat16_rn(sc * v);
 }
 
-// Packs the bias b [N] into the K = 16 operand (b_hi, b_lo, 0, ...).
-__global__ void k_packb(const float *b, int N, float sc, bf16 *out) {
+// Packs the bias b [rows] into the K = 16 operand (b_hi, b_lo, 0, ...) of N
+// rows, those from `rows` on zero.
+__global__ void k_packb(const float *b, int rows, int N, float sc, bf16 *out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N * 16) return;
     const int n = i / 16, k = i % 16;
-    const float v = k < 2 ? split_part(b[n], k) : 0.f;
+    const float v = k < 2 && n < rows ? split_part(b[n], k) : 0.f;
     out[(n >> 3) * (F_SBO_B0 / 2) + (k >> 3) * 64 + (n & 7) * 8 + (k & 7)] = __float2bfloat16_rn(sc * v);
 }
 
-// Packs W [N][256] (BF16 row-major) into 64-feature chunks laid out exactly
-// as the fused kernel's shared-memory weight buffer.
-__global__ void k_pack(const bf16 *W, int N, float sc, bf16 *out) {
+// Element of a weight operand of N rows packed in 64-feature chunks, each
+// laid out exactly as a shared-memory weight buffer (rows n0 .. n0 + 8 j of a
+// chunk are contiguous).
+__device__ __forceinline__ int pack_off(int n, int k, int N) {
+    const int kk = k % FK;
+    return k / FK * N * FK + (n >> 3) * (F_SBO_B / 2) + (kk >> 3) * 64 + (n & 7) * 8 + (kk & 7);
+}
+
+// Packs W [rows][256] (FP32, rows <= N, the others zero) as BF16, times sc.
+__global__ void k_pack(const float *W, int rows, int N, float sc, bf16 *out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N * 256) return;
-    const int n = i / 256, k = i % 256, kc = k / FK, kk = k % FK;
-    out[(size_t)kc * N * FK + (n >> 3) * (F_SBO_B / 2) + (kk >> 3) * 64 + (n & 7) * 8 + (kk & 7)] =
-        __float2bfloat16_rn(sc * __bfloat162float(W[i]));
+    const int n = i / 256, k = i % 256;
+    const float v = n < rows ? __bfloat162float(__float2bfloat16_rn(W[i])) : 0.f;
+    out[pack_off(n, k, N)] = __float2bfloat16_rn(sc * v);
+}
+
+// Packs W^T [256][N] (FP32 W [rows][256]) as BF16: the operand of a layer's
+// input gradient.
+__global__ void k_pack_t(const float *W, int rows, int N, bf16 *out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N * 256) return;
+    const int n = i / 256, k = i % 256;
+    out[pack_off(k, n, 256)] = __float2bfloat16_rn(n < rows ? W[i] : 0.f);
+}
+
+
+// ---------------------------------------------------------------- training
+// A training step on a batch of B rows was some 50 small launches (per layer
+// a GEMM, two transposes, column sums, sums of partials, two Adam kernels),
+// 466 us at B = 512 for 0.7 GFLOP: launches, and epilogues that read and
+// wrote one row per lane.  It is three launches now; of 5 layers at B = 512:
+// k_train_chain 58 us, k_train_grads 7.1 us, k_train_update 4.2 us.
+//
+// k_train_chain: one thread-block cluster of CS CTAs per 128-row tile runs the
+// whole forward pass, the softmax and loss, and the backward pass down to the
+// first layer.  CTA `rank` computes columns rank * 256/CS .. of every layer:
+// its slice of the weights arrives by bulk copies while the previous layer is
+// computed, the accumulator is a 128 x 256/CS tile in TMEM, and the finished
+// BF16 activations (or gradients) are written into the next A operand of all
+// CS CTAs through distributed shared memory, with one cluster barrier per
+// layer.  What it leaves in global memory is transposed, [column][batch], so
+// that a warp's 32 rows are contiguous and the weight gradients' operands are
+// K-major.  The tile is one row block of 128 (the M of the instruction); the
+// columns are what is split, because a batch of 512 has only four row blocks.
+// It is bound by the latency of its 2 (layers) dependent steps.
+// Every value is that of the layer-by-layer formulation: the K order of the
+// products, the FP32 epilogues and the BF16 roundings are the same.
+
+// Where the parameters of a layer lie in the packed vector W_1, b_1, ...
+struct ParamMap {
+    int nl, ncls;
+    __host__ __device__ int out(int l) const { return l == nl - 1 ? ncls : 256; }
+    __host__ __device__ int outp(int l) const { return l == nl - 1 ? 128 : 256; }
+    __host__ __device__ int in(int l) const { return l == 0 ? 4 : 256; }
+    __host__ __device__ int W(int l) const { return l == 0 ? 0 : 1280 + (l - 1) * (65536 + 256); }
+    __host__ __device__ int b(int l) const { return W(l) + out(l) * in(l); }
+    __host__ __device__ int count() const { return b(nl - 1) + ncls; }
+};
+
+struct TrainArgs {
+    const float *X, *T;
+    int B;
+    ParamMap pm;
+    float4 shift, scale;
+    const float *w;                // packed FP32 parameters
+    const bf16 *Wf[F_MAXL + 1];    // packed operands of layers >= 1 (pack_off): W and W^T
+    const bf16 *Wb[F_MAXL + 1];
+    float *xf;                     // [B][4] features
+    float *Z;                      // [hidden layer][256][B] pre-activations
+    bf16 *H;                       // [hidden layer][256][B] activations
+    bf16 *dZ;                      // [layer][256][B] loss gradients of the pre-activations (last layer: 128 rows)
+    float *rowloss;                // [B]
+    float inv_batch;
+    int *status;
+};
+
+constexpr int T_THREADS = 256;
+constexpr int T_LOGIT_LD = 113;    // odd, > MLP_MAX_CLASSES: rows of the staged logits fall in different banks
+constexpr int T_DLOG_LD = 136;
+
+template <int CS> struct TrainShape {
+    static constexpr int NS = 256 / CS;            // hidden columns of a CTA
+    static constexpr int NO = 128 / CS;            // output columns of a CTA
+    static constexpr int NBUF = CS == 2 ? 1 : 2;   // weight buffers (a whole layer's slice each)
+    static constexpr int RP = 128 / CS;            // rows of a CTA's softmax
+    static constexpr int WBYTES = NS * 256 * 2;
+    static constexpr size_t smem = 2 * (size_t)F_ACT_BYTES + NBUF * WBYTES + 64;
+};
+static_assert(TrainShape<2>::smem <= 232448, "training chain: shared memory above 227 KB");
+static_assert(64 * T_LOGIT_LD * 4 + 64 * T_DLOG_LD * 2 <= F_ACT_BYTES, "training chain: softmax stage");
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// Address of this CTA's shared-memory location `addr` in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, int rank) {
+    uint32_t d;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(addr), "r"(rank));
+    return d;
+}
+__device__ __forceinline__ void st_cluster(uint32_t addr, uint4 v) {
+    asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+                 : "memory");
+}
+__device__ __forceinline__ void st_cluster(uint32_t addr, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+// All CTAs of the cluster: generic writes to any of their shared memory are
+// visible, also to the tensor cores, after it.
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("fence.proxy.async;" ::: "memory");
+    umma::fence_before();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    umma::fence_after();
+    asm volatile("fence.proxy.async;" ::: "memory");
+}
+
+template <int CS>
+__global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_constant__ TrainArgs a) {
+    using S = TrainShape<CS>;
+    extern __shared__ __align__(1024) unsigned char sm[];
+    unsigned char *wbuf = sm + 2 * F_ACT_BYTES;
+    uint64_t *full = reinterpret_cast<uint64_t *>(wbuf + S::NBUF * S::WBYTES);   // [NBUF]
+    uint64_t *done = full + S::NBUF;                                            // accumulator complete
+    uint32_t *s_tmem = reinterpret_cast<uint32_t *>(done + 1);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = (int)cluster_rank(), m0 = (int)(blockIdx.x / CS) * 128;
+    const ParamMap pm = a.pm;
+    const int nl = pm.nl, B = a.B, nops = 2 * (nl - 1);
+    // a warp may read only the TMEM lanes 32 (warp mod 4) .. +31: warps 0-3
+    // take the first half of the CTA's columns, warps 4-7 the second
+    const int quad = warp & 3, half = warp >> 2, r = quad * 32 + lane;
+    constexpr uint32_t ncols = S::NS < 32 ? 32 : S::NS;
+    if (warp == 0) umma::tmem_alloc(s_tmem, ncols);
+    if (tid == 0) {
+        for (int i = 0; i < S::NBUF; ++i) umma::mbar_init(&full[i], 1);
+        umma::mbar_init(done, 1);
+        umma::mbar_fence_init();
+    }
+    umma::fence_before();
+    __syncthreads();
+    umma::fence_after();
+    const uint32_t tmem = *s_tmem, trow = tmem + ((uint32_t)(quad * 32) << 16);
+    const uint32_t act0 = umma::saddr(sm);
+    bool bad = false;
+    // operation g < nl - 1: layer g + 1 forward; then layers nl - 1 .. 1 backward
+    const auto op_layer = [&](int g) { return g < nl - 1 ? g + 1 : 2 * (nl - 1) - g; };
+    const auto load = [&](int g) {   // thread 0: this CTA's slice of the operation's weights
+        if (g >= nops) return;
+        const int l = op_layer(g);
+        const bool fwd = g < nl - 1;
+        const int N = fwd ? pm.outp(l) : 256, K = fwd ? 256 : pm.outp(l), ns = N / CS;
+        const bf16 *src = (fwd ? a.Wf[l] : a.Wb[l]) + rank * ns * FK;
+        unsigned char *dst = wbuf + (g % S::NBUF) * S::WBYTES;
+        uint64_t *bar = &full[g % S::NBUF];
+        umma::mbar_expect_tx(bar, (uint32_t)(ns * K * 2));
+        for (int kc = 0; kc < K / FK; ++kc)
+            umma::bulk_g2s(dst + kc * ns * FK * 2, src + (size_t)kc * N * FK, (uint32_t)(ns * FK * 2), bar);
+    };
+    const auto product = [&](int g, int cur) {   // thread 0: issue the operation's MMAs
+        const int l = op_layer(g);
+        const bool fwd = g < nl - 1;
+        const int ns = (fwd ? pm.outp(l) : 256) / CS, K = fwd ? 256 : pm.outp(l);
+        if (!umma::mbar_wait(&full[g % S::NBUF], (g / S::NBUF) & 1, GEMM_WAIT_NS)) {
+            bad = true;
+            return;
+        }
+        umma::fence_after();
+        const uint32_t idesc = umma::idesc_bf16(128, ns);
+        const uint64_t ad = umma::desc(act0 + cur * F_ACT_BYTES, 128, F_SBO_A);
+        const uint64_t bd = umma::desc(umma::saddr(wbuf + (g % S::NBUF) * S::WBYTES), 128, F_SBO_B);
+        for (int kc = 0; kc < K / FK; ++kc)
+#pragma unroll
+            for (int k4 = 0; k4 < FK / 16; ++k4)
+                umma::mma(tmem, ad + (uint64_t)((kc * (FK / 16) + k4) * 16),
+                          bd + (uint64_t)((kc * ns * FK * 2) >> 4) + (uint64_t)(k4 * 16), idesc, (kc | k4) ? 1u : 0u);
+        umma::commit(done);
+    };
+    // every thread: the operation's accumulator is complete; its weight buffer is free again
+    const auto finish = [&](int g) {
+        if (!bad && !umma::mbar_wait(done, g & 1, GEMM_WAIT_NS)) bad = true;
+        umma::fence_after();
+        if (tid == 0 && !bad) load(g + S::NBUF);
+    };
+    // 16 BF16 values of row r, columns c .. c + 15 of the layer, into the A operand `buf` of every CTA
+    const auto spread = [&](int buf, int c, const uint32_t (&h)[8]) {
+        const uint32_t o0 = act0 + buf * F_ACT_BYTES + act_off(r, c), o1 = act0 + buf * F_ACT_BYTES + act_off(r, c + 8);
+#pragma unroll
+        for (int q = 0; q < CS; ++q) {
+            st_cluster(cluster_addr(o0, q), make_uint4(h[0], h[1], h[2], h[3]));
+            st_cluster(cluster_addr(o1, q), make_uint4(h[4], h[5], h[6], h[7]));
+        }
+    };
+    const auto put_t = [&](bf16 *dst, int c, const uint32_t (&h)[8]) {   // the same, transposed in global memory
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            reinterpret_cast<uint16_t *>(dst)[(size_t)(c + i) * B + m0 + r] =
+                (uint16_t)(i & 1 ? h[i / 2] >> 16 : h[i / 2] & 0xffffu);
+    };
+    constexpr int CH = S::NS / 2 < 16 ? 16 : S::NS / 2;   // columns of a half
+    constexpr int CO = S::NO / 2 < 16 ? 16 : S::NO / 2;
+    if (tid == 0)
+        for (int g = 0; g < S::NBUF; ++g) load(g);
+    cluster_sync();   // every CTA of the cluster runs: its shared memory may be written
+    // ---- first layer (4 inputs) on the CUDA cores
+    {
+        const float4 x = make_float4(a.X[4 * (size_t)(m0 + r)], a.X[4 * (size_t)(m0 + r) + 1],
+                                     a.X[4 * (size_t)(m0 + r) + 2], a.X[4 * (size_t)(m0 + r) + 3]);
+        const float f0 = (x.x - a.shift.x) / a.scale.x, f1 = (x.y - a.shift.y) / a.scale.y;
+        const float f2 = (x.z - a.shift.z) / a.scale.z, f3 = (x.w - a.shift.w) / a.scale.w;
+        if (rank == 0 && half == 0) reinterpret_cast<float4 *>(a.xf)[m0 + r] = make_float4(f0, f1, f2, f3);
+        const float *W = a.w, *b = a.w + pm.b(0);
+        for (int c0 = half * CH; c0 < min(S::NS, half * CH + CH); c0 += 16) {
+            const int c = rank * S::NS + c0;
+            uint32_t h[8];
+            float hv[2];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const int o = c + i;
+                const float z = b[o] + W[4 * o + 0] * f0 + W[4 * o + 1] * f1 + W[4 * o + 2] * f2 + W[4 * o + 3] * f3;
+                a.Z[(size_t)o * B + m0 + r] = z;
+                hv[i & 1] = silu(z);
+                if (i & 1) h[i / 2] = pack_bf16(hv[0], hv[1]);
+            }
+            put_t(a.H, c, h);
+            spread(0, c, h);
+        }
+    }
+    cluster_sync();
+    int cur = 0;
+    // ---- hidden layers
+    for (int g = 0; g < nl - 2; ++g) {
+        if (tid == 0 && !bad) product(g, cur);
+        const float *b = a.w + pm.b(g + 1);
+        float *Z = a.Z + (size_t)(g + 1) * 256 * B;
+        bf16 *H = a.H + (size_t)(g + 1) * 256 * B;
+        finish(g);
+        for (int c0 = half * CH; c0 < min(S::NS, half * CH + CH); c0 += 16) {
+            const int c = rank * S::NS + c0;
+            float v[16];
+            umma::ld16(trow + (uint32_t)c0, v);
+            uint32_t h[8];
+            float hv[2];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const float z = v[i] + b[c + i];
+                Z[(size_t)(c + i) * B + m0 + r] = z;
+                hv[i & 1] = silu(z);
+                if (i & 1) h[i / 2] = pack_bf16(hv[0], hv[1]);
+            }
+            put_t(H, c, h);
+            spread(cur ^ 1, c, h);
+        }
+        cluster_sync();
+        cur ^= 1;
+    }
+    // ---- output layer: logits of row r to the CTA that owns the row, staged
+    // in its unused A operand
+    float *logits = reinterpret_cast<float *>(sm + (cur ^ 1) * F_ACT_BYTES);          // [RP][T_LOGIT_LD]
+    bf16 *dl = reinterpret_cast<bf16 *>(logits + S::RP * T_LOGIT_LD);                 // [RP][T_DLOG_LD]
+    {
+        const int g = nl - 2;
+        if (tid == 0 && !bad) product(g, cur);
+        const float *b = a.w + pm.b(nl - 1);
+        finish(g);
+        const uint32_t row = cluster_addr(umma::saddr(logits + (r % S::RP) * T_LOGIT_LD), r / S::RP);
+        for (int c0 = half * CO; c0 < min(S::NO, half * CO + CO); c0 += 16) {
+            const int c = rank * S::NO + c0;
+            float v[16];
+            umma::ld16(trow + (uint32_t)c0, v);
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                if (c + i < pm.ncls) st_cluster(row + 4u * (c + i), v[i] + b[c + i]);
+        }
+        cluster_sync();
+    }
+    // ---- softmax, the row's share of the mean KL loss, and d loss / d logits
+    // = (p sum(t) - t) / B as BF16 (zero in the padding columns); one warp per row
+    for (int q = warp; q < S::RP; q += T_THREADS / 32) {
+        const int ncls = pm.ncls, m = m0 + rank * S::RP + q;
+        const float *l = logits + q * T_LOGIT_LD;
+        const float *T = a.T + (size_t)m * ncls;
+        float t[4];
+        float mx = -INFINITY;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) t[k] = lane + 32 * k < ncls ? T[lane + 32 * k] : 0.f;
+        for (int c = lane; c < ncls; c += 32) mx = fmaxf(mx, l[c]);
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        float s = 0.f;
+        for (int c = lane; c < ncls; c += 32) s += __expf(l[c] - mx);
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        const float inv = 1.0f / s;
+        float ts = 0.f, loss = 0.f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (lane + 32 * k < ncls) ts += t[k];
+        for (int o = 16; o > 0; o >>= 1) ts += __shfl_xor_sync(0xffffffffu, ts, o);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int c = lane + 32 * k;
+            float d = 0.f;
+            if (c < ncls) {
+                const float p = __expf(l[c] - mx) * inv;
+                if (t[k] > 0.f) loss += t[k] * (__logf(t[k]) - __logf(p));
+                d = (p * ts - t[k]) * a.inv_batch;
+            }
+            dl[q * T_DLOG_LD + c] = __float2bfloat16_rn(d);
+        }
+        for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+        if (lane == 0) a.rowloss[m] = loss * a.inv_batch;
+    }
+    __syncthreads();
+    for (int e = tid; e < S::RP * 16; e += T_THREADS) {
+        const int q = e / 16, k = e % 16 * 8;
+        const uint4 v = *reinterpret_cast<const uint4 *>(&dl[q * T_DLOG_LD + k]);
+        const uint32_t o = act0 + cur * F_ACT_BYTES + act_off(rank * S::RP + q, k);
+#pragma unroll
+        for (int t = 0; t < CS; ++t) st_cluster(cluster_addr(o, t), v);
+    }
+    bf16 *dZ = a.dZ + (size_t)(nl - 1) * 256 * B;
+    for (int e = tid; e < S::RP * 128; e += T_THREADS)
+        dZ[(size_t)(e / S::RP) * B + m0 + rank * S::RP + e % S::RP] = dl[e % S::RP * T_DLOG_LD + e / S::RP];
+    cluster_sync();
+    // ---- backward: dZ_{l-1} = (dZ_l W_l) silu'(Z_{l-1})
+    for (int l = nl - 1; l >= 1; --l) {
+        const int g = 2 * (nl - 1) - l;
+        if (tid == 0 && !bad) product(g, cur);
+        const float *Z = a.Z + (size_t)(l - 1) * 256 * B;
+        dZ = a.dZ + (size_t)(l - 1) * 256 * B;
+        float z[CH];   // requested while the product runs
+#pragma unroll
+        for (int i = 0; i < CH; ++i)
+            z[i] = half * CH < S::NS ? Z[(size_t)(rank * S::NS + half * CH + i) * B + m0 + r] : 0.f;
+        finish(g);
+#pragma unroll
+        for (int c1 = 0; c1 < CH; c1 += 16) {
+            const int c0 = half * CH + c1, c = rank * S::NS + c0;
+            if (c0 >= S::NS) break;
+            float v[16];
+            umma::ld16(trow + (uint32_t)c0, v);
+            uint32_t h[8];
+#pragma unroll
+            for (int i = 0; i < 16; i += 2)
+                h[i / 2] = pack_bf16(v[i] * silu_grad(z[c1 + i]), v[i + 1] * silu_grad(z[c1 + i + 1]));
+            put_t(dZ, c, h);
+            if (l > 1) spread(cur ^ 1, c, h);
+        }
+        cluster_sync();   // after the last layer: no CTA leaves while another may write its shared memory
+        cur ^= 1;
+    }
+    if (bad) {
+        // a wait gave up: products may still run; wait (with a limit) before
+        // their TMEM is freed, and flag it
+        if (tid == 0) {
+            umma::commit(done);
+            umma::mbar_wait(done, nops & 1, GEMM_WAIT_NS);
+        }
+        atomicOr(a.status, 1);
+    }
+    umma::fence_before();
+    __syncthreads();
+    if (warp == 0) umma::tmem_free(tmem, ncols);
+}
+
+// ---- gradients' partial sums over the batch
+// CTAs [0, tiles * ks): 128 x 128 tiles of dW_l = dZ_l^T H_{l-1}, l >= 1, split
+// z of ks over the batch (both operands K-major: [column][batch]).  The rest:
+// sums of dZ over chunks of GRAD_ROWS rows (bias gradients) and, for the first
+// layer, of dZ x_f, one thread per column and chunk.  All are summed in split
+// and chunk order by k_train_update, so nothing depends on the launch.
+struct GradArgs {
+    const bf16 *H, *dZ;
+    const float *xf;
+    int B, ks;
+    ParamMap pm;
+    float *part;      // [ks][tiles][128][128]
+    float *bpart;     // [chunk][layer * 256 + column]
+    float *wpart;     // [chunk][256 * 4] first layer
+    int *status;
+};
+constexpr int G_STAGES = 3;
+constexpr int G_STAGE_BYTES = 2 * 128 * GBK * 2;
+constexpr size_t GRADS_SMEM = G_STAGES * G_STAGE_BYTES + 64;
+
+__host__ __device__ inline int grad_tiles(const ParamMap &pm) { return 4 * (pm.nl - 2) + 2; }
+// Tile of weight (r, c) of layer l >= 1.
+__host__ __device__ inline int grad_tile(int l, int r, int c) { return 4 * (l - 1) + (r >> 7) * 2 + (c >> 7); }
+__host__ __device__ inline int grad_sums(const ParamMap &pm) { return pm.nl * 256 - 128; }
+
+__global__ void __launch_bounds__(128) k_train_grads(const __grid_constant__ GradArgs a) {
+    extern __shared__ __align__(1024) unsigned char sm[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, B = a.B;
+    const int tiles = grad_tiles(a.pm);
+    if ((int)blockIdx.x >= tiles * a.ks) {
+        const int per = grad_sums(a.pm) / 128, e = (int)blockIdx.x - tiles * a.ks;
+        const int ch = e / per, i = e % per * 128 + tid, l = i >> 8, c = i & 255;   // block-uniform chunk and layer
+        const bf16 *d = a.dZ + ((size_t)l * 256 + c) * B + ch * GRAD_ROWS;
+        uint4 q[GRAD_ROWS / 8];
+#pragma unroll
+        for (int k = 0; k < GRAD_ROWS / 8; ++k) q[k] = reinterpret_cast<const uint4 *>(d)[k];
+        float s = 0.f;
+        if (l == 0) {
+            float4 *xs = reinterpret_cast<float4 *>(sm);
+            xs[tid] = reinterpret_cast<const float4 *>(a.xf)[ch * GRAD_ROWS + tid];
+            __syncthreads();
+            float w0 = 0.f, w1 = 0.f, w2 = 0.f, w3 = 0.f;
+#pragma unroll
+            for (int k = 0; k < GRAD_ROWS / 8; ++k) {
+                const uint32_t u[4] = {q[k].x, q[k].y, q[k].z, q[k].w};
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float v = __uint_as_float(j & 1 ? u[j / 2] & 0xffff0000u : u[j / 2] << 16);
+                    const float4 x = xs[8 * k + j];
+                    s += v;
+                    w0 += v * x.x;
+                    w1 += v * x.y;
+                    w2 += v * x.z;
+                    w3 += v * x.w;
+                }
+            }
+            reinterpret_cast<float4 *>(a.wpart)[ch * 256 + c] = make_float4(w0, w1, w2, w3);
+        } else {
+#pragma unroll
+            for (int k = 0; k < GRAD_ROWS / 8; ++k) {
+                const uint32_t u[4] = {q[k].x, q[k].y, q[k].z, q[k].w};
+#pragma unroll
+                for (int j = 0; j < 8; ++j) s += __uint_as_float(j & 1 ? u[j / 2] & 0xffff0000u : u[j / 2] << 16);
+            }
+        }
+        a.bpart[(size_t)ch * a.pm.nl * 256 + i] = s;
+        return;
+    }
+    const int tile = (int)blockIdx.x % tiles, z = (int)blockIdx.x / tiles;
+    const int l = tile / 4 + 1, mt = tile % 4 / 2, nt = tile % 2;
+    uint64_t *mbar = reinterpret_cast<uint64_t *>(sm + G_STAGES * G_STAGE_BYTES);   // [G_STAGES], then the drain
+    uint32_t *s_tmem = reinterpret_cast<uint32_t *>(mbar + G_STAGES + 1);
+    __shared__ int s_ok;
+    if (warp == 0) umma::tmem_alloc(s_tmem, 128);
+    if (tid == 0) {
+        for (int i = 0; i <= G_STAGES; ++i) umma::mbar_init(&mbar[i], 1);
+        umma::mbar_fence_init();
+        s_ok = 1;
+    }
+    umma::fence_before();
+    __syncthreads();
+    umma::fence_after();
+    const uint32_t tmem = *s_tmem;
+    const int K = B / a.ks, nk = K / GBK;
+    const bf16 *A = a.dZ + ((size_t)l * 256 + mt * 128) * B + (size_t)z * K;
+    const bf16 *Bm = a.H + ((size_t)(l - 1) * 256 + nt * 128) * B + (size_t)z * K;
+    const uint32_t idesc = umma::idesc_bf16(128, 128);
+    const auto fetch = [&](int kt) {
+        unsigned char *sa = sm + kt % G_STAGES * G_STAGE_BYTES, *sb = sa + G_STAGE_BYTES / 2;
+        for (int c = tid; c < 128 * 8; c += 128) {
+            const int r = c >> 3, k8 = c & 7;
+            cpa16(sa + tile_off(r, k8), A + (size_t)r * B + kt * GBK + k8 * 8);
+            cpa16(sb + tile_off(r, k8), Bm + (size_t)r * B + kt * GBK + k8 * 8);
+        }
+    };
+    for (int kt = 0; kt < G_STAGES - 1; ++kt) {
+        if (kt < nk) fetch(kt);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    for (int kt = 0; kt < nk; ++kt) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(G_STAGES - 2) : "memory");
+        umma::fence_proxy_smem();
+        __syncthreads();
+        const int s = kt % G_STAGES;
+        if (tid == 0) {
+            umma::fence_after();
+            const uint32_t a0 = umma::saddr(sm + s * G_STAGE_BYTES), b0 = a0 + G_STAGE_BYTES / 2;
+#pragma unroll
+            for (int k4 = 0; k4 < GBK / 16; ++k4)
+                umma::mma(tmem, umma::desc(a0 + k4 * 256, 128, 1024), umma::desc(b0 + k4 * 256, 128, 1024), idesc,
+                          (kt | k4) ? 1u : 0u);
+            umma::commit(&mbar[s]);
+        }
+        // the stage fetched next was last read by the products of stage kt - 1
+        const int nx = kt + G_STAGES - 1;
+        if (nx < nk) {
+            if (nx >= G_STAGES && !umma::mbar_wait(&mbar[nx % G_STAGES], (nx / G_STAGES - 1) & 1, GEMM_WAIT_NS)) s_ok = 0;
+            __syncthreads();
+            if (!s_ok) break;
+            fetch(nx);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if (s_ok && !umma::mbar_wait(&mbar[(nk - 1) % G_STAGES], ((nk - 1) / G_STAGES) & 1, GEMM_WAIT_NS)) s_ok = 0;
+    if (!s_ok && tid == 0) {
+        umma::commit(&mbar[G_STAGES]);
+        umma::mbar_wait(&mbar[G_STAGES], 0, GEMM_WAIT_NS);
+    }
+    __syncthreads();
+    umma::fence_after();
+    if (s_ok) {
+        float *C = a.part + ((size_t)z * tiles + tile) * 16384 + (size_t)(warp * 32 + lane) * 128;
+        for (int c0 = 0; c0 < 128; c0 += 16) {
+            float v[16];
+            umma::ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                reinterpret_cast<float4 *>(C + c0)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        }
+    } else if (tid == 0) {
+        atomicOr(a.status, 1);
+    }
+    umma::fence_before();
+    __syncthreads();
+    if (warp == 0) umma::tmem_free(tmem, 128);
+}
+
+// ---- sums of the partials, Adam
+struct AdamArgs {
+    float lr, b1, b2, c1, c2, eps;
+    float *g;          // not NULL: write the gradient here and update nothing
+};
+struct UpdateArgs {
+    ParamMap pm;
+    const float *part, *bpart, *wpart;
+    int ks, nch;
+    float *w, *mom, *var;
+    bf16 *Wf[F_MAXL + 1], *Wb[F_MAXL + 1];
+    const float *rowloss;
+    int B;
+    float *loss;       // may be NULL
+};
+
+// One thread per parameter; the last block adds the rows' losses.
+__global__ void __launch_bounds__(256) k_train_update(const __grid_constant__ UpdateArgs a, const AdamArgs ad) {
+    if (blockIdx.x == gridDim.x - 1) {
+        if (!a.loss) return;
+        __shared__ float s[256];
+        float acc = 0.f;
+        for (int i = threadIdx.x; i < a.B; i += 256) acc += a.rowloss[i];
+        s[threadIdx.x] = acc;
+        __syncthreads();
+        for (int o = 128; o > 0; o >>= 1) {
+            if ((int)threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) *a.loss = s[0];
+        return;
+    }
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    const ParamMap pm = a.pm;
+    if (i >= pm.count()) return;
+    // parameter i: layer l, weight (r, c) or bias r (c < 0)
+    int l = i < 1280 ? 0 : 1 + (i - 1280) / 65792;
+    if (l > pm.nl - 1) l = pm.nl - 1;
+    const int j = i - pm.W(l), nw = pm.out(l) * pm.in(l);
+    const int r = j < nw ? j / pm.in(l) : j - nw, c = j < nw ? j % pm.in(l) : -1;
+    const float *src;
+    size_t stride;
+    int nz;
+    if (c < 0) {
+        src = a.bpart + l * 256 + r;
+        stride = (size_t)pm.nl * 256;
+        nz = a.nch;
+    } else if (l == 0) {
+        src = a.wpart + j;
+        stride = 1024;
+        nz = a.nch;
+    } else {
+        src = a.part + (size_t)grad_tile(l, r, c) * 16384 + (r & 127) * 128 + (c & 127);
+        stride = (size_t)grad_tiles(pm) * 16384;
+        nz = a.ks;
+    }
+    float gr = 0.f;
+#pragma unroll 4
+    for (int z = 0; z < nz; ++z) gr += src[z * stride];
+    if (ad.g) {
+        ad.g[i] = gr;
+        return;
+    }
+    const float m = ad.b1 * a.mom[i] + (1.f - ad.b1) * gr;
+    const float v = ad.b2 * a.var[i] + (1.f - ad.b2) * gr * gr;
+    a.mom[i] = m;
+    a.var[i] = v;
+    const float nw_ = a.w[i] - ad.lr * (m / ad.c1) / (sqrtf(v / ad.c2) + ad.eps);
+    a.w[i] = nw_;
+    if (l > 0 && c >= 0) {
+        const bf16 h = __float2bfloat16_rn(nw_);
+        a.Wf[l][pack_off(r, c, pm.outp(l))] = h;
+        a.Wb[l][pack_off(c, r, 256)] = h;
+    }
 }
 
 }  // namespace mdlg
@@ -772,23 +1156,21 @@ struct mlp_model {
     int nl = 0;                   // linear layers (hidden + 1)
     int width = 256, ncls = 81, npad = 128, nin = 4;
     float shift[4], scale[4];
-    std::vector<int> out, in, outp;   // per layer l = 0..nl-1 (out padded in outp)
-    // FP32 master, Adam moments, gradients: per layer W [outp][in], b [outp]
-    std::vector<float *> W, b, mW, vW, mb, vb, gW, gb;
-    std::vector<bf16 *> Wh, Wt;   // BF16 [outp][in] and [in][outp] (layers >= 1)
+    // FP32 master parameters, Adam moments and gradient, packed as `params`
+    float *w = nullptr, *mom = nullptr, *var = nullptr, *g = nullptr;
+    std::vector<bf16 *> Wf, Wb;   // packed BF16 W and W^T of layers >= 1 (training)
     std::vector<bf16 *> Wp;       // chunk-packed copies for the fused forward pass
     std::vector<bf16 *> Bp;       // packed bias operands (layers >= 1)
     bool packed = false;
     int adam_t = 0;
     // workspace
     long long cap = 0;            // rows
-    float *xf = nullptr, *logits = nullptr, *rowloss = nullptr;
-    std::vector<float *> Z;       // [cap][width] per hidden layer
-    std::vector<bf16 *> H;        // [cap][width] per hidden layer
-    bf16 *dA = nullptr, *dB = nullptr, *dlog = nullptr, *tA = nullptr, *tB = nullptr;
-    float *part = nullptr;        // partial sums of the batch reductions of the gradients
+    float *xf = nullptr, *rowloss = nullptr, *Z = nullptr;
+    bf16 *H = nullptr, *dZ = nullptr;
+    float *part = nullptr, *bpart = nullptr, *wpart = nullptr;   // partial sums of the gradients
     int *status = nullptr;
     std::vector<void *> allocs, ws;
+    ParamMap map() const { return ParamMap{nl, ncls}; }
 };
 
 namespace {
@@ -800,33 +1182,37 @@ int malloc_into(std::vector<void *> &v, void **p, size_t bytes) {
     return MD_OK;
 }
 
+// Splits of the weight gradients over a batch: as many as leave every split
+// two stages of GBK rows at least.
+int grad_splits(int B) {
+    const int nkt = B / GBK;
+    int ks = 1;
+    while (ks * 2 <= GRAD_MAX_SPLIT && nkt % (ks * 2) == 0 && nkt / (ks * 2) >= 2) ks *= 2;
+    return ks;
+}
+
 // Grows the row workspace to hold `rows` rows (multiple of 128).
 int ensure_ws(mlp_model *m, long long rows) {
     if (rows <= m->cap) return MD_OK;
     cudaDeviceSynchronize();
     for (void *p : m->ws) cudaFree(p);
     m->ws.clear();
-    const size_t R = (size_t)rows, Wd = (size_t)m->width;
+    m->cap = 0;
+    const size_t R = (size_t)rows, nch = R / GRAD_ROWS;
     int rc = MD_OK;
     auto A = [&](void **p, size_t bytes) {
         if (rc == MD_OK) rc = malloc_into(m->ws, p, bytes);
     };
     A((void **)&m->xf, R * 4 * sizeof(float));
-    A((void **)&m->logits, R * m->npad * sizeof(float));
     A((void **)&m->rowloss, R * sizeof(float));
-    m->Z.assign(m->nl - 1, nullptr);
-    m->H.assign(m->nl - 1, nullptr);
-    for (int l = 0; l < m->nl - 1; ++l) {
-        A((void **)&m->Z[l], R * Wd * sizeof(float));
-        A((void **)&m->H[l], R * Wd * sizeof(bf16));
-    }
-    A((void **)&m->dA, R * Wd * sizeof(bf16));
-    A((void **)&m->dB, R * Wd * sizeof(bf16));
-    A((void **)&m->dlog, R * m->npad * sizeof(bf16));
-    A((void **)&m->tA, R * Wd * sizeof(bf16));
-    A((void **)&m->tB, R * Wd * sizeof(bf16));
-    A((void **)&m->part, std::max((size_t)GRAD_MAX_SPLIT * Wd * Wd,
-                                  ((size_t)rows / GRAD_ROWS + 1) * Wd * 4) * sizeof(float));
+    A((void **)&m->Z, R * 256 * (m->nl - 1) * sizeof(float));
+    A((void **)&m->H, R * 256 * (m->nl - 1) * sizeof(bf16));
+    A((void **)&m->dZ, R * 256 * m->nl * sizeof(bf16));
+    // a batch of fewer rows may have more splits: room for the most
+    A((void **)&m->part, (size_t)std::min<long long>(GRAD_MAX_SPLIT, std::max<long long>(1, rows / GBK / 2)) *
+                             grad_tiles(m->map()) * 16384 * sizeof(float));
+    A((void **)&m->bpart, nch * m->nl * 256 * sizeof(float));
+    A((void **)&m->wpart, nch * 1024 * sizeof(float));
     if (rc) return rc;
     m->cap = rows;
     return MD_OK;
@@ -834,143 +1220,99 @@ int ensure_ws(mlp_model *m, long long rows) {
 
 int refresh_bf16(mlp_model *m, cudaStream_t st) {
     m->packed = false;
+    const ParamMap pm = m->map();
     for (int l = 1; l < m->nl; ++l) {
-        const int n = m->outp[l] * m->in[l];
-        k_to_bf16<<<(n + 255) / 256, 256, 0, st>>>(m->W[l], n, m->Wh[l]);
-        dim3 tb(32, 8), gr((m->in[l] + 31) / 32, (m->outp[l] + 31) / 32);
-        k_transpose<<<gr, tb, 0, st>>>(m->Wh[l], m->outp[l], m->in[l], m->Wt[l]);
+        const int n = pm.outp(l) * 256;
+        k_pack<<<(n + 255) / 256, 256, 0, st>>>(m->w + pm.W(l), pm.out(l), pm.outp(l), 1.0f, m->Wf[l]);
+        k_pack_t<<<(n + 255) / 256, 256, 0, st>>>(m->w + pm.W(l), pm.out(l), pm.outp(l), m->Wb[l]);
     }
     MD_CUDA_TRY(cudaGetLastError());
     return MD_OK;
 }
 
-// Forward pass on rows [0, Mpad): H_l (and Z_l when keep_z), logits.
-int forward(mlp_model *m, const float *X, long long M, long long Mpad, bool keep_z, cudaStream_t st) {
-    const float4 sh = make_float4(m->shift[0], m->shift[1], m->shift[2], m->shift[3]);
-    const float4 sc = make_float4(m->scale[0], m->scale[1], m->scale[2], m->scale[3]);
-    const long long n1 = Mpad * m->width;
-    k_layer1<<<(unsigned)((n1 + 255) / 256), 256, 0, st>>>(X, (int)M, (int)Mpad, m->W[0], m->b[0], sh,
-                                                          sc, m->width, m->xf,
-                                                          keep_z ? m->Z[0] : nullptr, m->H[0]);
-    MD_CUDA_TRY(cudaGetLastError());
+template <int CS>
+int chain_launch(const TrainArgs &a, cudaStream_t st) {
+    MD_CUDA_TRY(cudaFuncSetAttribute(k_train_chain<CS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)TrainShape<CS>::smem));
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = CS;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(a.B / 128 * CS);
+    cfg.blockDim = dim3(T_THREADS);
+    cfg.dynamicSmemBytes = TrainShape<CS>::smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    MD_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_train_chain<CS>, a));
+    return MD_OK;
+}
+
+// The three launches of a training step on B rows (B % 128 == 0).
+int train_launch(mlp_model *m, const float *X, const float *T, int B, float *loss, const AdamArgs &ad, cudaStream_t st) {
+    int dev = 0, nsm = 0;
+    MD_CUDA_TRY(cudaGetDevice(&dev));
+    MD_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    TrainArgs t{};
+    t.X = X;
+    t.T = T;
+    t.B = B;
+    t.pm = m->map();
+    t.shift = make_float4(m->shift[0], m->shift[1], m->shift[2], m->shift[3]);
+    t.scale = make_float4(m->scale[0], m->scale[1], m->scale[2], m->scale[3]);
+    t.w = m->w;
     for (int l = 1; l < m->nl; ++l) {
-        GemmArgs g{};
-        g.A = m->H[l - 1];
-        g.lda = m->width;
-        g.B = m->Wh[l];
-        g.ldb = m->in[l];
-        g.M = (int)Mpad;
-        g.N = m->outp[l];
-        g.K = m->in[l];
-        g.bias = m->b[l];
-        g.status = m->status;
-        int rc;
-        if (l < m->nl - 1) {
-            g.C = keep_z ? m->Z[l] : nullptr;
-            g.ldc = m->width;
-            g.H = m->H[l];
-            g.ldh = m->width;
-            rc = gemm_launch<EPI_BIAS_SILU>(g, st);
-        } else {
-            g.C = m->logits;
-            g.ldc = m->npad;
-            rc = gemm_launch<EPI_BIAS_F32>(g, st);
-        }
-        if (rc) return rc;
+        t.Wf[l] = m->Wf[l];
+        t.Wb[l] = m->Wb[l];
     }
-    return MD_OK;
-}
-
-// Column sums of dZ [M][N] (bias gradient) over the batch, two passes.
-int colsum(const bf16 *dZ, int M, int N, float *part, float *out, cudaStream_t st) {
-    const int nch = (M + GRAD_ROWS - 1) / GRAD_ROWS;
-    k_colsum_part<<<dim3((N + 127) / 128, nch), 128, 0, st>>>(dZ, M, N, N, part);
-    k_sum_parts<<<(N + 255) / 256, 256, 0, st>>>(part, nch, N, 1, N, N, out, N);
-    MD_CUDA_TRY(cudaGetLastError());
-    return MD_OK;
-}
-
-int transpose(const bf16 *in, int R, int C, bf16 *out, cudaStream_t st) {
-    dim3 tb(32, 8), gr((C + 31) / 32, (R + 31) / 32);
-    k_transpose<<<gr, tb, 0, st>>>(in, R, C, out);
-    MD_CUDA_TRY(cudaGetLastError());
-    return MD_OK;
-}
-
-// Loss (device scalar, optional) and gradients of a batch of Mb rows
-// (Mb % 128 == 0) into gW / gb.
-int backward(mlp_model *m, const float *X, const float *T, int Mb, float *loss_dev, cudaStream_t st) {
-    int rc = forward(m, X, Mb, Mb, true, st);
+    t.xf = m->xf;
+    t.Z = m->Z;
+    t.H = m->H;
+    t.dZ = m->dZ;
+    t.rowloss = m->rowloss;
+    t.inv_batch = 1.0f / (float)B;
+    t.status = m->status;
+    // four CTAs per row block while the device has SMs for them, else two
+    // (CTAs beyond the device then queue)
+    int rc = B / 128 * 4 <= nsm ? chain_launch<4>(t, st) : chain_launch<2>(t, st);
     if (rc) return rc;
-    k_softmax<<<(Mb + 7) / 8, 256, 0, st>>>(m->logits, m->npad, Mb, m->ncls, nullptr, T, m->rowloss,
-                                            m->dlog, m->npad, 1.0f / (float)Mb);
+    GradArgs g{};
+    g.H = m->H;
+    g.dZ = m->dZ;
+    g.xf = m->xf;
+    g.B = B;
+    g.ks = grad_splits(B);
+    g.pm = t.pm;
+    g.part = m->part;
+    g.bpart = m->bpart;
+    g.wpart = m->wpart;
+    g.status = m->status;
+    const int nch = B / GRAD_ROWS;
+    MD_CUDA_TRY(cudaFuncSetAttribute(k_train_grads, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GRADS_SMEM));
+    k_train_grads<<<grad_tiles(g.pm) * g.ks + grad_sums(g.pm) / 128 * nch, 128, GRADS_SMEM, st>>>(g);
     MD_CUDA_TRY(cudaGetLastError());
-    if (loss_dev) {
-        k_sum<<<1, 256, 0, st>>>(m->rowloss, Mb, loss_dev);
-        MD_CUDA_TRY(cudaGetLastError());
+    UpdateArgs u{};
+    u.pm = t.pm;
+    u.part = m->part;
+    u.bpart = m->bpart;
+    u.wpart = m->wpart;
+    u.ks = g.ks;
+    u.nch = nch;
+    u.w = m->w;
+    u.mom = m->mom;
+    u.var = m->var;
+    for (int l = 1; l < m->nl; ++l) {
+        u.Wf[l] = m->Wf[l];
+        u.Wb[l] = m->Wb[l];
     }
-    // dZ of the current layer (layer L: dlogits) and its width
-    const bf16 *dZ = m->dlog;
-    int dzw = m->npad;
-    bf16 *bufs[2] = {m->dA, m->dB};
-    for (int l = m->nl - 1; l >= 1; --l) {
-        // dW_l = dZ^T H_{l-1}; db_l = colsum(dZ)
-        if ((rc = transpose(dZ, Mb, dzw, m->tA, st))) return rc;
-        if ((rc = transpose(m->H[l - 1], Mb, m->width, m->tB, st))) return rc;
-        GemmArgs g{};
-        g.A = m->tA;
-        g.lda = Mb;
-        g.B = m->tB;
-        g.ldb = Mb;
-        g.M = dzw;
-        g.N = m->width;
-        g.K = Mb;
-        g.ldc = m->in[l];
-        g.status = m->status;
-        // K = the batch: split over up to GRAD_MAX_SPLIT CTAs per tile row
-        // (two stages each at least), partial tiles summed in split order
-        const int nkt = Mb / GBK;
-        int ks = 1;
-        while (ks * 2 <= GRAD_MAX_SPLIT && nkt % (ks * 2) == 0 && nkt / (ks * 2) >= 2) ks *= 2;
-        if (ks == 1) {
-            g.C = m->gW[l];
-            if ((rc = gemm_launch<EPI_F32>(g, st))) return rc;
-        } else {
-            g.K = Mb / ks;
-            g.C = m->part;
-            g.c_split = (long long)dzw * g.ldc;
-            if ((rc = gemm_launch<EPI_F32>(g, st, ks))) return rc;
-            const long long n = (long long)dzw * m->width;
-            k_sum_parts<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(m->part, ks, g.c_split, dzw, m->width, g.ldc,
-                                                                    m->gW[l], g.ldc);
-        }
-        if ((rc = colsum(dZ, Mb, dzw, m->part, m->gb[l], st))) return rc;
-        // dZ_{l-1} = (dZ W_l) * silu'(Z_{l-1})
-        GemmArgs d{};
-        d.A = dZ;
-        d.lda = dzw;
-        d.B = m->Wt[l];
-        d.ldb = m->outp[l];
-        d.M = Mb;
-        d.N = m->width;
-        d.K = dzw;
-        d.H = bufs[l & 1];
-        d.ldh = m->width;
-        d.Zp = m->Z[l - 1];
-        d.ldz = m->width;
-        d.status = m->status;
-        if ((rc = gemm_launch<EPI_DSILU>(d, st))) return rc;
-        dZ = bufs[l & 1];
-        dzw = m->width;
-    }
-    const int nch = (Mb + GRAD_ROWS - 1) / GRAD_ROWS;
-    k_grad_layer1_part<<<dim3((m->width * 4 + 127) / 128, nch), 128, 0, st>>>(dZ, Mb, m->width, m->xf, m->part);
-    k_sum_parts<<<(m->width * 4 + 255) / 256, 256, 0, st>>>(m->part, nch, (long long)m->width * 4, 1,
-                                                            m->width * 4, m->width * 4, m->gW[0], m->width * 4);
+    u.rowloss = m->rowloss;
+    u.B = B;
+    u.loss = loss;
+    k_train_update<<<(t.pm.count() + 255) / 256 + 1, 256, 0, st>>>(u, ad);
     MD_CUDA_TRY(cudaGetLastError());
-    return colsum(dZ, Mb, m->width, m->part, m->gb[0], st);
+    return MD_OK;
 }
-
 
 }  // namespace
 
@@ -988,38 +1330,27 @@ int mlp_create(int32_t n_hidden, int32_t width, int32_t n_classes, const float *
     m->npad = 128;
     std::memcpy(m->shift, shift4, sizeof(m->shift));
     std::memcpy(m->scale, scale4, sizeof(m->scale));
-    for (int l = 0; l < m->nl; ++l) {
-        m->in.push_back(l == 0 ? 4 : width);
-        m->out.push_back(l == m->nl - 1 ? n_classes : width);
-        m->outp.push_back(l == m->nl - 1 ? m->npad : width);
-    }
+    const ParamMap pm = m->map();
     int rc = MD_OK;
     auto A = [&](void **p, size_t bytes) {
         if (rc == MD_OK) rc = malloc_into(m->allocs, p, bytes);
     };
-    m->W.assign(m->nl, nullptr);
-    m->b = m->mW = m->vW = m->mb = m->vb = m->gW = m->gb = m->W;
-    m->Wh.assign(m->nl, nullptr);
-    m->Wt.assign(m->nl, nullptr);
-    m->Wp.assign(m->nl, nullptr);
-    m->Bp.assign(m->nl, nullptr);
+    const size_t np = (size_t)pm.count() * sizeof(float);
+    A((void **)&m->w, np);
+    A((void **)&m->mom, np);
+    A((void **)&m->var, np);
+    A((void **)&m->g, np);
+    m->Wf.assign(m->nl, nullptr);
+    m->Wb = m->Wp = m->Bp = m->Wf;
     for (int l = 0; l < m->nl; ++l) {
-        const size_t nw = (size_t)m->outp[l] * m->in[l], nbias = (size_t)m->outp[l];
-        A((void **)&m->W[l], nw * 4);
-        A((void **)&m->mW[l], nw * 4);
-        A((void **)&m->vW[l], nw * 4);
-        A((void **)&m->gW[l], nw * 4);
-        A((void **)&m->b[l], nbias * 4);
-        A((void **)&m->mb[l], nbias * 4);
-        A((void **)&m->vb[l], nbias * 4);
-        A((void **)&m->gb[l], nbias * 4);
+        const size_t nw = (size_t)pm.outp(l) * pm.in(l);
         if (l > 0) {
-            A((void **)&m->Wh[l], nw * 2);
-            A((void **)&m->Wt[l], nw * 2);
+            A((void **)&m->Wf[l], nw * 2);
+            A((void **)&m->Wb[l], nw * 2);
             A((void **)&m->Wp[l], nw * 2);
-            A((void **)&m->Bp[l], (size_t)m->outp[l] * 16 * 2);
+            A((void **)&m->Bp[l], (size_t)pm.outp(l) * 16 * 2);
         } else {
-            A((void **)&m->Wp[0], (size_t)m->outp[0] * 16 * 2);
+            A((void **)&m->Wp[0], (size_t)pm.outp(0) * 16 * 2);
         }
     }
     A((void **)&m->status, sizeof(int));
@@ -1027,15 +1358,8 @@ int mlp_create(int32_t n_hidden, int32_t width, int32_t n_classes, const float *
         mlp_destroy(m);
         return rc;
     }
-    for (int l = 0; l < m->nl; ++l) {
-        const size_t nw = (size_t)m->outp[l] * m->in[l];
-        cudaMemset(m->W[l], 0, nw * 4);
-        cudaMemset(m->b[l], 0, m->outp[l] * 4);
-        cudaMemset(m->mW[l], 0, nw * 4);
-        cudaMemset(m->vW[l], 0, nw * 4);
-        cudaMemset(m->mb[l], 0, m->outp[l] * 4);
-        cudaMemset(m->vb[l], 0, m->outp[l] * 4);
-    }
+    cudaMemset(m->mom, 0, np);
+    cudaMemset(m->var, 0, np);
     cudaMemset(m->status, 0, sizeof(int));
     rc = mlp_set_params(m, params);
     if (rc) {
@@ -1054,23 +1378,11 @@ void mlp_destroy(mlp_model *m) {
     delete m;
 }
 
-int64_t mlp_param_count(mlp_model *m) {
-    if (!m) return 0;
-    int64_t n = 0;
-    for (int l = 0; l < m->nl; ++l) n += (int64_t)m->out[l] * m->in[l] + m->out[l];
-    return n;
-}
+int64_t mlp_param_count(mlp_model *m) { return m ? m->map().count() : 0; }
 
 int mlp_set_params(mlp_model *m, const float *params) {
     if (!m || !params) return fail(MD_E_ARG, "mlp_set_params: NULL argument");
-    size_t off = 0;
-    for (int l = 0; l < m->nl; ++l) {
-        const size_t nw = (size_t)m->out[l] * m->in[l];
-        MD_CUDA_TRY(cudaMemcpy(m->W[l], params + off, nw * 4, cudaMemcpyDefault));   // rows >= out stay 0
-        off += nw;
-        MD_CUDA_TRY(cudaMemcpy(m->b[l], params + off, m->out[l] * 4, cudaMemcpyDefault));
-        off += m->out[l];
-    }
+    MD_CUDA_TRY(cudaMemcpy(m->w, params, sizeof(float) * m->map().count(), cudaMemcpyDefault));
     int rc = refresh_bf16(m, nullptr);
     if (rc) return rc;
     MD_CUDA_TRY(cudaDeviceSynchronize());
@@ -1080,14 +1392,7 @@ int mlp_set_params(mlp_model *m, const float *params) {
 int mlp_get_params(mlp_model *m, float *params) {
     if (!m || !params) return fail(MD_E_ARG, "mlp_get_params: NULL argument");
     MD_CUDA_TRY(cudaDeviceSynchronize());
-    size_t off = 0;
-    for (int l = 0; l < m->nl; ++l) {
-        const size_t nw = (size_t)m->out[l] * m->in[l];
-        MD_CUDA_TRY(cudaMemcpy(params + off, m->W[l], nw * 4, cudaMemcpyDefault));
-        off += nw;
-        MD_CUDA_TRY(cudaMemcpy(params + off, m->b[l], m->out[l] * 4, cudaMemcpyDefault));
-        off += m->out[l];
-    }
+    MD_CUDA_TRY(cudaMemcpy(params, m->w, sizeof(float) * m->map().count(), cudaMemcpyDefault));
     return MD_OK;
 }
 
@@ -1097,12 +1402,13 @@ int mlp_forward(mlp_model *m, const float *X, int64_t M, float *P_out, void *str
     if ((uintptr_t)X & 15) return fail(MD_E_ARG, "mlp_forward: X must be 16-byte aligned");
     cudaStream_t st = (cudaStream_t)stream;
     if (!m->packed) {
-        k_pack0<<<16, 256, 0, st>>>(m->W[0], m->b[0], m->nl > 1 ? 0.5f : 1.0f, m->Wp[0]);
+        const ParamMap pm = m->map();
+        k_pack0<<<16, 256, 0, st>>>(m->w, m->w + pm.b(0), m->nl > 1 ? 0.5f : 1.0f, m->Wp[0]);
         for (int l = 1; l < m->nl; ++l) {
-            const int n = m->outp[l] * 256;
+            const int n = pm.outp(l) * 256;
             const float sc = l < m->nl - 1 ? 0.5f : 1.0f;
-            k_pack<<<(n + 255) / 256, 256, 0, st>>>(m->Wh[l], m->outp[l], sc, m->Wp[l]);
-            k_packb<<<(m->outp[l] * 16 + 255) / 256, 256, 0, st>>>(m->b[l], m->outp[l], sc, m->Bp[l]);
+            k_pack<<<(n + 255) / 256, 256, 0, st>>>(m->w + pm.W(l), pm.out(l), pm.outp(l), sc, m->Wp[l]);
+            k_packb<<<(pm.outp(l) * 16 + 255) / 256, 256, 0, st>>>(m->w + pm.b(l), pm.out(l), pm.outp(l), sc, m->Bp[l]);
         }
         MD_CUDA_TRY(cudaGetLastError());
         m->packed = true;
@@ -1138,40 +1444,30 @@ int mlp_grad(mlp_model *m, const float *X, const float *T, int32_t B, float *gra
     cudaStream_t st = (cudaStream_t)stream;
     int rc = ensure_ws(m, B);
     if (rc) return rc;
-    if ((rc = backward(m, X, T, B, loss_out, st))) return rc;
-    if (grad_out) {
-        size_t off = 0;
-        for (int l = 0; l < m->nl; ++l) {
-            const size_t nw = (size_t)m->out[l] * m->in[l];
-            MD_CUDA_TRY(cudaMemcpyAsync(grad_out + off, m->gW[l], nw * 4, cudaMemcpyDefault, st));
-            off += nw;
-            MD_CUDA_TRY(cudaMemcpyAsync(grad_out + off, m->gb[l], m->out[l] * 4, cudaMemcpyDefault, st));
-            off += m->out[l];
-        }
-    }
+    AdamArgs ad{};
+    ad.g = m->g;
+    if ((rc = train_launch(m, X, T, B, loss_out, ad, st))) return rc;
+    if (grad_out) MD_CUDA_TRY(cudaMemcpyAsync(grad_out, m->g, sizeof(float) * m->map().count(), cudaMemcpyDefault, st));
     return MD_OK;
 }
 
 int mlp_train_step(mlp_model *m, const float *X, const float *T, int32_t B, float lr,
                    float *loss_out, void *stream) {
     mdlg::Range range_("mlp_train_step");
-    int rc = mlp_grad(m, X, T, B, nullptr, loss_out, stream);
-    if (rc) return rc;
+    if (!m || !X || !T || B < 128 || B % 128) return fail(MD_E_ARG, "mlp_grad: batch must be a multiple of 128");
     cudaStream_t st = (cudaStream_t)stream;
+    int rc = ensure_ws(m, B);
+    if (rc) return rc;
+    AdamArgs ad{};
+    ad.lr = lr;
+    ad.b1 = 0.9f;
+    ad.b2 = 0.999f;
+    ad.eps = 1e-8f;
+    ad.c1 = 1.f - powf(ad.b1, (float)(m->adam_t + 1));
+    ad.c2 = 1.f - powf(ad.b2, (float)(m->adam_t + 1));
+    if ((rc = train_launch(m, X, T, B, loss_out, ad, st))) return rc;
     m->adam_t += 1;
     m->packed = false;
-    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    const float c1 = 1.f - powf(b1, (float)m->adam_t), c2 = 1.f - powf(b2, (float)m->adam_t);
-    for (int l = 0; l < m->nl; ++l) {
-        const int rows = m->out[l], cols = m->in[l];
-        k_adam<<<(rows * cols + 255) / 256, 256, 0, st>>>(m->W[l], m->mW[l], m->vW[l], m->gW[l], rows,
-                                                          cols, cols, lr, b1, b2, c1, c2, eps,
-                                                          l ? m->Wh[l] : nullptr,
-                                                          l ? m->Wt[l] : nullptr, m->outp[l]);
-        k_adam<<<(rows + 255) / 256, 256, 0, st>>>(m->b[l], m->mb[l], m->vb[l], m->gb[l], 1, rows, rows,
-                                                   lr, b1, b2, c1, c2, eps, nullptr, nullptr, 0);
-    }
-    MD_CUDA_TRY(cudaGetLastError());
     return MD_OK;
 }
 
@@ -1206,7 +1502,7 @@ int bf16_gemm_selftest(const void *A, const void *B, float *C, int32_t M, int32_
     g.dbg_skip_commit = 1;   // stage 0
     cudaStream_t st = (cudaStream_t)stream;
     MD_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int32_t), st));
-    int rc = gemm_launch<EPI_F32>(g, st);
+    int rc = gemm_launch(g, st);
     if (rc) return rc;
     int32_t h = 0;
     MD_CUDA_TRY(cudaMemcpyAsync(&h, status, sizeof(h), cudaMemcpyDeviceToHost, st));
@@ -1228,7 +1524,7 @@ int bf16_gemm_tn(const void *A, const void *B, float *C, int32_t M, int32_t N, i
     g.C = C;
     g.ldc = N;
     g.status = status;
-    return gemm_launch<EPI_F32>(g, (cudaStream_t)stream);
+    return gemm_launch(g, (cudaStream_t)stream);
 }
 
 }  // extern "C"
