@@ -169,7 +169,8 @@ int md_init_batch(const md_params *p, int32_t n_rep, const double *x, const doub
 void md_destroy(md_system *s);
 
 /* Advances every replica by nsteps velocity-Verlet steps (Sec. 4) in one
- * persistent cooperative kernel, sampling the MDLG histograms (Sec. 2) on
+ * persistent cooperative kernel (a single replica that fits the SMs' shared
+ * memory, from 16 steps on: the slab engine, see md_tune), sampling the MDLG histograms (Sec. 2) on
  * every step t = n_equil + m*lg_every[k] and rebuilding cell lists as
  * needed.  Asynchronous on the system's stream; device-side failures
  * (MD_E_TIMEOUT, MD_E_SKIN, MD_E_NONFINITE) are reported by md_sync. */
@@ -188,17 +189,24 @@ int md_step(md_system *s, int64_t nsteps);
  * the slabs of a replica exchanging their boundary rows through L2 and
  * meeting at a bounded per-replica barrier once per step; block_threads and
  * per_thread are ignored; MD_E_LIMIT if a replica fits no slab plan.
+ * staging 0 (and no md_tune at all) leaves the choice to the library: a
+ * system of a single replica whose state fits the SMs' shared memory (about
+ * 500,000 FP32 or 270,000 FP64 particles at phi = 0.08) runs calls of 16 steps
+ * or more in the slab engine, which holds one slab of cell rows per SM in
+ * shared memory for the whole call, in FP32 or FP64; everything else runs as
+ * with staging 1.  Staging 1, 2 and 3 keep to the global engine.
  * Results do not depend on the shape or the engine: particle order, force
  * summation order, every reduction order and the rebuild schedule (per
  * replica) are fixed by the data, not by the launch; only the FP64 moment
- * sums are grouped differently by the two engines (their last bits may
- * differ).  Used by md_autotune. */
+ * sums are grouped differently by the engines (their last bits may differ).
+ * Used by md_autotune. */
 int md_tune(md_system *s, int32_t block_threads, int32_t per_thread, int32_t staging);
 
 /* Autotuner: times md_step(steps_per_trial) twice for every launch shape
  * (block {256,128} x per_thread {1,2,4} x staging {1,2,3}; 3 skipped in
- * FP64; then staging 4 for FP32 batches of >= 2 replicas) and keeps the
- * fastest; the choice is cached for the process by (precision, replicas,
+ * FP64; then the slab engine for a single replica, or staging 4 for FP32
+ * batches of >= 2 replicas) and keeps the fastest (best3 names the fastest
+ * global shape also where the slab engine was faster still); the choice is cached for the process by (precision, replicas,
  * particle count rounded up to a power of two, list capacity) and reused
  * without trials.  The trial steps are real MD steps: the system advances
  * by them (the trajectory itself does not depend on the shape).  best3
@@ -261,9 +269,11 @@ int md_set_state(md_system *s, const double *x, const double *y, const double *v
  * sizes) and synchronises.  Running k steps, saving, loading into a fresh
  * system and running m more steps gives the same bits as k + m steps
  * straight: positions, velocities, snapshots, histograms and overflow on
- * either engine, the FP64 moment sums too on the global engine (the
- * resident engine sums a slab's moment terms in its slot order, which a
- * load resets, so their last bits may differ).  The buffer format is that
+ * every engine, the FP64 moment sums too on the global engine (the resident
+ * engine sums a slab's moment terms in its slot order, which a load resets,
+ * so their last bits may differ; the slab engine's sums do not depend on the
+ * order, but md_step calls must be split alike, since calls below 16 steps
+ * run on the global engine).  The buffer format is that
  * of this library build only. */
 int md_checkpoint_bytes(md_system *s, int64_t *bytes);
 int md_checkpoint_save(md_system *s, void *buf);

@@ -16,6 +16,7 @@
 #include "equilibria.cuh"
 #include "md_kernels.cuh"
 #include "md_resident.cuh"
+#include "md_slab.cuh"
 
 namespace mdlg {
 
@@ -632,6 +633,12 @@ struct md_system {
     // order; global: sorted within each chunk of the chunk table), so a new
     // shape's first launch rebuilds them (sort only)
     bool lists_valid = false;
+    // slab engine (a single replica): its plan and buffers (slab_ok: it has
+    // one), whether md_step may take it, and whether the state is as its last
+    // launch left it
+    SlabDev sl{};
+    size_t slab_smem = 0;
+    bool slab_ok = false, slab_on = true, slab_last = false;
     std::vector<void *> res_allocs;
     ResDev rd{};
     int res_grid = 0;
@@ -989,7 +996,7 @@ int configure_launch(md_system *s, int block, int ppt, int stage) {
     return MD_OK;
 }
 
-int launch_persistent(md_system *s, long long nsteps, int force_rebuild);
+int launch_persistent(md_system *s, long long nsteps, int force_rebuild, const long long *left = nullptr);
 
 // The global engine's invariants (slots sorted by cell, by id inside a cell,
 // cell_start, Verlet lists) after a resident launch: a sort-only rebuild,
@@ -1000,7 +1007,8 @@ int ensure_sorted(md_system *s) {
     return launch_persistent(s, 0, RB_NONE);
 }
 
-int launch_persistent(md_system *s, long long nsteps, int force_rebuild) {
+int launch_persistent(md_system *s, long long nsteps, int force_rebuild, const long long *left) {
+    s->slab_last = false;
     if (force_rebuild != RB_ALL) {
         if (s->needs_sort || !s->lists_valid) force_rebuild = RB_NONE;
         s->needs_sort = false;
@@ -1011,10 +1019,114 @@ int launch_persistent(md_system *s, long long nsteps, int force_rebuild) {
     const void *fn = persistent_fn(s->prec, s->block, s->stage);
     long long step0 = s->step;
     int phase = s->phase_half;
-    void *args[] = {&s->sd, &step0, &nsteps, &phase, &force_rebuild};
+    void *args[] = {&s->sd, &step0, &nsteps, &phase, &force_rebuild, &left};
     MD_CUDA_TRY(cudaMemsetAsync(&s->d_ctl->claims, 0, sizeof(unsigned long long), s->st));
     MD_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3(s->grid), dim3(s->block), args, s->smem, s->st));
     return MD_OK;
+}
+
+// ---- slab engine ------------------------------------------------------------
+const void *slab_fn(int prec) {
+    return prec == MD_FP64 ? (const void *)k_md_slab<double> : (const void *)k_md_slab<float>;
+}
+SlabLayout slab_layout_of(const md_system *s, int p_cap, int h_cap, int e_cap, int ncells, int threads) {
+    const size_t hb = smem_hist_bytes(s->n_lg, s->n_dx, s->nb);
+    return s->prec == MD_FP64 ? slab_layout<double>(hb, p_cap, h_cap, e_cap, ncells, threads)
+                              : slab_layout<float>(hb, p_cap, h_cap, e_cap, ncells, threads);
+}
+
+// Plans the slabs of a single replica: as many as SMs, of at least two cell
+// rows in FP32 and one in FP64 (whose force pass is long enough to pay for
+// more slabs), with all the room the SM's shared memory gives beyond what the
+// mean density needs (at least 1.05 times the largest slab's mean count and
+// 1.1 times a row's, plus five standard deviations of a Poisson count; lists
+// 1.25 times the mean neighbour count plus 2 per particle).  No plan where
+// that does not fit, e.g. more than about 4,000 FP32 particles per SM.
+int plan_slab(md_system *s) {
+    if (s->nrep != 1) return MD_OK;
+    const RepDev &R = s->reps[0];
+    int optin = 0;
+    MD_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, s->dev));
+    cudaFuncAttributes fa{};
+    MD_CUDA_TRY(cudaFuncGetAttributes(&fa, slab_fn(s->prec)));
+    const size_t smem = (size_t)optin - fa.sharedSizeBytes;
+    int g = std::min(std::min(s->nsm, s->prec == MD_FP64 ? R.nc : R.nc / 2), R.cap / 32);
+    if (g < 2) g = 1;
+    const int rows = (R.nc + g - 1) / g, ncells = (g == 1 ? R.nc : rows + 2) * R.nc;
+    const double pmax = (double)R.n * rows / R.nc, row = (double)R.n / R.nc;
+    const double cbar = M_PI * R.rv2 * (double)R.n / (R.L * R.L);
+    const double p_want = 1.05 * pmax + 5.0 * std::sqrt(pmax) + 32.0;
+    const double h_want = g == 1 ? 0.0 : 1.1 * row + 5.0 * std::sqrt(row) + 32.0;
+    // FP64 shares a particle's pairs among lanes, so small slabs take more warps than particles
+    const int lo = s->prec == MD_FP64 ? 256 : 128;
+    const int threads = std::min(s->prec == MD_FP64 ? SLAB_THREADS<double> : SLAB_THREADS<float>, std::max(lo, round_up((long long)std::ceil(s->prec == MD_FP64 ? 4.0 * pmax : pmax), 32)));
+    SlabDev D{};
+    for (double f = 3.0; f > 0.99 && !D.p_cap; f -= 0.05) {
+        const int p = (int)std::min<double>(R.n, std::ceil(f * p_want));
+        const int h = (int)std::min<double>(R.n, std::ceil(f * h_want));
+        const double e = std::ceil(p * (1.25 * cbar + 2.0)) + 256.0;
+        if (p + 2 * h >= SLAB_MAX_IDX || e > 1e6) continue;
+        if (slab_layout_of(s, p, h, (int)e, ncells, threads).end > smem) continue;
+        D.p_cap = p;
+        D.h_cap = std::max(h, 1);
+        D.e_cap = (int)e;
+    }
+    if (!D.p_cap) return MD_OK;
+    D.g = g;
+    D.ncells = ncells;
+    D.threads = threads;
+    const size_t vsz = s->prec == MD_FP64 ? sizeof(double2) : sizeof(float2), gh = (size_t)g * D.h_cap;
+    int rc = MD_OK;
+    auto A = [&](void **p, size_t bytes) {
+        if (rc == MD_OK) rc = dalloc(s, p, bytes);
+    };
+    A((void **)&D.word, sizeof(unsigned long long) * 2 * g * g);
+    A(&D.halo_off, vsz * 4 * gh);
+    A((void **)&D.halo_ci, sizeof(uint2) * 2 * gh);
+    A((void **)&D.halo_n, sizeof(int32_t) * 2 * g);
+    A(&D.mig_off, vsz * 2 * gh);
+    A(&D.mig_vel, vsz * 2 * gh);
+    A((void **)&D.mig_ci, sizeof(uint2) * 2 * gh);
+    A((void **)&D.mig_n, sizeof(int32_t) * 2 * g);
+    A((void **)&D.slab_n, sizeof(int32_t) * g);
+    A((void **)&D.left, sizeof(long long));
+    if (rc) return rc;
+    s->slab_smem = slab_layout_of(s, D.p_cap, D.h_cap, D.e_cap, ncells, threads).end;
+    MD_CUDA_TRY(cudaFuncSetAttribute(slab_fn(s->prec), cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes));
+    int occ = 0;
+    MD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, slab_fn(s->prec), threads, s->slab_smem));
+    s->sl = D;
+    s->slab_ok = occ >= 1;
+    return MD_OK;
+}
+
+int launch_slab(md_system *s, long long nsteps) {
+    if (!s->slab_last) {
+        // cell_start must describe the slots' order
+        int rc = ensure_sorted(s);
+        if (rc) return rc;
+    }
+    long long step0 = s->step;
+    int phase = s->phase_half;
+    void *args[] = {&s->sd, &s->sl, &step0, &nsteps, &phase};
+    MD_CUDA_TRY(cudaMemsetAsync(s->sl.word, 0, sizeof(unsigned long long) * 2 * s->sl.g * s->sl.g, s->st));
+    MD_CUDA_TRY(cudaLaunchCooperativeKernel(slab_fn(s->prec), dim3(s->sl.g), dim3(s->sl.threads), args, s->slab_smem,
+                                            s->st));
+    int rc = launch_persistent(s, nsteps, RB_NONE, s->sl.left);
+    if (rc) return rc;
+    s->needs_sort = true;
+    s->slab_last = true;
+    return MD_OK;
+}
+
+// A slab launch loads, builds its lists, writes back and is followed by the
+// (empty) global launch, about 25 us, and a readout after it has to sort; it
+// gains 2 to 30 us per step.  From this many steps on it is taken (and always
+// from a state that it left itself).
+constexpr int64_t SLAB_MIN_STEPS = 16;
+
+bool takes_slab(const md_system *s, int64_t nsteps) {
+    return s->engine == 0 && s->slab_ok && s->slab_on && (s->slab_last || nsteps >= SLAB_MIN_STEPS);
 }
 
 int status_to_code(int ds) {
@@ -1294,6 +1406,7 @@ int md_init_batch(const md_params *p, int32_t n_rep, const double *x, const doub
         tryc(cudaGetLastError());
     }
     if (rc == MD_OK) rc = configure_launch(s, 256, default_ppt(s), 1);
+    if (rc == MD_OK) rc = plan_slab(s);
     if (rc == MD_OK) rc = upload_state(s, x, y, vx, vy);
     if (rc) {
         md_destroy(s);
@@ -1348,7 +1461,8 @@ int md_step(md_system *s, int64_t nsteps) {
     mdlg::Range range_("md_step");
     if (!s || nsteps < 0) return fail(MD_E_ARG, "md_step: bad arguments");
     if (nsteps == 0) return MD_OK;
-    int rc = s->engine == 1 ? launch_resident(s, nsteps) : launch_persistent(s, nsteps, 0);
+    int rc = s->engine == 1 ? launch_resident(s, nsteps)
+                            : (takes_slab(s, nsteps) ? launch_slab(s, nsteps) : launch_persistent(s, nsteps, 0));
     if (rc) return rc;
     s->step += nsteps;
     s->phase_half = 1;
@@ -1359,7 +1473,9 @@ int md_tune(md_system *s, int32_t block_threads, int32_t per_thread, int32_t sta
     if (!s) return fail(MD_E_ARG, "md_tune: NULL system");
     if (block_threads == 0) block_threads = 256;
     if (per_thread == 0) per_thread = default_ppt(s);
+    const bool slab = staging == 0;   // the default: the slab engine where a single replica has a plan
     if (staging == 0) staging = 1;
+    if (staging >= 1 && staging <= 3) s->slab_on = slab;
     return configure_launch(s, block_threads, per_thread, staging);
 }
 
@@ -1812,6 +1928,7 @@ namespace {
 std::mutex g_tune_mu;
 std::map<std::tuple<int, int, int, int>, std::tuple<int, int, int>> g_tune_cache;
 std::map<std::tuple<int, int, int, int>, std::vector<double>> g_tune_costs;   // resident slab times
+std::map<std::tuple<int, int, int, int>, bool> g_tune_slab;   // the slab engine was the fastest
 }
 
 int md_autotune(md_system *s, int64_t steps_per_trial, int32_t *best3) {
@@ -1831,6 +1948,7 @@ int md_autotune(md_system *s, int64_t steps_per_trial, int32_t *best3) {
                          : configure_launch(s, std::get<0>(it->second), std::get<1>(it->second),
                                             std::get<2>(it->second));
             if (rc) return rc;
+            s->slab_on = g_tune_slab[key];
             if (best3) {
                 best3[0] = std::get<0>(it->second);
                 best3[1] = std::get<1>(it->second);
@@ -1846,6 +1964,7 @@ int md_autotune(md_system *s, int64_t steps_per_trial, int32_t *best3) {
     int bb = 256, bp = 1, bs = 1;
     const int blocks[2] = {256, 128}, ppts[3] = {1, 2, 4}, stages[3] = {1, 2, 3};
     int rc = MD_OK;
+    s->slab_on = false;
     for (int b : blocks)
         for (int p : ppts)
             for (int st : stages) {
@@ -1867,6 +1986,21 @@ int md_autotune(md_system *s, int64_t steps_per_trial, int32_t *best3) {
                     bs = st;
                 }
             }
+    // the slab engine of a single replica, whatever the global shape
+    bool slab = false;
+    if (rc == MD_OK && s->slab_ok && configure_launch(s, bb, bp, bs) == MD_OK) {
+        s->slab_on = true;
+        rc = md_step(s, steps_per_trial);
+        cudaEventRecord(e0, s->st);
+        if (rc == MD_OK) rc = md_step(s, steps_per_trial);
+        cudaEventRecord(e1, s->st);
+        cudaEventSynchronize(e1);
+        float ms = 0.0f;
+        cudaEventElapsedTime(&ms, e0, e1);
+        slab = ms < best_ms;
+    }
+    if (steps_per_trial < SLAB_MIN_STEPS) slab = s->slab_ok;   // too short to have run there
+    s->slab_on = slab;
     // the shared-memory-resident engine (batched FP32 ensembles): a trial
     // with the modelled slab costs, then one with the schedule re-planned
     // from the slabs' measured times (the per-replica work split this
@@ -1913,6 +2047,7 @@ int md_autotune(md_system *s, int64_t steps_per_trial, int32_t *best3) {
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         g_tune_cache[key] = std::make_tuple(bb, bp, bs);
+        g_tune_slab[key] = slab;
         g_tune_costs[key] = res_cost;
     }
     if (best3) {

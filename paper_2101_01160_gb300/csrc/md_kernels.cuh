@@ -65,7 +65,7 @@ struct Control {
     unsigned bar_count, bar_gen;
     int status;
     int set, cur;
-    int pad0;
+    int slab_order;       // the state is in the order a slab launch left it in (SlabDev::slab_n), not sorted
     long long n_rebuilds;
     unsigned vmax[3];     // global engine: per-step max |v| dt / half_skin (float bits), by step mod 3
     unsigned pad1;
@@ -155,6 +155,14 @@ __device__ __forceinline__ double fmaT(double a, double b, double c) { return __
 __device__ __forceinline__ float axpyT(float a, float b, float c) { return __fadd_rn(a, __fmul_rn(b, c)); }
 __device__ __forceinline__ double axpyT(double a, double b, double c) { return __dadd_rn(a, __dmul_rn(b, c)); }
 
+// Force over distance of a pair within the cutoff; s6 = (sigma / r)^6.
+template <typename T> __device__ __forceinline__ T lj_pair_fr(T r2, T eps24, T sig2, T &s6) {
+    const T ir2 = inv_r2(r2);
+    const T s2 = sig2 * ir2;
+    s6 = s2 * s2 * s2;
+    return eps24 * s6 * fmaT(T(2), s6, T(-1)) * ir2;
+}
+
 // One pair: separation (rx, ry) = x_j - x_i; accumulates the force on i.
 // Written with explicit fused multiply-adds so that every caller evaluates
 // it with the same roundings.
@@ -163,10 +171,8 @@ __device__ __forceinline__ void lj_pair_acc(T rx, T ry, T rc2, T eps24, T sig2, 
                                             double vshift, double &pe, double &fabs_sum) {
     const T r2 = fmaT(rx, rx, ry * ry);
     if (r2 < rc2) {
-        const T ir2 = inv_r2(r2);
-        const T s2 = sig2 * ir2;
-        const T s6 = s2 * s2 * s2;
-        const T fr = eps24 * s6 * fmaT(T(2), s6, T(-1)) * ir2;
+        T s6;
+        const T fr = lj_pair_fr<T>(r2, eps24, sig2, s6);
         fx = fmaT(-fr, rx, fx);
         fy = fmaT(-fr, ry, fy);
         if (kPE) {
@@ -835,7 +841,10 @@ __device__ bool rebuild(const SysDev &S, int &set, int &cur, unsigned &gen, int 
         }
         if (__syncthreads_or(over) && tid == 0) atomicOr(&C->status, (int)DS_NBR_OVERFLOW);
     }
-    if (blockIdx.x == 0 && tid == 0) C->n_rebuilds += 1;
+    if (blockIdx.x == 0 && tid == 0) {
+        C->n_rebuilds += 1;
+        C->slab_order = 0;
+    }
     if (!S.stage && !grid_sync(bar, gen, S.timeout_ns)) return false;
     return true;
 }
@@ -1005,7 +1014,8 @@ template <typename T, int BLOCK, bool DENSE>
 __global__ void __launch_bounds__(BLOCK, md_min_ctas(BLOCK, DENSE)) k_md_persistent(SysDev S, long long step0,
                                                                            long long nsteps,
                                                                            int phase_half,
-                                                                           int force_rebuild) {
+                                                                           int force_rebuild,
+                                                                           const long long *left) {
     using V = typename V2<T>::type;
     extern __shared__ __align__(16) unsigned char smem[];
     const int chunk = S.ppt * BLOCK;
@@ -1019,6 +1029,15 @@ __global__ void __launch_bounds__(BLOCK, md_min_ctas(BLOCK, DENSE)) k_md_persist
     __shared__ float s_vmax[BLOCK / 32];
     __shared__ double s_dmax[BLOCK / 32];
     Control *C = S.ctl;
+    // Behind a slab launch: the last *left steps, after a sort (an early end
+    // leaves the state unsorted); as a rule there are none.  (The kernel's
+    // parameters stay as they are, in constant memory: copies of them would
+    // take registers of the 32-register budget.)
+    long long it = 0;
+    if (left) {
+        if (*left == 0 && C->slab_order) return;
+        it = nsteps - *left;
+    }
     const GridBarrier bar{&C->bar_count, &C->bar_gen, &C->status};
     const int tid = threadIdx.x, lane = tid & 31;
     unsigned gen = 0;
@@ -1050,7 +1069,7 @@ __global__ void __launch_bounds__(BLOCK, md_min_ctas(BLOCK, DENSE)) k_md_persist
             s_desc[i] = make_desc(S, S.cell[set], own_chunk(i), WinParts<T>::value);
     }
     __syncthreads();
-    for (long long it = 0; it < nsteps; ++it) {
+    for (; it < nsteps; ++it) {
         const long long s = step0 + it;
         if (tid == 0) {
             unsigned due = 0;
