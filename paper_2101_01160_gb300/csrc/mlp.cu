@@ -587,20 +587,24 @@ __global__ void k_pack_t(const float *W, int rows, int N, bf16 *out) {
 // a GEMM, two transposes, column sums, sums of partials, two Adam kernels),
 // 466 us at B = 512 for 0.7 GFLOP: launches, and epilogues that read and
 // wrote one row per lane.  It is three launches now; of 5 layers at B = 512:
-// k_train_chain 58 us, k_train_grads 7.1 us, k_train_update 4.2 us.
+// k_train_chain 41 us, k_train_grads 7.1 us, k_train_update 4.2 us.
 //
 // k_train_chain: one thread-block cluster of CS CTAs per 128-row tile runs the
 // whole forward pass, the softmax and loss, and the backward pass down to the
 // first layer.  CTA `rank` computes columns rank * 256/CS .. of every layer:
 // its slice of the weights arrives by bulk copies while the previous layer is
 // computed, the accumulator is a 128 x 256/CS tile in TMEM, and the finished
-// BF16 activations (or gradients) are written into the next A operand of all
-// CS CTAs through distributed shared memory, with one cluster barrier per
-// layer.  What it leaves in global memory is transposed, [column][batch], so
+// BF16 activations (or gradients) go into the CTA's own next A operand and
+// from there, as contiguous 64-column slabs, to the other CTAs' by bulk copies
+// through distributed shared memory that signal the receiver's mbarrier: no
+// cluster barrier per layer.  (Storing every 16 bytes into all CTAs and
+// meeting at a cluster barrier took 44 us per step in place of 41.)  What it leaves in global memory is transposed, [column][batch], so
 // that a warp's 32 rows are contiguous and the weight gradients' operands are
 // K-major.  The tile is one row block of 128 (the M of the instruction); the
 // columns are what is split, because a batch of 512 has only four row blocks.
-// It is bound by the latency of its 2 (layers) dependent steps.
+// It is bound by the latency of its 2 (layers) dependent steps: of about 7,000
+// clocks each, the exchange takes 2,700, the product 1,400, the epilogue 2,800
+// (16 columns of a row per thread).
 // Every value is that of the layer-by-layer formulation: the K order of the
 // products, the FP32 epilogues and the BF16 roundings are the same.
 
@@ -632,7 +636,14 @@ struct TrainArgs {
     int *status;
 };
 
-constexpr int T_THREADS = 256;
+constexpr int T_THREADS = 512;
+constexpr int T_GROUPS = T_THREADS / 128;   // column groups of a CTA's epilogue
+// A operand: slabs of 128 rows x 64 columns, each contiguous (8-row groups of
+// 1024 bytes, as the weights' chunks)
+constexpr int T_SLAB = 128 * FK * 2;
+__device__ __forceinline__ int tact_off(int r, int k) {
+    return (k >> 6) * T_SLAB + (r >> 3) * F_SBO_B + ((k >> 3) & 7) * 128 + (r & 7) * 16 + (k & 7) * 2;
+}
 constexpr int T_LOGIT_LD = 113;    // odd, > MLP_MAX_CLASSES: rows of the staged logits fall in different banks
 constexpr int T_DLOG_LD = 136;
 
@@ -643,6 +654,7 @@ template <int CS> struct TrainShape {
     static constexpr int RP = 128 / CS;            // rows of a CTA's softmax
     static constexpr int WBYTES = NS * 256 * 2;
     static constexpr size_t smem = 2 * (size_t)F_ACT_BYTES + NBUF * WBYTES + 64;
+    static_assert(CS == 2 || CS == 4, "a CTA's columns are whole 64-column slabs");
 };
 static_assert(TrainShape<2>::smem <= 232448, "training chain: shared memory above 227 KB");
 static_assert(64 * T_LOGIT_LD * 4 + 64 * T_DLOG_LD * 2 <= F_ACT_BYTES, "training chain: softmax stage");
@@ -658,8 +670,11 @@ __device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, int rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(addr), "r"(rank));
     return d;
 }
-__device__ __forceinline__ void st_cluster(uint32_t addr, uint4 v) {
-    asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+// Bulk copy of `bytes` of this CTA's shared memory to `dst` in another CTA of
+// the cluster, counted on that CTA's mbarrier `bar` (cluster addresses).
+__device__ __forceinline__ void bulk_s2cluster(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "r"(src), "r"(bytes), "r"(bar)
                  : "memory");
 }
 __device__ __forceinline__ void st_cluster(uint32_t addr, float v) {
@@ -683,19 +698,22 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
     unsigned char *wbuf = sm + 2 * F_ACT_BYTES;
     uint64_t *full = reinterpret_cast<uint64_t *>(wbuf + S::NBUF * S::WBYTES);   // [NBUF]
     uint64_t *done = full + S::NBUF;                                            // accumulator complete
-    uint32_t *s_tmem = reinterpret_cast<uint32_t *>(done + 1);
+    uint64_t *arr = done + 1;                                                   // [2] the other CTAs' columns of an A operand are here
+    uint32_t *s_tmem = reinterpret_cast<uint32_t *>(arr + 2);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int rank = (int)cluster_rank(), m0 = (int)(blockIdx.x / CS) * 128;
     const ParamMap pm = a.pm;
     const int nl = pm.nl, B = a.B, nops = 2 * (nl - 1);
-    // a warp may read only the TMEM lanes 32 (warp mod 4) .. +31: warps 0-3
-    // take the first half of the CTA's columns, warps 4-7 the second
-    const int quad = warp & 3, half = warp >> 2, r = quad * 32 + lane;
+    // a warp may read only the TMEM lanes 32 (warp mod 4) .. +31: four warps
+    // take the 128 rows of one group of the CTA's columns
+    const int quad = warp & 3, grp = warp >> 2, r = quad * 32 + lane;
     constexpr uint32_t ncols = S::NS < 32 ? 32 : S::NS;
     if (warp == 0) umma::tmem_alloc(s_tmem, ncols);
     if (tid == 0) {
         for (int i = 0; i < S::NBUF; ++i) umma::mbar_init(&full[i], 1);
         umma::mbar_init(done, 1);
+        umma::mbar_init(&arr[0], 1);
+        umma::mbar_init(&arr[1], 1);
         umma::mbar_fence_init();
     }
     umma::fence_before();
@@ -704,6 +722,10 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
     const uint32_t tmem = *s_tmem, trow = tmem + ((uint32_t)(quad * 32) << 16);
     const uint32_t act0 = umma::saddr(sm);
     bool bad = false;
+    uint32_t arr_par = 0;   // thread 0: parity of the next phase of arr[0], arr[1]
+    // operation g reads operand g & 1 up to the output layer; the backward
+    // pass starts over from the output layer's
+    const auto a_buf = [&](int g) { return g < nl - 1 ? g & 1 : (g - 1) & 1; };
     // operation g < nl - 1: layer g + 1 forward; then layers nl - 1 .. 1 backward
     const auto op_layer = [&](int g) { return g < nl - 1 ? g + 1 : 2 * (nl - 1) - g; };
     const auto load = [&](int g) {   // thread 0: this CTA's slice of the operation's weights
@@ -718,22 +740,27 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
         for (int kc = 0; kc < K / FK; ++kc)
             umma::bulk_g2s(dst + kc * ns * FK * 2, src + (size_t)kc * N * FK, (uint32_t)(ns * FK * 2), bar);
     };
-    const auto product = [&](int g, int cur) {   // thread 0: issue the operation's MMAs
+    const auto product = [&](int g) {   // thread 0: issue the operation's MMAs; operand g & 1
         const int l = op_layer(g);
         const bool fwd = g < nl - 1;
-        const int ns = (fwd ? pm.outp(l) : 256) / CS, K = fwd ? 256 : pm.outp(l);
+        const int ns = (fwd ? pm.outp(l) : 256) / CS, K = fwd ? 256 : pm.outp(l), cur = a_buf(g);
+        // waited for also after a failure: the copies always come, and no
+        // CTA may leave before those into it have landed
+        if (!umma::mbar_wait(&arr[cur], arr_par >> cur & 1u, GEMM_WAIT_NS)) bad = true;
+        arr_par ^= 1u << cur;
+        if (bad) return;
         if (!umma::mbar_wait(&full[g % S::NBUF], (g / S::NBUF) & 1, GEMM_WAIT_NS)) {
             bad = true;
             return;
         }
         umma::fence_after();
         const uint32_t idesc = umma::idesc_bf16(128, ns);
-        const uint64_t ad = umma::desc(act0 + cur * F_ACT_BYTES, 128, F_SBO_A);
+        const uint64_t ad = umma::desc(act0 + cur * F_ACT_BYTES, 128, F_SBO_B);
         const uint64_t bd = umma::desc(umma::saddr(wbuf + (g % S::NBUF) * S::WBYTES), 128, F_SBO_B);
         for (int kc = 0; kc < K / FK; ++kc)
 #pragma unroll
             for (int k4 = 0; k4 < FK / 16; ++k4)
-                umma::mma(tmem, ad + (uint64_t)((kc * (FK / 16) + k4) * 16),
+                umma::mma(tmem, ad + (uint64_t)((kc * T_SLAB) >> 4) + (uint64_t)(k4 * 16),
                           bd + (uint64_t)((kc * ns * FK * 2) >> 4) + (uint64_t)(k4 * 16), idesc, (kc | k4) ? 1u : 0u);
         umma::commit(done);
     };
@@ -743,23 +770,41 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
         umma::fence_after();
         if (tid == 0 && !bad) load(g + S::NBUF);
     };
-    // 16 BF16 values of row r, columns c .. c + 15 of the layer, into the A operand `buf` of every CTA
-    const auto spread = [&](int buf, int c, const uint32_t (&h)[8]) {
-        const uint32_t o0 = act0 + buf * F_ACT_BYTES + act_off(r, c), o1 = act0 + buf * F_ACT_BYTES + act_off(r, c + 8);
-#pragma unroll
-        for (int q = 0; q < CS; ++q) {
-            st_cluster(cluster_addr(o0, q), make_uint4(h[0], h[1], h[2], h[3]));
-            st_cluster(cluster_addr(o1, q), make_uint4(h[4], h[5], h[6], h[7]));
+    // 16 BF16 values of row r, columns c .. c + 15 of the layer, into this CTA's operand `buf`
+    const auto put = [&](int buf, int c, const uint32_t (&h)[8]) {
+        unsigned char *o = sm + buf * F_ACT_BYTES;
+        *reinterpret_cast<uint4 *>(o + tact_off(r, c)) = make_uint4(h[0], h[1], h[2], h[3]);
+        *reinterpret_cast<uint4 *>(o + tact_off(r, c + 8)) = make_uint4(h[4], h[5], h[6], h[7]);
+    };
+    // All threads, after their puts: sends `n` pieces of `bytes` of operand
+    // `buf`, `stride` apart from `off` on, to the other CTAs.  Their operand
+    // is free: a CTA computes this layer only with this CTA's columns of the
+    // last one, sent after the product that read the operand had finished.
+    const auto send = [&](int buf, int off, int n, int stride, uint32_t bytes) {
+        umma::fence_proxy_smem();
+        umma::fence_before();
+        __syncthreads();
+        umma::fence_after();
+        if (tid == 0) {
+            umma::mbar_expect_tx(&arr[buf], (uint32_t)(CS - 1) * n * bytes);
+            const uint32_t src = act0 + buf * F_ACT_BYTES + off, bar = umma::saddr(&arr[buf]);
+            for (int q = 1; q < CS; ++q) {
+                const int to = (rank + q) % CS;
+                for (int i = 0; i < n; ++i)
+                    bulk_s2cluster(cluster_addr(src + i * stride, to), src + i * stride, bytes, cluster_addr(bar, to));
+            }
         }
     };
+    const int my_slab = rank * (S::NS / FK) * T_SLAB;
+    constexpr uint32_t SLABS = S::NS / FK * T_SLAB;
     const auto put_t = [&](bf16 *dst, int c, const uint32_t (&h)[8]) {   // the same, transposed in global memory
 #pragma unroll
         for (int i = 0; i < 16; ++i)
             reinterpret_cast<uint16_t *>(dst)[(size_t)(c + i) * B + m0 + r] =
                 (uint16_t)(i & 1 ? h[i / 2] >> 16 : h[i / 2] & 0xffffu);
     };
-    constexpr int CH = S::NS / 2 < 16 ? 16 : S::NS / 2;   // columns of a half
-    constexpr int CO = S::NO / 2 < 16 ? 16 : S::NO / 2;
+    constexpr int CH = S::NS / T_GROUPS < 16 ? 16 : S::NS / T_GROUPS;   // columns of a group
+    constexpr int CO = S::NO / T_GROUPS < 16 ? 16 : S::NO / T_GROUPS;
     if (tid == 0)
         for (int g = 0; g < S::NBUF; ++g) load(g);
     cluster_sync();   // every CTA of the cluster runs: its shared memory may be written
@@ -769,86 +814,122 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
                                      a.X[4 * (size_t)(m0 + r) + 2], a.X[4 * (size_t)(m0 + r) + 3]);
         const float f0 = (x.x - a.shift.x) / a.scale.x, f1 = (x.y - a.shift.y) / a.scale.y;
         const float f2 = (x.z - a.shift.z) / a.scale.z, f3 = (x.w - a.shift.w) / a.scale.w;
-        if (rank == 0 && half == 0) reinterpret_cast<float4 *>(a.xf)[m0 + r] = make_float4(f0, f1, f2, f3);
-        const float *W = a.w, *b = a.w + pm.b(0);
-        for (int c0 = half * CH; c0 < min(S::NS, half * CH + CH); c0 += 16) {
+        if (rank == 0 && grp == 0) reinterpret_cast<float4 *>(a.xf)[m0 + r] = make_float4(f0, f1, f2, f3);
+        const float4 *W = reinterpret_cast<const float4 *>(a.w);
+        const float *b = a.w + pm.b(0);
+        for (int c0 = grp * CH; c0 < min(S::NS, grp * CH + CH); c0 += 16) {
             const int c = rank * S::NS + c0;
             uint32_t h[8];
-            float hv[2];
+            float hv[2], zz[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const float4 w = __ldg(W + c + i);
+                zz[i] = __ldg(b + c + i) + w.x * f0 + w.y * f1 + w.z * f2 + w.w * f3;
+            }
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
                 const int o = c + i;
-                const float z = b[o] + W[4 * o + 0] * f0 + W[4 * o + 1] * f1 + W[4 * o + 2] * f2 + W[4 * o + 3] * f3;
+                const float z = zz[i];
                 a.Z[(size_t)o * B + m0 + r] = z;
                 hv[i & 1] = silu(z);
                 if (i & 1) h[i / 2] = pack_bf16(hv[0], hv[1]);
             }
             put_t(a.H, c, h);
-            spread(0, c, h);
+            put(0, c, h);
         }
     }
-    cluster_sync();
-    int cur = 0;
+    send(0, my_slab, 1, 0, SLABS);
     // ---- hidden layers
     for (int g = 0; g < nl - 2; ++g) {
-        if (tid == 0 && !bad) product(g, cur);
-        const float *b = a.w + pm.b(g + 1);
+        if (tid == 0) product(g);
+        const float *b = a.w + pm.b(g + 1) + rank * S::NS + grp * CH;
         float *Z = a.Z + (size_t)(g + 1) * 256 * B;
         bf16 *H = a.H + (size_t)(g + 1) * 256 * B;
+        float bias[CH];   // requested while the product runs
+#pragma unroll
+        for (int i = 0; i < CH; ++i) bias[i] = grp * CH < S::NS ? __ldg(b + i) : 0.f;
         finish(g);
-        for (int c0 = half * CH; c0 < min(S::NS, half * CH + CH); c0 += 16) {
-            const int c = rank * S::NS + c0;
+#pragma unroll
+        for (int c1 = 0; c1 < CH; c1 += 16) {
+            const int c0 = grp * CH + c1, c = rank * S::NS + c0;
+            if (c0 >= S::NS) break;
             float v[16];
             umma::ld16(trow + (uint32_t)c0, v);
             uint32_t h[8];
             float hv[2];
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
-                const float z = v[i] + b[c + i];
+                const float z = v[i] + bias[c1 + i];
                 Z[(size_t)(c + i) * B + m0 + r] = z;
                 hv[i & 1] = silu(z);
                 if (i & 1) h[i / 2] = pack_bf16(hv[0], hv[1]);
             }
             put_t(H, c, h);
-            spread(cur ^ 1, c, h);
+            put(a_buf(g + 1), c, h);
         }
-        cluster_sync();
-        cur ^= 1;
+        send(a_buf(g + 1), my_slab, 1, 0, SLABS);
+    }
+    // targets of this warp's softmax rows, requested while the output layer runs
+    constexpr int SR = (S::RP + T_THREADS / 32 - 1) / (T_THREADS / 32);   // rows per warp
+    float tgt[SR][4];
+#pragma unroll
+    for (int u = 0; u < SR; ++u) {
+        const int q = warp + u * (T_THREADS / 32);
+        const float *T = a.T + (size_t)(m0 + rank * S::RP + q) * pm.ncls;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) tgt[u][k] = q < S::RP && lane + 32 * k < pm.ncls ? __ldg(T + lane + 32 * k) : 0.f;
     }
     // ---- output layer: logits of row r to the CTA that owns the row, staged
     // in its unused A operand
+    const int cur = a_buf(nl - 2);
     float *logits = reinterpret_cast<float *>(sm + (cur ^ 1) * F_ACT_BYTES);          // [RP][T_LOGIT_LD]
     bf16 *dl = reinterpret_cast<bf16 *>(logits + S::RP * T_LOGIT_LD);                 // [RP][T_DLOG_LD]
     {
         const int g = nl - 2;
-        if (tid == 0 && !bad) product(g, cur);
+        if (tid == 0) product(g);
         const float *b = a.w + pm.b(nl - 1);
+        float bias[CO];
+#pragma unroll
+        for (int i = 0; i < CO; ++i) {
+            const int c = rank * S::NO + grp * CO + i;
+            bias[i] = grp * CO < S::NO && c < pm.ncls ? __ldg(b + c) : 0.f;
+        }
         finish(g);
         const uint32_t row = cluster_addr(umma::saddr(logits + (r % S::RP) * T_LOGIT_LD), r / S::RP);
-        for (int c0 = half * CO; c0 < min(S::NO, half * CO + CO); c0 += 16) {
-            const int c = rank * S::NO + c0;
+#pragma unroll
+        for (int c1 = 0; c1 < CO; c1 += 16) {
+            const int c0 = grp * CO + c1, c = rank * S::NO + c0;
+            if (c0 >= S::NO) break;
             float v[16];
             umma::ld16(trow + (uint32_t)c0, v);
 #pragma unroll
             for (int i = 0; i < 16; ++i)
-                if (c + i < pm.ncls) st_cluster(row + 4u * (c + i), v[i] + b[c + i]);
+                if (c + i < pm.ncls) st_cluster(row + 4u * (c + i), v[i] + bias[c1 + i]);
         }
         cluster_sync();
     }
     // ---- softmax, the row's share of the mean KL loss, and d loss / d logits
     // = (p sum(t) - t) / B as BF16 (zero in the padding columns); one warp per row
-    for (int q = warp; q < S::RP; q += T_THREADS / 32) {
+#pragma unroll
+    for (int u = 0; u < SR; ++u) {
+        const int q = warp + u * (T_THREADS / 32);
+        if (q >= S::RP) break;
         const int ncls = pm.ncls, m = m0 + rank * S::RP + q;
         const float *l = logits + q * T_LOGIT_LD;
-        const float *T = a.T + (size_t)m * ncls;
-        float t[4];
-        float mx = -INFINITY;
+        const float(&t)[4] = tgt[u];
+        float x[4], mx = -INFINITY;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) t[k] = lane + 32 * k < ncls ? T[lane + 32 * k] : 0.f;
-        for (int c = lane; c < ncls; c += 32) mx = fmaxf(mx, l[c]);
+        for (int k = 0; k < 4; ++k) {
+            x[k] = lane + 32 * k < ncls ? l[lane + 32 * k] : -INFINITY;
+            mx = fmaxf(mx, x[k]);
+        }
         for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         float s = 0.f;
-        for (int c = lane; c < ncls; c += 32) s += __expf(l[c] - mx);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            x[k] = __expf(x[k] - mx);
+            if (lane + 32 * k < ncls) s += x[k];
+        }
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         const float inv = 1.0f / s;
         float ts = 0.f, loss = 0.f;
@@ -861,7 +942,7 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
             const int c = lane + 32 * k;
             float d = 0.f;
             if (c < ncls) {
-                const float p = __expf(l[c] - mx) * inv;
+                const float p = x[k] * inv;
                 if (t[k] > 0.f) loss += t[k] * (__logf(t[k]) - __logf(p));
                 d = (p * ts - t[k]) * a.inv_batch;
             }
@@ -873,29 +954,29 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
     __syncthreads();
     for (int e = tid; e < S::RP * 16; e += T_THREADS) {
         const int q = e / 16, k = e % 16 * 8;
-        const uint4 v = *reinterpret_cast<const uint4 *>(&dl[q * T_DLOG_LD + k]);
-        const uint32_t o = act0 + cur * F_ACT_BYTES + act_off(rank * S::RP + q, k);
-#pragma unroll
-        for (int t = 0; t < CS; ++t) st_cluster(cluster_addr(o, t), v);
+        *reinterpret_cast<uint4 *>(sm + cur * F_ACT_BYTES + tact_off(rank * S::RP + q, k)) =
+            *reinterpret_cast<const uint4 *>(&dl[q * T_DLOG_LD + k]);
     }
     bf16 *dZ = a.dZ + (size_t)(nl - 1) * 256 * B;
     for (int e = tid; e < S::RP * 128; e += T_THREADS)
         dZ[(size_t)(e / S::RP) * B + m0 + rank * S::RP + e % S::RP] = dl[e % S::RP * T_DLOG_LD + e / S::RP];
-    cluster_sync();
+    // (every CTA's product of the output layer is complete: the cluster met;
+    // after this no thread reads the stage, which the next layer overwrites)
+    send(cur, rank * S::RP / 8 * F_SBO_B, 2, T_SLAB, S::RP / 8 * F_SBO_B);
     // ---- backward: dZ_{l-1} = (dZ_l W_l) silu'(Z_{l-1})
     for (int l = nl - 1; l >= 1; --l) {
         const int g = 2 * (nl - 1) - l;
-        if (tid == 0 && !bad) product(g, cur);
+        if (tid == 0) product(g);
         const float *Z = a.Z + (size_t)(l - 1) * 256 * B;
         dZ = a.dZ + (size_t)(l - 1) * 256 * B;
         float z[CH];   // requested while the product runs
 #pragma unroll
         for (int i = 0; i < CH; ++i)
-            z[i] = half * CH < S::NS ? Z[(size_t)(rank * S::NS + half * CH + i) * B + m0 + r] : 0.f;
+            z[i] = grp * CH < S::NS ? Z[(size_t)(rank * S::NS + grp * CH + i) * B + m0 + r] : 0.f;
         finish(g);
 #pragma unroll
         for (int c1 = 0; c1 < CH; c1 += 16) {
-            const int c0 = half * CH + c1, c = rank * S::NS + c0;
+            const int c0 = grp * CH + c1, c = rank * S::NS + c0;
             if (c0 >= S::NS) break;
             float v[16];
             umma::ld16(trow + (uint32_t)c0, v);
@@ -904,11 +985,11 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
             for (int i = 0; i < 16; i += 2)
                 h[i / 2] = pack_bf16(v[i] * silu_grad(z[c1 + i]), v[i + 1] * silu_grad(z[c1 + i + 1]));
             put_t(dZ, c, h);
-            if (l > 1) spread(cur ^ 1, c, h);
+            if (l > 1) put(a_buf(g + 1), c, h);
         }
-        cluster_sync();   // after the last layer: no CTA leaves while another may write its shared memory
-        cur ^= 1;
+        if (l > 1) send(a_buf(g + 1), my_slab, 1, 0, SLABS);
     }
+    cluster_sync();   // no CTA leaves while another may read or write its shared memory
     if (bad) {
         // a wait gave up: products may still run; wait (with a limit) before
         // their TMEM is freed, and flag it
