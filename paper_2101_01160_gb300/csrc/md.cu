@@ -1004,18 +1004,15 @@ int launch_persistent(md_system *s, long long nsteps, int force_rebuild, const l
 int ensure_sorted(md_system *s) {
     if (!s->needs_sort) return MD_OK;
     s->needs_sort = false;
-    return launch_persistent(s, 0, RB_NONE);
+    // behind the slab engine without the lists: its next launch builds its own
+    return launch_persistent(s, 0, s->slab_last ? RB_SORT : RB_NONE);
 }
 
 int launch_persistent(md_system *s, long long nsteps, int force_rebuild, const long long *left) {
     s->slab_last = false;
-    if (force_rebuild != RB_ALL) {
-        if (s->needs_sort || !s->lists_valid) force_rebuild = RB_NONE;
-        s->needs_sort = false;
-    } else {
-        s->needs_sort = false;
-    }
-    s->lists_valid = true;
+    if (force_rebuild != RB_ALL && force_rebuild != RB_SORT && (s->needs_sort || !s->lists_valid)) force_rebuild = RB_NONE;
+    s->needs_sort = false;
+    s->lists_valid = force_rebuild != RB_SORT;
     const void *fn = persistent_fn(s->prec, s->block, s->stage);
     long long step0 = s->step;
     int phase = s->phase_half;
@@ -1060,6 +1057,18 @@ int plan_slab(md_system *s) {
     // FP64 shares a particle's pairs among lanes, so small slabs take more warps than particles
     const int lo = s->prec == MD_FP64 ? 256 : 128;
     const int threads = std::min(s->prec == MD_FP64 ? SLAB_THREADS<double> : SLAB_THREADS<float>, std::max(lo, round_up((long long)std::ceil(s->prec == MD_FP64 ? 4.0 * pmax : pmax), 32)));
+    // FP64 is bound by its pipe, so the fullest slab counts (whole rows: up to
+    // twice the mean), and long lists leave the global engine fewer idle lanes.
+    // Microseconds per step of both, fitted to runs from 1,024 to 262,144
+    // particles at phi 0.08 to 0.3 (e.g. 262,144 at 0.08: 44 against 71 us;
+    // 99,856 at 0.2: 57 against 66; 150,000 at 0.3: 139 against 86; 16,384 at
+    // 0.3: 30 against 25).  FP32 slabs were faster at all of them.
+    if (s->prec == MD_FP64) {
+        const long long chunks = (R.n + 255) / 256, waves = (chunks + 2 * s->nsm - 1) / (2 * s->nsm);
+        const double slab = 5.0 + pmax * (0.0091 * cbar - 0.0054);
+        const double global = chunks <= s->nsm ? 9.3 + 1.43 * cbar : waves * (11.5 + 2.9 * cbar);
+        if (slab > global) return MD_OK;
+    }
     SlabDev D{};
     for (double f = 3.0; f > 0.99 && !D.p_cap; f -= 0.05) {
         const int p = (int)std::min<double>(R.n, std::ceil(f * p_want));

@@ -136,9 +136,25 @@ template <> __device__ __forceinline__ double rd<double>(double d, float) { retu
 template <> __device__ __forceinline__ float rd<float>(double, float f) { return f; }
 
 // 1/r^2 of a pair: the hardware reciprocal in FP32 (relative error ~1e-7,
-// far below the force tolerance), IEEE division in FP64.
+// far below the force tolerance); in FP64 the hardware's gross approximation y
+// (relative error e below 2^-19) and one third-order iteration (Householder's
+// method for 1/x), y (1 + e + e^2) with e = 1 - r2 y: 2^-57 before the last
+// rounding.  Three FP64 instructions in place of an IEEE division's eight or
+// more, of some 25 per pair on the pipe that bounds the FP64 force.
 __device__ __forceinline__ float inv_r2(float r2) { return __fdividef(1.0f, r2); }
-__device__ __forceinline__ double inv_r2(double r2) { return 1.0 / r2; }
+__device__ __forceinline__ double inv_r2(double r2) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r2));
+    const double e = __fma_rn(-r2, y, 1.0);
+    return __fma_rn(y, __fma_rn(e, e, e), y);
+}
+
+// r2 < rc2 for a sum of squares: in FP64 as an unsigned compare of the bits
+// (the order of non-negative doubles; a NaN is above all), off the FP64 pipe.
+__device__ __forceinline__ bool within(float r2, float rc2) { return r2 < rc2; }
+__device__ __forceinline__ bool within(double r2, double rc2) {
+    return (unsigned long long)__double_as_longlong(r2) < (unsigned long long)__double_as_longlong(rc2);
+}
 
 // Lennard-Jones sum (Sec. 4: V = 4 eps [(s/r)^12 - (s/r)^6] for r < rc, the
 // force being the derivative of the unshifted potential) over slots [a, e)
@@ -170,7 +186,7 @@ template <typename T, bool kPE>
 __device__ __forceinline__ void lj_pair_acc(T rx, T ry, T rc2, T eps24, T sig2, T &fx, T &fy,
                                             double vshift, double &pe, double &fabs_sum) {
     const T r2 = fmaT(rx, rx, ry * ry);
-    if (r2 < rc2) {
+    if (within(r2, rc2)) {
         T s6;
         const T fr = lj_pair_fr<T>(r2, eps24, sig2, s6);
         fx = fmaT(-fr, rx, fx);
@@ -651,13 +667,14 @@ __device__ __forceinline__ void chunk_lists_sorted(const SysDev &S, int set, con
 // With mode RB_ALL every particle gets its canonical cell (the MD cell its
 // offset now lies in, the offset re-expressed from that cell's corner); with
 // RB_NONE every particle keeps its cell (a sort of a state written in
-// another order).  Then a counting sort of all particles by cell, particles
+// another order), and RB_SORT stops before the lists (a sort for a readout,
+// which walks the cells).  Then a counting sort of all particles by cell, particles
 // inside one cell ordered by id, so the order -- and therefore every force
 // sum -- is reproducible and independent of the launch shape; then the
 // neighbour lists.  Six grid barriers (seven in the global-memory shapes,
 // whose lists other CTAs read next).  Padding slots keep perm = -1 (set at
 // creation).
-enum RebuildMode { RB_ALL = 1, RB_NONE = 2 };
+enum RebuildMode { RB_ALL = 1, RB_NONE = 2, RB_SORT = 4 };
 
 template <typename T, int BLOCK>
 __device__ bool rebuild(const SysDev &S, int &set, int &cur, unsigned &gen, int nloc,
@@ -814,6 +831,13 @@ __device__ bool rebuild(const SysDev &S, int &set, int &cur, unsigned &gen, int 
     if (!grid_sync(bar, gen, S.timeout_ns)) return false;
     set ^= 1;
     cur = 0;
+    if (mode == RB_SORT) {
+        if (blockIdx.x == 0 && tid == 0) {
+            C->n_rebuilds += 1;
+            C->slab_order = 0;
+        }
+        return true;
+    }
     // R7: neighbour lists.  Staged shapes: the chunk windows and lists of
     // the CTA's own chunks in slot order, read only by this CTA, so no
     // barrier follows.  Global-memory shapes: chunks claimed by CTAs, lists

@@ -20,10 +20,10 @@
 // once.
 //
 // Measured per step, against the best global shape (phi 0.0784, T 20): FP32
-// 1,024 particles 6.8 -> 4.5 us, 99,856 10.3 -> 8.8 us, 262,144 16.6 -> 11.1 us;
-// FP64 1,024 14.6 -> 6.6 us, 99,856 42 -> 25 us, 262,144 78 -> 47 us.  Of the
-// 11.1 us of 262,144 FP32 particles the forces take 3.0, the exchange 3.7, halo
-// and drift 2.3, the rebuilds (one in 22 steps) 1.8.
+// 1,024 particles 6.8 -> 4.2 us, 99,856 10.3 -> 8.0 us, 262,144 16.2 -> 9.9 us;
+// FP64 1,024 13.3 -> 6.3 us, 99,856 39 -> 23 us, 262,144 71 -> 44 us.  Of the
+// 9.9 us of 262,144 FP32 particles the forces take 2.9, the exchange 3.3, halo
+// and drift 2.1, the rebuilds (one in 22 steps) 1.6.
 //
 // FP64.  GB300 issues one FP64 warp instruction per 15 clocks and SM, so what
 // counts is how many of its lanes work.  A warp first tests its particles'
@@ -595,7 +595,7 @@ __device__ __forceinline__ void slab_forces(const SysDev &S, const SlabMem<doubl
                 ry = oj.y + __dsub_rn(hy, oi.y);
                 const double r2 = __fma_rn(rx, rx, ry * ry);
                 double s6;
-                if (r2 < P.rc2) fr = lj_pair_fr<double>(r2, P.eps24, P.sig2, s6);
+                if (within(r2, P.rc2)) fr = lj_pair_fr<double>(r2, P.eps24, P.sig2, s6);
             }
             __syncwarp();
             const int n = pos - first_pos;                    // this owner's pairs of the window
