@@ -4,6 +4,7 @@
 // launches (at most (2*MD_MAX_W+1)^2 = 441 classes).
 #include <cstdarg>
 #include <cmath>
+#include <mutex>
 
 #include "common.cuh"
 #include "equilibria.cuh"
@@ -22,6 +23,56 @@ int fail(int code, const char *fmt, ...) {
     va_end(ap);
     g_last_error = buf;
     return code;
+}
+
+// The pool of a device, made on the first call there; after the device's
+// context has changed (a device reset), which its unique id tells, a new one.
+cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t st) {
+    using CtxGetIdFn = int (*)(void *, unsigned long long *);
+    static const CtxGetIdFn ctx_id = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q{};
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            f = nullptr;
+        return reinterpret_cast<CtxGetIdFn>(f);
+    }();
+    constexpr int MAX_DEV = 64;
+    struct Slot {
+        unsigned long long id = 0;
+        cudaMemPool_t pool = nullptr;
+    };
+    static std::mutex mu;
+    static Slot slots[MAX_DEV];
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    unsigned long long id = 0;
+    cudaMemPool_t pool = nullptr;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
+        return cudaMallocAsync(p, bytes, st);   // a graph's allocation node, whose memory the graph keeps
+    if (dev < MAX_DEV && ctx_id && ctx_id(nullptr, &id) == 0) {
+        std::lock_guard<std::mutex> lk(mu);
+        Slot &s = slots[dev];
+        if (!s.pool || s.id != id) {
+            cudaMemPoolProps pr{};
+            pr.allocType = cudaMemAllocationTypePinned;
+            pr.location.type = cudaMemLocationTypeDevice;
+            pr.location.id = dev;
+            uint64_t keep = SCRATCH_KEEP;
+            s.id = id;
+            s.pool = nullptr;
+            if (cudaMemPoolCreate(&s.pool, &pr) != cudaSuccess) s.pool = nullptr;
+            else cudaMemPoolSetAttribute(s.pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        }
+        pool = s.pool;
+    }
+    if (!pool) {   // no such entry point or pool: the default pool
+        cudaGetLastError();
+        return cudaMallocAsync(p, bytes, st);
+    }
+    return cudaMallocFromPoolAsync(p, bytes, pool, st);
 }
 
 __global__ void k_feq_gaussian(double a2, double ux, double uy, int W, double *P) {

@@ -507,9 +507,9 @@ extern "C" int mdlg_bin(const md_snapshot *t0, const md_snapshot *t1, int64_t n,
     if (n <= BIN_CLUSTER_MAX) return bin_launch_cluster(t0, t1, n, lx, W, hist_out, overflow_out, mom_out, st);
     const int grid = bin_grid(t0, t1, n, W);
     double *part = nullptr;
-    MD_CUDA_TRY(cudaMallocAsync((void **)&part, 2 * sizeof(double) * grid, st));
+    MD_CUDA_TRY(scratch_alloc((void **)&part, 2 * sizeof(double) * grid, st));
     rc = bin_launch(t0, t1, n, lx, W, hist_out, overflow_out, mom_out, part, grid, st);
-    cudaError_t e = cudaFreeAsync(part, st);
+    cudaError_t e = scratch_free(part, st);
     if (rc) return rc;
     if (e != cudaSuccess) return fail(MD_E_CUDA, "mdlg_bin: cudaFreeAsync: %s", cudaGetErrorString(e));
     return MD_OK;

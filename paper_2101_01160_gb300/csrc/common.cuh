@@ -36,6 +36,15 @@ int fail(int code, const char *fmt, ...);
                                 #expr, cudaGetErrorString(e_));                   \
     } while (0)
 
+// Stream-ordered scratch of one call (scratch_free on the same stream).  The
+// memory comes from a pool of the library's own per device that keeps up to
+// SCRATCH_KEEP bytes between calls: the device's default pool gives everything
+// back at each synchronisation, and a call that synchronises then pays about
+// 0.1 ms to map its scratch anew.
+constexpr uint64_t SCRATCH_KEEP = 32ull << 20;
+cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t st);
+inline cudaError_t scratch_free(void *p, cudaStream_t st) { return cudaFreeAsync(p, st); }
+
 // Device status word values (a device-side failure sets one, the host reads
 // it at md_sync).
 enum DevStatus : int { DS_OK = 0, DS_TIMEOUT = 1, DS_SKIN = 2, DS_NONFINITE = 4, DS_NBR_OVERFLOW = 8, DS_CAPACITY = 16 };

@@ -621,6 +621,7 @@ struct md_system {
     RepDev *d_reps = nullptr;
     int32_t *d_gran = nullptr;
     Control *d_ctl = nullptr;
+    int *h_status = nullptr;     // pinned: the status word's landing place
     double *d_epart = nullptr;
     double *d_small = nullptr;   // readout scratch (2*nb + 8 doubles, 4 energy)
     long long *d_hist64 = nullptr;
@@ -1150,9 +1151,10 @@ int status_to_code(int ds) {
 }
 
 int sync_status(md_system *s) {
+    // the status word follows the work into pinned memory: one wait
+    MD_CUDA_TRY(cudaMemcpyAsync(s->h_status, &s->d_ctl->status, sizeof(int), cudaMemcpyDeviceToHost, s->st));
     MD_CUDA_TRY(cudaStreamSynchronize(s->st));
-    int ds = 0;
-    MD_CUDA_TRY(cudaMemcpy(&ds, &s->d_ctl->status, sizeof(int), cudaMemcpyDeviceToHost));
+    const int ds = *s->h_status;
     if (ds) {
         MD_CUDA_TRY(cudaMemset(&s->d_ctl->status, 0, sizeof(int)));
         // a wait that gave up leaves the arrival count behind; no kernel of
@@ -1202,7 +1204,7 @@ int upload_state(md_system *s, const double *x, const double *y, const double *v
     if (!x || !y || !vx || !vy) return fail(MD_E_ARG, "state arrays must not be NULL");
     const size_t bytes = sizeof(double) * (size_t)s->ntot;
     double *tmp = nullptr;
-    MD_CUDA_TRY(cudaMallocAsync((void **)&tmp, 4 * bytes, s->st));
+    MD_CUDA_TRY(scratch_alloc((void **)&tmp, 4 * bytes, s->st));
     int rc = MD_OK;
     const double *src[4] = {x, y, vx, vy};
     for (int k = 0; k < 4 && rc == MD_OK; ++k) {
@@ -1224,7 +1226,7 @@ int upload_state(md_system *s, const double *x, const double *y, const double *v
         if (e != cudaSuccess) rc = fail(MD_E_CUDA, "init kernel: %s", cudaGetErrorString(e));
     }
     if (rc == MD_OK) rc = launch_persistent(s, 0, 1);
-    cudaFreeAsync(tmp, s->st);
+    scratch_free(tmp, s->st);
     if (rc) return rc;
     s->phase_half = 0;
     // a state placed on a sampling boundary starts the next window there
@@ -1368,6 +1370,10 @@ int md_init_batch(const md_params *p, int32_t n_rep, const double *x, const doub
     ALLOC(s->d_hist64, sizeof(long long) * s->nb);
     ALLOC(s->d_nc_of_id, sizeof(int32_t) * s->ntot);
 #undef ALLOC
+    if (rc == MD_OK && cudaMallocHost((void **)&s->h_status, sizeof(int)) != cudaSuccess) {
+        s->h_status = nullptr;
+        rc = fail(MD_E_NOMEM, "md_init_batch: pinned memory");
+    }
     if (rc) {
         md_destroy(s);
         return rc;
@@ -1463,6 +1469,7 @@ void md_destroy(md_system *s) {
     if (s->st) cudaStreamSynchronize(s->st);
     free_resident(s);
     for (void *p : s->allocs) cudaFree(p);
+    if (s->h_status) cudaFreeHost(s->h_status);
     delete s;
 }
 
@@ -1645,7 +1652,7 @@ int md_get_state(md_system *s, double *x, double *y, double *vx, double *vy) {
     if (!s || !x || !y || !vx || !vy) return fail(MD_E_ARG, "md_get_state: NULL argument");
     const size_t bytes = sizeof(double) * s->ntot;
     double *tmp = nullptr;
-    MD_CUDA_TRY(cudaMallocAsync((void **)&tmp, 4 * bytes, s->st));
+    MD_CUDA_TRY(scratch_alloc((void **)&tmp, 4 * bytes, s->st));
     ObsArgs a{};
     a.x = tmp;
     a.y = tmp + s->ntot;
@@ -1657,7 +1664,7 @@ int md_get_state(md_system *s, double *x, double *y, double *vx, double *vy) {
         cudaError_t e = cudaMemcpyAsync(dst[k], tmp + k * s->ntot, bytes, cudaMemcpyDefault, s->st);
         if (e != cudaSuccess) rc = fail(MD_E_CUDA, "md_get_state: %s", cudaGetErrorString(e));
     }
-    cudaFreeAsync(tmp, s->st);
+    scratch_free(tmp, s->st);
     if (rc) return rc;
     return sync_status(s);
 }
@@ -1694,7 +1701,7 @@ int md_forces(md_system *s, double *fx, double *fy, double *fabs_sum) {
     if (!s || !fx || !fy) return fail(MD_E_ARG, "md_forces: NULL argument");
     const size_t bytes = sizeof(double) * s->ntot;
     double *tmp = nullptr;
-    MD_CUDA_TRY(cudaMallocAsync((void **)&tmp, 3 * bytes, s->st));
+    MD_CUDA_TRY(scratch_alloc((void **)&tmp, 3 * bytes, s->st));
     ObsArgs a{};
     a.fx = tmp;
     a.fy = tmp + s->ntot;
@@ -1706,7 +1713,7 @@ int md_forces(md_system *s, double *fx, double *fy, double *fabs_sum) {
         cudaError_t e = cudaMemcpyAsync(dst[k], tmp + k * s->ntot, bytes, cudaMemcpyDefault, s->st);
         if (e != cudaSuccess) rc = fail(MD_E_CUDA, "md_forces: %s", cudaGetErrorString(e));
     }
-    cudaFreeAsync(tmp, s->st);
+    scratch_free(tmp, s->st);
     if (rc) return rc;
     return sync_status(s);
 }
@@ -1716,7 +1723,7 @@ int md_step_forces(md_system *s, int64_t nsteps, double *fx, double *fy) {
     if (!s || nsteps < 1 || !fx || !fy) return fail(MD_E_ARG, "md_step_forces: bad arguments");
     const size_t bytes = sizeof(double) * s->ntot;
     double *tmp = nullptr;
-    MD_CUDA_TRY(cudaMallocAsync((void **)&tmp, 2 * bytes, s->st));
+    MD_CUDA_TRY(scratch_alloc((void **)&tmp, 2 * bytes, s->st));
     s->sd.dbg_fx = tmp;
     s->sd.dbg_fy = tmp + s->ntot;
     int rc = md_step(s, nsteps);
@@ -1726,7 +1733,7 @@ int md_step_forces(md_system *s, int64_t nsteps, double *fx, double *fy) {
         cudaError_t e = cudaMemcpyAsync(dst[k], tmp + k * s->ntot, bytes, cudaMemcpyDefault, s->st);
         if (e != cudaSuccess) rc = fail(MD_E_CUDA, "md_step_forces: %s", cudaGetErrorString(e));
     }
-    cudaFreeAsync(tmp, s->st);
+    scratch_free(tmp, s->st);
     if (rc) return rc;
     return sync_status(s);
 }
@@ -1756,12 +1763,12 @@ int md_energy_batch(md_system *s, double *out) {
     const bool dev = cudaPointerGetAttributes(&at, out) == cudaSuccess && at.type == cudaMemoryTypeDevice;
     cudaGetLastError();
     double *dst = out;
-    if (!dev) MD_CUDA_TRY(cudaMallocAsync((void **)&dst, bytes, s->st));
+    if (!dev) MD_CUDA_TRY(scratch_alloc((void **)&dst, bytes, s->st));
     k_sum_energy_batch<<<s->nrep, 256, 0, s->st>>>(s->d_epart, s->d_reps, dst);
     cudaError_t e = cudaGetLastError();
     if (!dev) {
         if (e == cudaSuccess) e = cudaMemcpyAsync(out, dst, bytes, cudaMemcpyDeviceToHost, s->st);
-        cudaFreeAsync(dst, s->st);
+        scratch_free(dst, s->st);
     }
     if (e != cudaSuccess) return fail(MD_E_CUDA, "md_energy_batch: %s", cudaGetErrorString(e));
     return sync_status(s);
@@ -1873,7 +1880,7 @@ int feq_bootstrap(md_system *s, int32_t lg, int32_t dxi, int32_t symmetrize, int
     const bool dev = cudaPointerGetAttributes(&at, sigma_out) == cudaSuccess && at.type == cudaMemoryTypeDevice;
     cudaGetLastError();
     double *dst = sigma_out;
-    if (!dev) MD_CUDA_TRY(cudaMallocAsync((void **)&dst, bytes, s->st));
+    if (!dev) MD_CUDA_TRY(scratch_alloc((void **)&dst, bytes, s->st));
     A.sigma = dst;
     const int ncls = boot_classes(s->W, A.sym);
     const int keep = boot_p_bytes(A.B, ncls) <= BOOT_KEEP_BYTES;
@@ -1887,7 +1894,7 @@ int feq_bootstrap(md_system *s, int32_t lg, int32_t dxi, int32_t symmetrize, int
     }
     if (!dev) {
         if (e == cudaSuccess) e = cudaMemcpyAsync(sigma_out, dst, bytes, cudaMemcpyDeviceToHost, s->st);
-        cudaFreeAsync(dst, s->st);
+        scratch_free(dst, s->st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
     }
     if (e != cudaSuccess) return fail(MD_E_CUDA, "feq_bootstrap: %s", cudaGetErrorString(e));
@@ -1916,13 +1923,13 @@ int feq_batch(md_system *s, int32_t lg, int32_t dxi, int32_t symmetrize, double 
     const bool dev = cudaPointerGetAttributes(&at, out) == cudaSuccess && at.type == cudaMemoryTypeDevice;
     cudaGetLastError();
     double *dst = out;
-    if (!dev) MD_CUDA_TRY(cudaMallocAsync((void **)&dst, bytes, s->st));
+    if (!dev) MD_CUDA_TRY(scratch_alloc((void **)&dst, bytes, s->st));
     A.out = dst;
     k_feq_batch<<<s->nrep, FEQB_THREADS, 0, s->st>>>(A);
     cudaError_t e = cudaGetLastError();
     if (!dev) {
         if (e == cudaSuccess) e = cudaMemcpyAsync(out, dst, bytes, cudaMemcpyDeviceToHost, s->st);
-        cudaFreeAsync(dst, s->st);
+        scratch_free(dst, s->st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
     }
     if (e != cudaSuccess) return fail(MD_E_CUDA, "feq_batch: %s", cudaGetErrorString(e));

@@ -156,18 +156,19 @@ def _stream(stream=None):
     import torch
 
     s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    return s.cuda_stream
 
 
 def _ptr(a):
-    """Device pointer of a torch tensor, or host pointer of a numpy array."""
+    """Device pointer of a torch tensor, or host pointer of a numpy array, as
+    an integer (what the c_void_p arguments take fastest)."""
     if a is None:
         return None
     if isinstance(a, np.ndarray):
         assert a.flags.c_contiguous
-        return C.c_void_p(a.ctypes.data)
+        return a.ctypes.data
     assert a.is_contiguous()
-    return C.c_void_p(a.data_ptr())
+    return a.data_ptr()
 
 
 def make_params(n, L, dt=5e-4, rc=2.5, eps=1.0, sigma=1.0, mass=1.0, skin=0.5,
@@ -395,20 +396,25 @@ def _snapshots(cell0, ox0, oy0, cell1, ox1, oy1, ncell, h):
     import torch
 
     arrs = (cell0, ox0, oy0, cell1, ox1, oy1)
-    if not all(isinstance(a, torch.Tensor) for a in arrs):
-        raise ValueError("snapshot arrays must be torch tensors")
+    for a in arrs:
+        if not isinstance(a, torch.Tensor):
+            raise ValueError("snapshot arrays must be torch tensors")
     n = cell0.numel()
-    if any(a.dim() != 1 or a.numel() != n or not a.is_contiguous() for a in arrs):
-        raise ValueError("snapshot arrays must be contiguous 1-D tensors of one length")
+    for a in arrs:
+        if a.dim() != 1 or a.numel() != n or not a.is_contiguous():
+            raise ValueError("snapshot arrays must be contiguous 1-D tensors of one length")
     if cell0.dtype != torch.int32 or cell1.dtype != torch.int32:
         raise ValueError("snapshot cells must be int32")
-    if ox0.dtype not in (torch.float32, torch.float64) or any(a.dtype != ox0.dtype for a in (oy0, ox1, oy1)):
+    ft = ox0.dtype
+    f64 = ft == torch.float64
+    if not (f64 or ft == torch.float32) or oy0.dtype != ft or ox1.dtype != ft or oy1.dtype != ft:
         raise ValueError("snapshot offsets must all be float32 or all float64")
-    if any(a.device.type != "cuda" for a in arrs) or len({a.device for a in arrs}) != 1:
+    dev = cell0.device
+    if not cell0.is_cuda or any(a.device != dev for a in arrs[1:]):
         raise ValueError("snapshot arrays must be on one CUDA device")
-    f64 = int(ox0.dtype == torch.float64)
-    s0 = md_snapshot(_ptr(cell0).value, _ptr(ox0).value, _ptr(oy0).value, f64, int(ncell), float(h))
-    s1 = md_snapshot(_ptr(cell1).value, _ptr(ox1).value, _ptr(oy1).value, f64, int(ncell), float(h))
+    ncell, h = int(ncell), float(h)
+    s0 = md_snapshot(cell0.data_ptr(), ox0.data_ptr(), oy0.data_ptr(), f64, ncell, h)
+    s1 = md_snapshot(cell1.data_ptr(), ox1.data_ptr(), oy1.data_ptr(), f64, ncell, h)
     return s0, s1, n
 
 
