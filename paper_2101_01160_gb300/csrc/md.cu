@@ -1024,13 +1024,34 @@ int launch_persistent(md_system *s, long long nsteps, int force_rebuild, const l
 }
 
 // ---- slab engine ------------------------------------------------------------
-const void *slab_fn(int prec) {
-    return prec == MD_FP64 ? (const void *)k_md_slab<double> : (const void *)k_md_slab<float>;
+const void *slab_fn(int prec, bool cluster) {
+    if (prec == MD_FP64) return (const void *)k_md_slab<double, false>;
+    return cluster ? (const void *)k_md_slab<float, true> : (const void *)k_md_slab<float, false>;
 }
-SlabLayout slab_layout_of(const md_system *s, int p_cap, int h_cap, int e_cap, int ncells, int threads) {
+SlabLayout slab_layout_of(const md_system *s, int p_cap, int h_cap, int e_cap, int ncells) {
     const size_t hb = smem_hist_bytes(s->n_lg, s->n_dx, s->nb);
-    return s->prec == MD_FP64 ? slab_layout<double>(hb, p_cap, h_cap, e_cap, ncells, threads)
-                              : slab_layout<float>(hb, p_cap, h_cap, e_cap, ncells, threads);
+    return s->prec == MD_FP64 ? slab_layout<double>(hb, p_cap, h_cap, e_cap, ncells)
+                              : slab_layout<float>(hb, p_cap, h_cap, e_cap, ncells);
+}
+
+// One cooperative launch (every CTA resident), or one cluster.
+cudaLaunchConfig_t slab_config(md_system *s, cudaLaunchAttribute *at) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(s->sl.g);
+    cfg.blockDim = dim3(s->sl.threads);
+    cfg.dynamicSmemBytes = s->slab_smem;
+    cfg.stream = s->st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (s->sl.cluster) {
+        at->id = cudaLaunchAttributeClusterDimension;
+        at->val.clusterDim.x = s->sl.g;
+        at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    } else {
+        at->id = cudaLaunchAttributeCooperative;
+        at->val.cooperative = 1;
+    }
+    return cfg;
 }
 
 // Plans the slabs of a single replica: as many as SMs, of at least two cell
@@ -1040,16 +1061,29 @@ SlabLayout slab_layout_of(const md_system *s, int p_cap, int h_cap, int e_cap, i
 // 1.1 times a row's, plus five standard deviations of a Poisson count; lists
 // 1.25 times the mean neighbour count plus 2 per particle).  No plan where
 // that does not fit, e.g. more than about 4,000 FP32 particles per SM.
-int plan_slab(md_system *s) {
+int plan_slab(md_system *s, bool may_cluster = true) {
     if (s->nrep != 1) return MD_OK;
     const RepDev &R = s->reps[0];
+    int g = std::min(std::min(s->nsm, s->prec == MD_FP64 ? R.nc : R.nc / 2), R.cap / 32);
+    if (g < 2) g = 1;
+    // A cluster's exchange is shorter but leaves 16 SMs.  In FP32 it pays to
+    // about 500 particles a slab (us/step, cluster against grid: 1,024
+    // particles 3.2/4.3, 4,096 3.7/4.8, 2,000 at phi 0.3 4.4/5.4, 8,000
+    // 5.2/5.3, 16,384 8.2/5.7).  In FP64 the pairs want every SM's pipe
+    // (1,024 6.3/6.4, 2,048 7.7/6.7, 4,096 10.1/7.1): never.
+    bool cluster = false;
+    if (may_cluster && g > 1 && s->prec != MD_FP64) {
+        const int gc = std::min(g, SLAB_CLUSTER);
+        const double pc = (double)R.n * ((R.nc + gc - 1) / gc) / R.nc;
+        cluster = pc <= 512.0;
+        if (cluster) g = gc;
+    }
+    const void *fn = slab_fn(s->prec, cluster);
     int optin = 0;
     MD_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, s->dev));
     cudaFuncAttributes fa{};
-    MD_CUDA_TRY(cudaFuncGetAttributes(&fa, slab_fn(s->prec)));
+    MD_CUDA_TRY(cudaFuncGetAttributes(&fa, fn));
     const size_t smem = (size_t)optin - fa.sharedSizeBytes;
-    int g = std::min(std::min(s->nsm, s->prec == MD_FP64 ? R.nc : R.nc / 2), R.cap / 32);
-    if (g < 2) g = 1;
     const int rows = (R.nc + g - 1) / g, ncells = (g == 1 ? R.nc : rows + 2) * R.nc;
     const double pmax = (double)R.n * rows / R.nc, row = (double)R.n / R.nc;
     const double cbar = M_PI * R.rv2 * (double)R.n / (R.L * R.L);
@@ -1057,7 +1091,11 @@ int plan_slab(md_system *s) {
     const double h_want = g == 1 ? 0.0 : 1.1 * row + 5.0 * std::sqrt(row) + 32.0;
     // FP64 shares a particle's pairs among lanes, so small slabs take more warps than particles
     const int lo = s->prec == MD_FP64 ? 256 : 128;
-    const int threads = std::min(s->prec == MD_FP64 ? SLAB_THREADS<double> : SLAB_THREADS<float>, std::max(lo, round_up((long long)std::ceil(s->prec == MD_FP64 ? 4.0 * pmax : pmax), 32)));
+    const int hi = s->prec == MD_FP64 ? SLAB_THREADS<double, false>
+                                      : (cluster ? SLAB_THREADS<float, true> : SLAB_THREADS<float, false>);
+    // FP32: one particle per thread also where a slab holds more than its mean
+    const double want = std::ceil(s->prec == MD_FP64 ? 4.0 * pmax : pmax + 3.0 * std::sqrt(pmax));
+    const int threads = std::min(hi, std::max(lo, round_up((long long)want, 32)));
     // FP64 is bound by its pipe, so the fullest slab counts (whole rows: up to
     // twice the mean), and long lists leave the global engine fewer idle lanes.
     // Microseconds per step of both, fitted to runs from 1,024 to 262,144
@@ -1076,7 +1114,7 @@ int plan_slab(md_system *s) {
         const int h = (int)std::min<double>(R.n, std::ceil(f * h_want));
         const double e = std::ceil(p * (1.25 * cbar + 2.0)) + 256.0;
         if (p + 2 * h >= SLAB_MAX_IDX || e > 1e6) continue;
-        if (slab_layout_of(s, p, h, (int)e, ncells, threads).end > smem) continue;
+        if (slab_layout_of(s, p, h, (int)e, ncells).end > smem) continue;
         D.p_cap = p;
         D.h_cap = std::max(h, 1);
         D.e_cap = (int)e;
@@ -1101,11 +1139,20 @@ int plan_slab(md_system *s) {
     A((void **)&D.slab_n, sizeof(int32_t) * g);
     A((void **)&D.left, sizeof(long long));
     if (rc) return rc;
-    s->slab_smem = slab_layout_of(s, D.p_cap, D.h_cap, D.e_cap, ncells, threads).end;
-    MD_CUDA_TRY(cudaFuncSetAttribute(slab_fn(s->prec), cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes));
+    s->slab_smem = slab_layout_of(s, D.p_cap, D.h_cap, D.e_cap, ncells).end;
+    MD_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes));
     int occ = 0;
-    MD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, slab_fn(s->prec), threads, s->slab_smem));
+    MD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, s->slab_smem));
+    D.cluster = cluster;
     s->sl = D;
+    if (cluster) {
+        MD_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        cudaLaunchAttribute at{};
+        cudaLaunchConfig_t cfg = slab_config(s, &at);
+        int nclu = 0;
+        MD_CUDA_TRY(cudaOccupancyMaxActiveClusters(&nclu, fn, &cfg));
+        if (nclu < 1) return plan_slab(s, false);
+    }
     s->slab_ok = occ >= 1;
     return MD_OK;
 }
@@ -1119,9 +1166,11 @@ int launch_slab(md_system *s, long long nsteps) {
     long long step0 = s->step;
     int phase = s->phase_half;
     void *args[] = {&s->sd, &s->sl, &step0, &nsteps, &phase};
-    MD_CUDA_TRY(cudaMemsetAsync(s->sl.word, 0, sizeof(unsigned long long) * 2 * s->sl.g * s->sl.g, s->st));
-    MD_CUDA_TRY(cudaLaunchCooperativeKernel(slab_fn(s->prec), dim3(s->sl.g), dim3(s->sl.threads), args, s->slab_smem,
-                                            s->st));
+    if (!s->sl.cluster)
+        MD_CUDA_TRY(cudaMemsetAsync(s->sl.word, 0, sizeof(unsigned long long) * 2 * s->sl.g * s->sl.g, s->st));
+    cudaLaunchAttribute at{};
+    const cudaLaunchConfig_t cfg = slab_config(s, &at);
+    MD_CUDA_TRY(cudaLaunchKernelExC(&cfg, slab_fn(s->prec, s->sl.cluster), args));
     int rc = launch_persistent(s, nsteps, RB_NONE, s->sl.left);
     if (rc) return rc;
     s->needs_sort = true;

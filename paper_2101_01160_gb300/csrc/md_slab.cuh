@@ -15,12 +15,15 @@
 //     no atomic is serialised, and a CTA polls only lines that nobody else
 //     reads (slab_sync; 152 CTAs polling one word per CTA took 6 us, this takes
 //     3.5 us with the imbalance of the slabs).
+// A small FP32 replica's slabs are one thread-block cluster (at most 16 CTAs):
+// the exchange is then stores into the CTAs' shared memory and a cluster
+// barrier, 1,860 clocks a step against 3,140 (1,024 particles, 16 slabs/32).
 // A step has two phases: forces and kick (velocities are private to their
 // particle), then, after a CTA barrier, drift in place, so offsets are held
 // once.
 //
 // Measured per step, against the best global shape (phi 0.0784, T 20): FP32
-// 1,024 particles 6.8 -> 4.2 us, 99,856 10.3 -> 8.0 us, 262,144 16.2 -> 9.9 us;
+// 1,024 particles 6.8 -> 3.2 us, 99,856 10.3 -> 8.0 us, 262,144 16.2 -> 9.9 us;
 // FP64 1,024 13.3 -> 6.3 us, 99,856 39 -> 23 us, 262,144 71 -> 44 us.  Of the
 // 9.9 us of 262,144 FP32 particles the forces take 2.9, the exchange 3.3, halo
 // and drift 2.1, the rebuilds (one in 22 steps) 1.6.
@@ -52,9 +55,13 @@
 
 namespace mdlg {
 
-constexpr int SLAB_MAX_THREADS = 1024;
-// FP64 is bound by its pipe, which 16 warps keep busy with twice the registers
-template <typename T> constexpr int SLAB_THREADS = sizeof(T) == 8 ? 512 : 1024;
+constexpr int SLAB_MAX_THREADS = 768;
+// FP64 is bound by its pipe, which 16 warps keep busy with twice the registers,
+// and a cluster's CTAs hold a few hundred particles.  The FP32 grid's step does
+// not spill at 768 threads (80 registers); at 1,024 (64) it did: 262,144
+// particles 13.3 -> 13.1 us, 16,384 at phi 0.3 7.4 -> 6.6 us.
+template <typename T, bool CL> constexpr int SLAB_THREADS = sizeof(T) == 8 || CL ? 512 : 768;
+constexpr int SLAB_CLUSTER = 16;        // most CTAs of a cluster
 constexpr int SLAB_MAX_IDX = 1 << 14;   // list entries: 14-bit index, 2-bit column tag
 
 struct SlabDev {
@@ -67,17 +74,17 @@ struct SlabDev {
     int32_t *mig_n;             // [g][2]
     int32_t *slab_n;            // [g]: particles of each slab in the state written back
     long long *left;            // steps that the launch leaves to the global engine
-    int32_t g, p_cap, h_cap, e_cap, ncells, threads;   // ncells: MD cells of the largest slab with its halo rows
+    int32_t g, p_cap, h_cap, e_cap, ncells, threads, cluster;   // ncells: MD cells of the largest slab with its halo rows
 };
 
 // Byte offsets of a slab's arrays in dynamic shared memory (after the
 // histograms).  Own particles: indices [0, p_cap); halo: [p_cap, p_cap + 2
 // h_cap), the upper neighbour's first row, then the lower one's last.
 struct SlabLayout {
-    uint32_t off, foff, vel, cell, id, lst, rend, bpos, mem, ccs, pair, ent, end;   // ccs: ncells + 1
+    uint32_t off, foff, vel, cell, id, lst, rend, bpos, mem, ccs, ent, end;   // ccs: ncells + 1
 };
 template <typename T>
-__host__ __device__ inline SlabLayout slab_layout(size_t base, int p_cap, int h_cap, int e_cap, int ncells, int threads) {
+__host__ __device__ inline SlabLayout slab_layout(size_t base, int p_cap, int h_cap, int e_cap, int ncells) {
     SlabLayout L;
     const size_t ph = (size_t)p_cap + 2 * (size_t)h_cap;
     size_t p = base;
@@ -96,7 +103,6 @@ __host__ __device__ inline SlabLayout slab_layout(size_t base, int p_cap, int h_
     L.bpos = take((size_t)p_cap * sizeof(uint16_t));
     L.mem = take(ph * sizeof(uint16_t));
     L.ccs = take(((size_t)ncells + 1) * sizeof(int32_t));
-    L.pair = sizeof(T) == 8 ? take((size_t)threads * sizeof(uint32_t)) : (uint32_t)p;   // one pair per lane
     L.ent = take((size_t)e_cap * sizeof(uint16_t));
     L.end = (uint32_t)p;
     return L;
@@ -115,7 +121,6 @@ template <typename T> struct SlabMem {
     __device__ __forceinline__ uint16_t *bpos() const { return reinterpret_cast<uint16_t *>(res_smem + L.bpos); }
     __device__ __forceinline__ uint16_t *mem() const { return reinterpret_cast<uint16_t *>(res_smem + L.mem); }
     __device__ __forceinline__ int32_t *ccs() const { return reinterpret_cast<int32_t *>(res_smem + L.ccs); }
-    __device__ __forceinline__ uint32_t *pair() const { return reinterpret_cast<uint32_t *>(res_smem + L.pair); }
     __device__ __forceinline__ uint16_t *ent() const { return reinterpret_cast<uint16_t *>(res_smem + L.ent); }
     // sets the offset of particle j (own or halo) and its float copy
     __device__ __forceinline__ void put_off(int j, V o) const {
@@ -130,6 +135,7 @@ struct SlabCta {
     int last;                     // published row of the lower neighbour that is its last: 1, or 0 if it has one row
     int p, nh[2], par;            // own particles, halo particles, parity of the published offsets
     unsigned seq;                 // exchanges done
+    unsigned *box;                // cluster: the others' payloads, [2][SLAB_CLUSTER] in shared memory
 };
 
 __device__ __forceinline__ unsigned long long ld_acquire_gpu64(const unsigned long long *p) {
@@ -153,10 +159,31 @@ __device__ __forceinline__ unsigned long long *slab_mail(const SlabDev &D, const
 // which a CTA posts after reading its mailbox of this one.  The wait is
 // bounded (S.timeout_ns): a CTA that waits longer flags DS_TIMEOUT, and every
 // CTA leaves the kernel at its next exchange (ok = false).
+template <bool CL>
 __device__ __forceinline__ unsigned slab_sync(const SysDev &S, const SlabDev &D, SlabCta &X, unsigned payload,
                                               bool &ok) {
     __shared__ unsigned s_wmax[SLAB_MAX_THREADS / 32], s_pay;
     __shared__ int s_fail;
+    if constexpr (CL) {
+        // one 32-bit word per sender in every CTA's shared memory, by parity
+        // of the exchange; the barrier releases and acquires for the cluster
+        const unsigned par = ++X.seq & 1u;
+        if (threadIdx.x == 0) s_pay = payload;
+        __syncthreads();
+        if ((int)threadIdx.x < X.g) {
+            uint32_t at;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                         : "=r"(at)
+                         : "r"(smem_u32(&X.box[par * SLAB_CLUSTER + X.k])), "r"(threadIdx.x));
+            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(at), "r"(s_pay) : "memory");
+        }
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        unsigned r = 0;
+        for (int j = 0; j < X.g; ++j) r = max(r, X.box[par * SLAB_CLUSTER + j]);
+        ok = true;
+        return r;
+    }
     const int tid = threadIdx.x;
     const unsigned seq = ++X.seq;
     unsigned long long *w = slab_mail(D, X);
@@ -206,9 +233,14 @@ __device__ __forceinline__ unsigned slab_sync(const SysDev &S, const SlabDev &D,
 
 // Sum of `own` over the CTAs before this one, from the words of the last
 // exchange (whose payloads were the CTAs' own values).
+template <bool CL>
 __device__ __forceinline__ int slab_before(const SlabDev &D, const SlabCta &X) {
-    const unsigned long long *w = slab_mail(D, X);
     int o = 0;
+    if constexpr (CL) {
+        for (int j = 0; j < X.k; ++j) o += (int)X.box[(X.seq & 1u) * SLAB_CLUSTER + j];
+        return o;
+    }
+    const unsigned long long *w = slab_mail(D, X);
     for (int j = 0; j < X.k; ++j) o += (int)(unsigned)ld_acquire_gpu64(&w[j]);
     return o;
 }
@@ -528,6 +560,25 @@ __device__ __forceinline__ void slab_forces(const SysDev &S, const SlabMem<float
     }
 }
 
+// The k-th (from 0) set bit of m1:m0; past the last, entries from 64 on.
+__device__ __forceinline__ uint32_t slab_kth(uint32_t m0, uint32_t m1, uint32_t k) {
+    const uint32_t n0 = __popc(m0), n = n0 + __popc(m1);
+    if (k >= n) return 64u + k - n;
+    const bool up = k >= n0;
+    uint32_t w = up ? m1 : m0, at = up ? 32u : 0u;
+    if (up) k -= n0;
+#pragma unroll
+    for (int step = 16; step; step >>= 1) {
+        const uint32_t c = __popc(w & ((1u << step) - 1u));
+        if (k >= c) {
+            k -= c;
+            w >>= step;
+            at += step;
+        }
+    }
+    return at;
+}
+
 // FP64: per warp up to 32 owners (fewer in a small slab, so that all warps
 // share the work); pairs 32 at a time over the warp's lanes.
 __device__ __forceinline__ void slab_forces(const SysDev &S, const SlabMem<double> &M, const SlabCta &X,
@@ -536,7 +587,6 @@ __device__ __forceinline__ void slab_forces(const SysDev &S, const SlabMem<doubl
     const float2 *fo = M.foff();
     const uint16_t *ent = M.ent();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    uint32_t *buf = M.pair() + warp * 32;
     const int pw = X.p <= 8 * nw ? 8 : (X.p <= 16 * nw ? 16 : 32);
     const float hf = (float)P.h;
     for (int base = warp * pw; base < X.p; base += nw * pw) {
@@ -551,12 +601,20 @@ __device__ __forceinline__ void slab_forces(const SysDev &S, const SlabMem<doubl
             const uint32_t re = M.rend()[i];
             r1 = re & 0xffu;
             r2 = re >> 8;
-            for (uint32_t e = 0; e < min(len, 64u); ++e) {
-                const uint32_t v = ent[st + e];
-                const float2 o = fo[v & RES_IDX];
-                const float kx = (float)((int)(v >> 14) - 1), ky = e < r1 ? -1.0f : (e < r2 ? 0.0f : 1.0f);
-                const float rx = o.x + __fmaf_rn(kx, hf, -oi.x), ry = o.y + __fmaf_rn(ky, hf, -oi.y);
-                if (rx * rx + ry * ry < P.rc2f) mask |= 1ull << e;
+            for (uint32_t e0 = 0; e0 < min(len, 64u); e0 += 4) {   // four entries' loads at a time
+                uint32_t v[4];
+                float2 o[4];
+#pragma unroll
+                for (uint32_t u = 0; u < 4; ++u) v[u] = ent[st + min(e0 + u, len - 1)];
+#pragma unroll
+                for (uint32_t u = 0; u < 4; ++u) o[u] = fo[v[u] & RES_IDX];
+#pragma unroll
+                for (uint32_t u = 0; u < 4; ++u) {
+                    const uint32_t e = e0 + u, row = (e >= r1) + (e >= r2);
+                    const float rx = o[u].x + __fmaf_rn((float)((int)(v[u] >> 14) - 1), hf, -oi.x);
+                    const float ry = o[u].y + __fmaf_rn((float)((int)row - 1), hf, -oi.y);
+                    if (e < len && rx * rx + ry * ry < P.rc2f) mask |= 1ull << e;
+                }
             }
         }
         const uint32_t more = len > 64u ? len - 64u : 0u;
@@ -567,29 +625,28 @@ __device__ __forceinline__ void slab_forces(const SysDev &S, const SlabMem<doubl
             if (lane >= o) incl += t;
         }
         const int total = __shfl_sync(0xffffffffu, incl, 31);
-        int pos = incl - cnt;          // this owner's next pair
-        uint32_t tail = 64;            // next entry past the mask
+        const int excl = incl - cnt;
         double fx = 0.0, fy = 0.0;
         for (int c0 = 0; c0 < total; c0 += 32) {
-            const int first_pos = pos;
-            while (pos < incl && pos < c0 + 32) {
-                uint32_t e;
-                if (mask) {
-                    e = (uint32_t)__ffsll((long long)mask) - 1u;
-                    mask &= mask - 1ull;
-                } else {
-                    e = tail++;
-                }
-                const uint32_t row = e < r1 ? 0u : (e < r2 ? 1u : 2u);
-                buf[pos - c0] = (uint32_t)ent[st + e] | row << 16 | (uint32_t)lane << 18;
-                ++pos;
-            }
-            __syncwarp();
+            // this lane's pair: its owner by bisection of the running counts,
+            // its entry as the owner's k-th surviving one.  (Owners writing
+            // their pairs into a window took 14,470 clocks a step in a dense
+            // system, 2,000 particles at phi 0.3: one lane at a time; this way the
+            // whole step went from 16.2 to 14.7 us.)
+            const int q = c0 + lane;
+            int o = 0;
+#pragma unroll
+            for (int step = 16; step; step >>= 1)
+                if (__shfl_sync(0xffffffffu, incl, o + step - 1) <= q) o += step;
+            const uint32_t k = (uint32_t)(q - __shfl_sync(0xffffffffu, excl, o));
+            const uint32_t m0 = __shfl_sync(0xffffffffu, (uint32_t)mask, o);
+            const uint32_t m1 = __shfl_sync(0xffffffffu, (uint32_t)(mask >> 32), o);
+            const uint32_t est = __shfl_sync(0xffffffffu, st, o), rows = __shfl_sync(0xffffffffu, r1 | r2 << 8, o);
             double fr = 0.0, rx = 0.0, ry = 0.0;
-            if (c0 + lane < total) {
-                const uint32_t v = buf[lane];
-                const double2 oi = off[base + (int)(v >> 18)], oj = off[v & RES_IDX];
-                const uint32_t tx = (v >> 14) & 3u, ty = (v >> 16) & 3u;
+            if (q < total) {
+                const uint32_t e = slab_kth(m0, m1, k), v = ent[est + e];
+                const double2 oi = off[base + o], oj = off[v & RES_IDX];
+                const uint32_t tx = v >> 14, ty = (e >= (rows & 0xffu)) + (e >= rows >> 8);
                 const double hx = tx == 0 ? -P.h : (tx == 1 ? 0.0 : P.h), hy = ty == 0 ? -P.h : (ty == 1 ? 0.0 : P.h);
                 rx = oj.x + __dsub_rn(hx, oi.x);
                 ry = oj.y + __dsub_rn(hy, oi.y);
@@ -597,9 +654,8 @@ __device__ __forceinline__ void slab_forces(const SysDev &S, const SlabMem<doubl
                 double s6;
                 if (within(r2, P.rc2)) fr = lj_pair_fr<double>(r2, P.eps24, P.sig2, s6);
             }
-            __syncwarp();
-            const int n = pos - first_pos;                    // this owner's pairs of the window
-            const int nmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)n);
+            const int first_pos = max(excl, c0), n = min(incl, c0 + 32) - first_pos;   // this owner's pairs here
+            const int nmax = __reduce_max_sync(0xffffffffu, n);
             for (int k = 0; k < nmax; ++k) {
                 const int src = first_pos - c0 + k;           // taken modulo 32 by the shuffle
                 const double f = __shfl_sync(0xffffffffu, fr, src), x = __shfl_sync(0xffffffffu, rx, src),
@@ -633,9 +689,9 @@ __device__ __forceinline__ void dd_add(DD &a, double hi, double lo) {
 }
 
 // ---------------------------------------------------------------- kernel
-template <typename T>
-__global__ void __launch_bounds__(SLAB_THREADS<T>, 1) k_md_slab(SysDev S, SlabDev D, long long step0, long long nsteps,
-                                                                int phase_half) {
+template <typename T, bool CL>
+__global__ void __launch_bounds__(SLAB_THREADS<T, CL>, 1)
+    k_md_slab(SysDev S, SlabDev D, long long step0, long long nsteps, int phase_half) {
     using V = typename V2<T>::type;
     __shared__ int s_w[33];
     __shared__ unsigned s_vm[SLAB_MAX_THREADS / 32];
@@ -650,7 +706,7 @@ __global__ void __launch_bounds__(SLAB_THREADS<T>, 1) k_md_slab(SysDev S, SlabDe
     const int per_lg = S.n_dx * S.nb;
     int *sh_hist = reinterpret_cast<int *>(res_smem);
     SlabMem<T> M;
-    M.L = slab_layout<T>(smem_hist_bytes(S.n_lg, S.n_dx, S.nb), D.p_cap, D.h_cap, D.e_cap, D.ncells, nt);
+    M.L = slab_layout<T>(smem_hist_bytes(S.n_lg, S.n_dx, S.nb), D.p_cap, D.h_cap, D.e_cap, D.ncells);
     SlabCta X;
     X.k = (int)blockIdx.x;
     X.g = D.g;
@@ -661,6 +717,12 @@ __global__ void __launch_bounds__(SLAB_THREADS<T>, 1) k_md_slab(SysDev S, SlabDe
     X.last = (int)((long long)(X.down + 1) * R.nc / X.g) - (int)((long long)X.down * R.nc / X.g) > 1;
     X.par = 0;
     X.seq = 0;
+    if constexpr (CL) {   // every CTA runs: its shared memory may be written
+        __shared__ unsigned s_box[2 * SLAB_CLUSTER];
+        X.box = s_box;
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
     SlabPar<T> P;
     P.h = rd<T>(R.h, R.hf);
     P.rc2 = rd<T>(R.rc2, R.rc2f);
@@ -703,11 +765,11 @@ __global__ void __launch_bounds__(SLAB_THREADS<T>, 1) k_md_slab(SysDev S, SlabDe
     }
     __syncthreads();
     fits = slab_publish_rows<T>(D, M, X) && fits;
-    unsigned over = slab_sync(S, D, X, !fits, ok);
+    unsigned over = slab_sync<CL>(S, D, X, !fits, ok);
     if (!ok) return;
     if (!over) {
         slab_read_rows<T>(D, M, X);
-        over = slab_sync(S, D, X, !slab_lists<T>(R, D, M, X, s_w), ok);
+        over = slab_sync<CL>(S, D, X, !slab_lists<T>(R, D, M, X, s_w), ok);
         if (!ok) return;
     }
     if (over) {   // nothing was changed: all steps are left
@@ -757,7 +819,7 @@ __global__ void __launch_bounds__(SLAB_THREADS<T>, 1) k_md_slab(SysDev S, SlabDe
         unsigned vmax = 0;
         if (tid == 0)
             for (int w = 0; w < nw; ++w) vmax = max(vmax, s_vm[w]);
-        vmax = slab_sync(S, D, X, vmax, ok);
+        vmax = slab_sync<CL>(S, D, X, vmax, ok);
         if (!ok) return;
         slab_read_offsets<T>(D, M, X);
         disp += (double)__uint_as_float(vmax) * 1.0000001;
@@ -851,7 +913,7 @@ __global__ void __launch_bounds__(SLAB_THREADS<T>, 1) k_md_slab(SysDev S, SlabDe
                 nout[1] += t1;
             }
             if (tid < 2) D.mig_n[X.k * 2 + tid] = nout[tid];
-            over = slab_sync(S, D, X, nout[0] > D.h_cap || nout[1] > D.h_cap, ok);
+            over = slab_sync<CL>(S, D, X, nout[0] > D.h_cap || nout[1] > D.h_cap, ok);
             if (!ok) return;
             if (over) {   // nobody has moved yet
                 early = true;
@@ -897,7 +959,7 @@ __global__ void __launch_bounds__(SLAB_THREADS<T>, 1) k_md_slab(SysDev S, SlabDe
             X.p = fits ? keep + in0 + in1 : keep;
             __syncthreads();
             fits = slab_publish_rows<T>(D, M, X) && fits;
-            over = slab_sync(S, D, X, !fits, ok);
+            over = slab_sync<CL>(S, D, X, !fits, ok);
             if (!ok) return;
             if (over) {   // every slab writes its stayers and its own leavers
                 X.p = keep;
@@ -908,7 +970,7 @@ __global__ void __launch_bounds__(SLAB_THREADS<T>, 1) k_md_slab(SysDev S, SlabDe
             }
             slab_read_rows<T>(D, M, X);
         }
-        over = slab_sync(S, D, X, !slab_lists<T>(R, D, M, X, s_w), ok);
+        over = slab_sync<CL>(S, D, X, !slab_lists<T>(R, D, M, X, s_w), ok);
         if (!ok) return;
         if (over) {
             early = true;
@@ -918,9 +980,9 @@ __global__ void __launch_bounds__(SLAB_THREADS<T>, 1) k_md_slab(SysDev S, SlabDe
     }
     // ---- write back into the other set, slab after slab
     const int own = X.p + extra;
-    slab_sync(S, D, X, (unsigned)own, ok);
+    slab_sync<CL>(S, D, X, (unsigned)own, ok);
     if (!ok) return;
-    if (tid == 0) s_before = slab_before(D, X);
+    if (tid == 0) s_before = slab_before<CL>(D, X);
     __syncthreads();
     {
         V *pos = static_cast<V *>(S.pos[nset][0]);

@@ -105,3 +105,16 @@ def test_slab_overflow_goes_on_globally(mdlg, prec, kind):
     p.nbr_max = 200
     a, b = _pair(mdlg, p, (x, y, st.vx, vy), steps)
     _check(b, a)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("n,phi,skin", [(300, 0.6, 2.2), (8100, 0.0784, 0.5), (8700, 0.0784, 0.5)])
+def test_slab_long_lists_and_cluster_edge(mdlg, prec, n, phi, skin):
+    """Lists of more than 64 entries, and sizes on both sides of the one up to
+    which FP32 slabs form a cluster: equal bits on both engines."""
+    L = inputs.box_length(n, phi)
+    st = inputs.lattice_gas_state(n, L, 3.0, seed=n)
+    p = mdlg.make_params(n, L, precision=prec, skin=skin, lg_every=(25, 40), lx=(int(L), int(L / 2)))
+    p.nbr_max = 200
+    a, b = _pair(mdlg, p, (st.x, st.y, st.vx, st.vy), (40, 60))
+    _check(b, a)
