@@ -14,6 +14,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -174,7 +175,7 @@ int gemm_launch(const GemmArgs &g, cudaStream_t st) {
 //   warp 0 lane 0  producer: streams weight chunks, pre-packed in global
 //                  memory in the exact shared-memory layout, with one bulk
 //                  copy (TMA) each into a ring of F_STAGES buffers;
-//   warp 1 lane 0  MMA issuer: per (tile pair, layer, slot) waits for the
+//   warp 1         MMA issuer: per (tile pair, layer, slot) waits for the
 //                  slot's activations, issues tcgen05.mma into the slot's
 //                  128 x 256 FP32 accumulator in TMEM, commits;
 //   warps 2..17    epilogue, 8 warps per slot: stage the inputs, then per
@@ -192,19 +193,31 @@ int gemm_launch(const GemmArgs &g, cudaStream_t st) {
 // so the epilogue reads finished pre-activations from TMEM.
 // A warp may read only the TMEM lanes 32 (warp mod 4) .. +31, so epilogue
 // warp w serves rows 32 (w mod 4) + lane and one half of the columns.
+// What bounds it: each slot alternates between its MMAs (about 2,500 clocks
+// per hidden layer) and its epilogue (2,350: the SFU), so two slots keep either
+// unit a little over half busy.  Time per 1,048,576 queries (81 classes): 397
+// us.  It was 490 while one lane of a divergent branch issued the MMAs: 650
+// clocks passed between a layer's first two chunks and the issuer, not the
+// tensor core, was the bound (with 3/4 of the MMAs left out it still took 437
+// us).  The issuing warp now runs in uniform control flow and elects the lane.
+// Ring stages of 6 x 16 KB: 430 us; 4 x 24 KB as 3 x 32 KB; a CTA pair per 256
+// rows (cta_group::2, half the weight traffic) needs an exchange between the
+// CTAs per chunk and layer and took 748 us with the old issuer.
 // Every wait is bounded; a wait that gives up sets the status flag and the
 // roles wind down (uniformly within a slot) instead of hanging.
-constexpr int FK = 64;                     // features per weight chunk
+constexpr int FK = 64;                     // features per weight chunk (training)
 constexpr int F_STAGES = 3;
 constexpr int F_SBO_A = 256 / 8 * 128;     // 8-row groups of the 256-wide activation tile
-constexpr int F_SBO_B = FK / 8 * 128;      // 8-row groups of a weight chunk
-constexpr int F_SBO_B0 = 16 / 8 * 128;     // 8-row groups of the K = 16 layer-1 operand
-constexpr int F_CHUNK_BYTES = 256 * FK * 2;
+constexpr int F_SBO_B = FK / 8 * 128;      // 8-row groups of a weight chunk (training)
+constexpr int F_SBO_IN = 16 / 8 * 128;     // 8-row groups of the staged K = 16 input rows
+constexpr int F_CHUNK_BYTES = 32768;
+constexpr int F_SLICES = 1 + 256 / 16;     // of a layer's operand: the bias, then the weights
 constexpr int F_MAXL = 15;
 constexpr int F_EPI_WARPS = 8;             // per slot
 constexpr int F_THREADS = (2 + 2 * F_EPI_WARPS) * 32;
 constexpr int F_ACT_BYTES = 128 * 256 * 2;
 constexpr int F_RED_OFF = 60 * 1024;       // softmax partials inside a slot's tile
+constexpr int F_IN_OFF = 56 * 1024;        // the next tile's inputs inside a slot's tile
 constexpr int MLP_MAX_CLASSES = 112;       // FP32 stage rows must end below them
 
 struct FusedArgs {
@@ -214,7 +227,6 @@ struct FusedArgs {
     int ncls;
     float4 shift, scale;
     const bf16 *Wp[F_MAXL + 1];    // packed operand of every layer (layer 0: split K = 16 with bias)
-    const bf16 *Bp[F_MAXL + 1];    // packed bias operand (N x 16) of layers >= 1
     int nt;                        // layers; the last one is the output
     int p_aligned;                 // P 16-byte aligned: output tiles by bulk copy
     int *status;
@@ -240,9 +252,13 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<uint32_t *>(&v);
 }
 
-// ring chunks of layer l: layer 0 one K = 16 chunk; the others a bias
-// chunk (N x 16) followed by the weight chunks
-__device__ __forceinline__ int layer_chunks(int l) { return l == 0 ? 1 : 1 + 256 / FK; }
+// A layer's packed operand is a run of K = 16 slices of N x 16 (layer 0: one;
+// the others: the bias, then 16 of the weights), each [K / 8][N][8]: core
+// matrices of 8 rows follow one another along N, so that any run of slices is
+// contiguous.  A ring chunk is as many slices as fit a stage.
+__device__ __forceinline__ int layer_slices(int l) { return l == 0 ? 1 : F_SLICES; }
+__device__ __forceinline__ int chunk_slices(int N) { return F_CHUNK_BYTES / (N * 32); }
+__device__ __forceinline__ int slice_off(int n, int k, int N) { return ((k >> 3) * N + n) * 8 + (k & 7); }
 
 __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(FusedArgs a) {
     extern __shared__ __align__(1024) unsigned char sm[];
@@ -253,7 +269,8 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(FusedArgs a) {
     uint64_t *actr = accf + 2;             // per slot: activations written, TMEM read
     uint32_t *s_tmem = reinterpret_cast<uint32_t *>(actr + 2);
     unsigned char *ones = reinterpret_cast<unsigned char *>(s_tmem + 4);   // 8 x 16 BF16 block
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // (warp index by a shuffle: known to be uniform, so is the issuer's control flow)
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     if (warp == 1) umma::tmem_alloc(s_tmem, 512);
     if (tid < 128) {
         // BF16 element e of the block is (r, k) = ((e % 64) / 8, 8 (e / 64) + e % 8)
@@ -292,11 +309,10 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(FusedArgs a) {
                 for (int l = 0; l < nt && !bad; ++l)
                     for (int s = 0; s < 2 && !bad; ++s) {
                         if (2 * p + s >= my_tiles) continue;
-                        const int N = l == nt - 1 ? 128 : 256;
-                        for (int kc = 0; kc < layer_chunks(l); ++kc, ++c) {
-                            const bool small = l == 0 || kc == 0;     // K = 16 chunk
-                            const uint32_t bytes = (uint32_t)(N * (small ? 16 : FK) * 2);
-                            const bf16 *srcp = l == 0 ? a.Wp[0] : kc == 0 ? a.Bp[l] : a.Wp[l] + (size_t)(kc - 1) * N * FK;
+                        const int N = l == nt - 1 ? 128 : 256, ns = layer_slices(l), cs = chunk_slices(N);
+                        for (int j = 0; j < ns; j += cs, ++c) {
+                            const uint32_t bytes = (uint32_t)(N * 32 * min(cs, ns - j));
+                            const bf16 *srcp = a.Wp[l] + (size_t)j * N * 16;
                             // from the second pass on, wait until the MMAs of
                             // the previous pass have released the stage
                             if (c >= F_STAGES && !umma::mbar_wait(&empty[st], ph ^ 1u, GEMM_WAIT_NS)) {
@@ -325,61 +341,69 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(FusedArgs a) {
         __syncwarp();
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            int st = 0;
-            uint32_t ph = 0;
-            long long c = 0;          // chunks consumed
-            int last_st = 0;
-            uint32_t last_ph = 0;
-            const uint64_t ring_desc = umma::desc(umma::saddr(ring), 128, F_SBO_B);
-            const uint64_t ring_desc0 = umma::desc(umma::saddr(ring), 128, F_SBO_B0);
-            const uint64_t ones_desc = umma::desc(umma::saddr(ones), 128, 0);   // every row group: the same 8 rows
-            uint32_t kpar[2] = {0u, 0u};   // per slot: parity of the next actr phase
-            for (long long p = 0; p < npairs && !bad; ++p)
-                for (int l = 0; l < nt && !bad; ++l)
-                    for (int s = 0; s < 2 && !bad; ++s) {
-                        if (2 * p + s >= my_tiles) continue;
-                        if (!umma::mbar_wait(&actr[s], kpar[s], GEMM_WAIT_NS)) {
-                            bad = true;
-                            break;
-                        }
-                        kpar[s] ^= 1u;
-                        umma::fence_after();
-                        const uint32_t idesc = umma::idesc_bf16(128, l == nt - 1 ? 128 : 256);
-                        const uint64_t act_desc = umma::desc(umma::saddr(sm + s * F_ACT_BYTES), 128, F_SBO_A);
-                        const uint32_t d = tmem + (uint32_t)(s * 256);
-                        for (int kc = 0; kc < layer_chunks(l); ++kc, ++c) {
-                            if (!umma::mbar_wait(&full[st], ph, GEMM_WAIT_NS)) {
-                                bad = true;
-                                break;
-                            }
-                            umma::fence_after();
-                            const uint64_t soff = (uint64_t)((st * F_CHUNK_BYTES) >> 4);
-                            if (l == 0) {
-                                umma::mma(d, act_desc, ring_desc0 + soff, idesc, 0u);
-                            } else if (kc == 0) {
-                                umma::mma(d, ones_desc, ring_desc0 + soff, idesc, 0u);     // accumulator = bias
-                            } else {
-                                const uint64_t adesc = act_desc + (uint64_t)(((kc - 1) * (FK / 8) * 128) >> 4);
+        // the whole warp runs the loop, one elected lane issues
+        int st = 0;
+        uint32_t ph = 0;
+        long long c = 0;          // chunks consumed
+        int last_st = 0;
+        uint32_t last_ph = 0;
+        const uint64_t ones_desc = umma::desc(umma::saddr(ones), 128, 0);   // every row group: the same 8 rows
+        uint32_t kpar[2] = {0u, 0u};   // per slot: parity of the next actr phase
+        const auto layer = [&](auto n_, auto ns_, int s, uint64_t first) {   // operand rows, slices; A of slice 0
+            constexpr int N = decltype(n_)::value, NS = decltype(ns_)::value, CS = F_CHUNK_BYTES / (N * 32);
+            const uint32_t idesc = umma::idesc_bf16(128, N);
+            const uint64_t act_desc = umma::desc(umma::saddr(sm + s * F_ACT_BYTES), 128, F_SBO_A);
+            const uint64_t ring_desc = umma::desc(umma::saddr(ring), N * 16, 128);
+            const uint32_t d = tmem + (uint32_t)(s * 256);
+            for (int j = 0; j < NS; j += CS, ++c) {
+                if (__any_sync(0xffffffffu, !umma::mbar_wait(&full[st], ph, GEMM_WAIT_NS))) return false;
+                umma::fence_after();
+                const uint64_t bdesc = ring_desc + (uint64_t)((st * F_CHUNK_BYTES) >> 4);
+                const uint64_t adesc = act_desc + (uint64_t)(j * 16);
+                if (umma::elect_one()) {
 #pragma unroll
-                                for (int k4 = 0; k4 < FK / 16; ++k4)
-                                    umma::mma(d, adesc + (uint64_t)(k4 * 16), ring_desc + soff + (uint64_t)(k4 * 16),
-                                              idesc, 1u);
-                            }
-                            umma::commit(&empty[st]);
-                            last_st = st;
-                            last_ph = ph;
-                            if (++st == F_STAGES) {
-                                st = 0;
-                                ph ^= 1u;
-                            }
-                        }
-                        if (!bad) umma::commit(&accf[s]);
+                    for (int q = 0; q < CS; ++q)
+                        if (j + q < NS)
+                            umma::mma(d, q || j ? adesc + (uint64_t)(q * 16) - 16 : first, bdesc + (uint64_t)(q * N * 2),
+                                      idesc, q || j ? 1u : 0u);
+                    umma::commit(&empty[st]);
+                }
+                __syncwarp();
+                last_st = st;
+                last_ph = ph;
+                if (++st == F_STAGES) {
+                    st = 0;
+                    ph ^= 1u;
+                }
+            }
+            if (umma::elect_one()) umma::commit(&accf[s]);
+            __syncwarp();
+            return true;
+        };
+        for (long long p = 0; p < npairs && !bad; ++p)
+            for (int l = 0; l < nt && !bad; ++l)
+                for (int s = 0; s < 2 && !bad; ++s) {
+                    if (2 * p + s >= my_tiles) continue;
+                    if (__any_sync(0xffffffffu, !umma::mbar_wait(&actr[s], kpar[s], GEMM_WAIT_NS))) {
+                        bad = true;
+                        break;
                     }
-            // the last MMAs must be complete before TMEM is released
-            if (c > 0 && !umma::mbar_wait(&empty[last_st], last_ph, GEMM_WAIT_NS)) bad = true;
-            if (bad) atomicOr(a.status, 1);
-        }
+                    kpar[s] ^= 1u;
+                    umma::fence_after();
+                    using C1 = std::integral_constant<int, 1>;
+                    using CF = std::integral_constant<int, F_SLICES>;
+                    using N128 = std::integral_constant<int, 128>;
+                    using N256 = std::integral_constant<int, 256>;
+                    bool ok;
+                    if (l == 0)
+                        ok = layer(N256{}, C1{}, s, umma::desc(umma::saddr(sm + s * F_ACT_BYTES + F_IN_OFF), 128, F_SBO_IN));
+                    else if (l < nt - 1) ok = layer(N256{}, CF{}, s, ones_desc);
+                    else ok = layer(N128{}, CF{}, s, ones_desc);
+                    bad = !ok;
+                }
+        // the last MMAs must be complete before TMEM is released
+        if (c > 0 && __any_sync(0xffffffffu, !umma::mbar_wait(&empty[last_st], last_ph, GEMM_WAIT_NS))) bad = true;
+        if (bad && lane == 0) atomicOr(a.status, 1);
         __syncwarp();
     } else {
         // ------------------------------------------------ epilogue slots
@@ -394,6 +418,11 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(FusedArgs a) {
         const int hs = (ncls + 31) / 32 * 16;                   // softmax columns per half
         const int cbeg = half * hs, cend = min(cbeg + hs, ncls);
         uint32_t kpar = 0u;                                     // parity of the next accf phase
+        const auto input = [&](long long m) {
+            return half == 0 && m + r < a.M ? __ldg(reinterpret_cast<const float4 *>(a.X) + m + r)
+                                            : make_float4(0.f, 0.f, 0.f, 0.f);
+        };
+        float4 x = input((blockIdx.x + (long long)s * gridDim.x) * 128);
         for (long long p = 0; p < npairs; ++p) {
             const long long j = 2 * p + s;
             if (j >= my_tiles) break;
@@ -402,7 +431,6 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(FusedArgs a) {
             if (half == 0) {
                 uint4 u0 = make_uint4(0, 0, 0, 0), u1 = u0;
                 if (m0 + r < a.M) {
-                    const float4 x = __ldg(reinterpret_cast<const float4 *>(a.X) + m0 + r);
                     const float f0 = (x.x - a.shift.x) / a.scale.x, f1 = (x.y - a.shift.y) / a.scale.y;
                     const float f2 = (x.z - a.shift.z) / a.scale.z, f3 = (x.w - a.shift.w) / a.scale.w;
                     const __nv_bfloat162 h01 = __floats2bfloat162_rn(f0, f1), h23 = __floats2bfloat162_rn(f2, f3);
@@ -415,8 +443,9 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(FusedArgs a) {
                     u1.y = u0.y;
                     u1.z = pack_bf16(1.f, 1.f);     // k = 12, 13: the bias columns
                 }
-                *reinterpret_cast<uint4 *>(act + act_off(r, 0)) = u0;
-                *reinterpret_cast<uint4 *>(act + act_off(r, 8)) = u1;
+                unsigned char *in = act + F_IN_OFF + (r >> 3) * F_SBO_IN + (r & 7) * 16;
+                *reinterpret_cast<uint4 *>(in) = u0;
+                *reinterpret_cast<uint4 *>(in + 128) = u1;
                 umma::fence_proxy_smem();
             }
             umma::mbar_arrive(&actr[s]);
@@ -424,6 +453,8 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(FusedArgs a) {
             for (int l = 0; l < nt && !bad; ++l) {
                 const bool ok = umma::mbar_wait(&accf[s], kpar, GEMM_WAIT_NS);
                 kpar ^= 1u;
+                // the last tile's rows have left the stage that the activations overwrite
+                if (l == 0 && ts == 0) umma::bulk_wait_read();
                 if (!umma::bar_and(bar_id, nthr, ok)) {
                     bad = true;
                     break;
@@ -458,6 +489,7 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(FusedArgs a) {
                     // normalised rows are staged densely (stride ncls) over
                     // the slot's tile, which is then one contiguous block of
                     // P, written by a single bulk copy (TMA)
+                    x = input(m0 + 2ll * gridDim.x * 128);   // of the slot's next tile
                     float mx = -INFINITY;
                     for (int c0 = cbeg; c0 < cend; c0 += 16) {
                         uint32_t v[16];
@@ -471,6 +503,7 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(FusedArgs a) {
                     umma::bar_sync(bar_id, nthr);
                     mx = fmaxf(red[r], red[128 + r]);
                     float sum = 0.f;
+                    float *row = stage + r * ncls;
                     for (int c0 = cbeg; c0 < cend; c0 += 16) {
                         uint32_t v[16];
                         umma::ld16_async(trow + (uint32_t)c0, v);
@@ -480,14 +513,21 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(FusedArgs a) {
                             if (c0 + i < cend) {
                                 const float ez = __expf(__uint_as_float(v[i]) - mx);
                                 sum += ez;
-                                stage[r * ncls + c0 + i] = ez;
+                                row[c0 + i] = ez;
                             }
                     }
                     umma::fence_before();
                     red[256 + half * 128 + r] = sum;
                     umma::bar_sync(bar_id, nthr);
                     const float inv = 1.0f / (red[256 + r] + red[384 + r]);
-                    for (int c = cbeg; c < cend; ++c) stage[r * ncls + c] *= inv;
+                    for (int c = cbeg; c < cend; c += 8) {   // eight loads in flight
+                        float q[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) q[i] = row[min(c + i, cend - 1)] * inv;
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            if (c + i < cend) row[c + i] = q[i];
+                    }
                     umma::fence_proxy_smem();
                     umma::bar_sync(bar_id, nthr);
                     if (ts == 0) {
@@ -498,12 +538,10 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(FusedArgs a) {
                             if (n4) umma::bulk_s2g(dst, stage, n4 * 4);
                             umma::bulk_commit();
                             for (uint32_t i = n4; i < n; ++i) dst[i] = stage[i];
-                            umma::bulk_wait_read();
                         } else {
                             for (uint32_t i = 0; i < n; ++i) dst[i] = stage[i];
                         }
                     }
-                    umma::bar_sync(bar_id, nthr);    // the next tile's inputs overwrite the stage
                 }
             }
             if (bad) break;
@@ -520,8 +558,9 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_mlp_fused(FusedArgs a) {
 
 constexpr size_t FUSED_SMEM = 2 * F_ACT_BYTES + F_STAGES * F_CHUNK_BYTES + (2 * F_STAGES + 4) * 8 + 16 + 256;
 static_assert(FUSED_SMEM <= 232448, "fused MLP shared memory above 227 KB");
-static_assert(128 * MLP_MAX_CLASSES * 4 <= F_RED_OFF && F_RED_OFF + 4 * 128 * 4 <= F_ACT_BYTES,
-              "softmax stage overlaps the partials");
+static_assert(128 * MLP_MAX_CLASSES * 4 <= F_IN_OFF && F_IN_OFF + 128 * 32 <= F_RED_OFF &&
+                  F_RED_OFF + 4 * 128 * 4 <= F_ACT_BYTES,
+              "softmax stage, inputs and partials overlap");
 
 // Splits v into BF16 parts: part 0 = bf16(v), part 1 = bf16(v - part 0).
 __device__ __forceinline__ float split_part(float v, int part) {
@@ -542,7 +581,7 @@ __global__ void k_pack0(const float *W, const float *b, float sc, bf16 *out) {
     float v = 0.f;
     if (k < 12) v = split_part(W[n * 4 + (k & 3)], k < 8 ? 0 : 1);
     else if (k < 14) v = split_part(b[n], k - 12);
-    out[(n >> 3) * (F_SBO_B0 / 2) + (k >> 3) * 64 + (n & 7) * 8 + (k & 7)] = __float2bfloat16_rn(sc * v);
+    out[slice_off(n, k, 256)] = __float2bfloat16_rn(sc * v);
 }
 
 // Packs the bias b [rows] into the K = 16 operand (b_hi, b_lo, 0, ...) of N
@@ -552,24 +591,25 @@ __global__ void k_packb(const float *b, int rows, int N, float sc, bf16 *out) {
     if (i >= N * 16) return;
     const int n = i / 16, k = i % 16;
     const float v = k < 2 && n < rows ? split_part(b[n], k) : 0.f;
-    out[(n >> 3) * (F_SBO_B0 / 2) + (k >> 3) * 64 + (n & 7) * 8 + (k & 7)] = __float2bfloat16_rn(sc * v);
+    out[slice_off(n, k, N)] = __float2bfloat16_rn(sc * v);
 }
 
 // Element of a weight operand of N rows packed in 64-feature chunks, each
 // laid out exactly as a shared-memory weight buffer (rows n0 .. n0 + 8 j of a
-// chunk are contiguous).
+// chunk are contiguous): the training chain's.
 __device__ __forceinline__ int pack_off(int n, int k, int N) {
     const int kk = k % FK;
     return k / FK * N * FK + (n >> 3) * (F_SBO_B / 2) + (kk >> 3) * 64 + (n & 7) * 8 + (kk & 7);
 }
 
-// Packs W [rows][256] (FP32, rows <= N, the others zero) as BF16, times sc.
-__global__ void k_pack(const float *W, int rows, int N, float sc, bf16 *out) {
+// Packs W [rows][256] (FP32, rows <= N, the others zero) as BF16, times sc, in
+// slices or in chunks.
+template <bool SLICES> __global__ void k_pack(const float *W, int rows, int N, float sc, bf16 *out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N * 256) return;
     const int n = i / 256, k = i % 256;
     const float v = n < rows ? __bfloat162float(__float2bfloat16_rn(W[i])) : 0.f;
-    out[pack_off(n, k, N)] = __float2bfloat16_rn(sc * v);
+    out[SLICES ? slice_off(n, k, N) : pack_off(n, k, N)] = __float2bfloat16_rn(sc * v);
 }
 
 // Packs W^T [256][N] (FP32 W [rows][256]) as BF16: the operand of a layer's
@@ -1240,8 +1280,7 @@ struct mlp_model {
     // FP32 master parameters, Adam moments and gradient, packed as `params`
     float *w = nullptr, *mom = nullptr, *var = nullptr, *g = nullptr;
     std::vector<bf16 *> Wf, Wb;   // packed BF16 W and W^T of layers >= 1 (training)
-    std::vector<bf16 *> Wp;       // chunk-packed copies for the fused forward pass
-    std::vector<bf16 *> Bp;       // packed bias operands (layers >= 1)
+    std::vector<bf16 *> Wp;       // bias and weights in slices for the fused forward pass
     bool packed = false;
     int adam_t = 0;
     // workspace
@@ -1304,7 +1343,7 @@ int refresh_bf16(mlp_model *m, cudaStream_t st) {
     const ParamMap pm = m->map();
     for (int l = 1; l < m->nl; ++l) {
         const int n = pm.outp(l) * 256;
-        k_pack<<<(n + 255) / 256, 256, 0, st>>>(m->w + pm.W(l), pm.out(l), pm.outp(l), 1.0f, m->Wf[l]);
+        k_pack<false><<<(n + 255) / 256, 256, 0, st>>>(m->w + pm.W(l), pm.out(l), pm.outp(l), 1.0f, m->Wf[l]);
         k_pack_t<<<(n + 255) / 256, 256, 0, st>>>(m->w + pm.W(l), pm.out(l), pm.outp(l), m->Wb[l]);
     }
     MD_CUDA_TRY(cudaGetLastError());
@@ -1422,14 +1461,13 @@ int mlp_create(int32_t n_hidden, int32_t width, int32_t n_classes, const float *
     A((void **)&m->var, np);
     A((void **)&m->g, np);
     m->Wf.assign(m->nl, nullptr);
-    m->Wb = m->Wp = m->Bp = m->Wf;
+    m->Wb = m->Wp = m->Wf;
     for (int l = 0; l < m->nl; ++l) {
         const size_t nw = (size_t)pm.outp(l) * pm.in(l);
         if (l > 0) {
             A((void **)&m->Wf[l], nw * 2);
             A((void **)&m->Wb[l], nw * 2);
-            A((void **)&m->Wp[l], nw * 2);
-            A((void **)&m->Bp[l], (size_t)pm.outp(l) * 16 * 2);
+            A((void **)&m->Wp[l], (nw + (size_t)pm.outp(l) * 16) * 2);
         } else {
             A((void **)&m->Wp[0], (size_t)pm.outp(0) * 16 * 2);
         }
@@ -1488,8 +1526,9 @@ int mlp_forward(mlp_model *m, const float *X, int64_t M, float *P_out, void *str
         for (int l = 1; l < m->nl; ++l) {
             const int n = pm.outp(l) * 256;
             const float sc = l < m->nl - 1 ? 0.5f : 1.0f;
-            k_pack<<<(n + 255) / 256, 256, 0, st>>>(m->w + pm.W(l), pm.out(l), pm.outp(l), sc, m->Wp[l]);
-            k_packb<<<(pm.outp(l) * 16 + 255) / 256, 256, 0, st>>>(m->w + pm.b(l), pm.out(l), pm.outp(l), sc, m->Bp[l]);
+            const int nb = pm.outp(l) * 16;   // the bias slice comes first
+            k_packb<<<(nb + 255) / 256, 256, 0, st>>>(m->w + pm.b(l), pm.out(l), pm.outp(l), sc, m->Wp[l]);
+            k_pack<true><<<(n + 255) / 256, 256, 0, st>>>(m->w + pm.W(l), pm.out(l), pm.outp(l), sc, m->Wp[l] + nb);
         }
         MD_CUDA_TRY(cudaGetLastError());
         m->packed = true;
@@ -1504,7 +1543,6 @@ int mlp_forward(mlp_model *m, const float *X, int64_t M, float *P_out, void *str
     a.nt = m->nl;
     for (int l = 0; l < m->nl; ++l) {
         a.Wp[l] = m->Wp[l];
-        a.Bp[l] = m->Bp[l];
     }
     a.p_aligned = ((uintptr_t)P_out & 15) == 0;
     a.status = m->status;
