@@ -740,7 +740,7 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
     uint64_t *done = full + S::NBUF;                                            // accumulator complete
     uint64_t *arr = done + 1;                                                   // [2] the other CTAs' columns of an A operand are here
     uint32_t *s_tmem = reinterpret_cast<uint32_t *>(arr + 2);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int rank = (int)cluster_rank(), m0 = (int)(blockIdx.x / CS) * 128;
     const ParamMap pm = a.pm;
     const int nl = pm.nl, B = a.B, nops = 2 * (nl - 1);
@@ -762,7 +762,7 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
     const uint32_t tmem = *s_tmem, trow = tmem + ((uint32_t)(quad * 32) << 16);
     const uint32_t act0 = umma::saddr(sm);
     bool bad = false;
-    uint32_t arr_par = 0;   // thread 0: parity of the next phase of arr[0], arr[1]
+    uint32_t arr_par = 0;   // warp 0: parity of the next phase of arr[0], arr[1]
     // operation g reads operand g & 1 up to the output layer; the backward
     // pass starts over from the output layer's
     const auto a_buf = [&](int g) { return g < nl - 1 ? g & 1 : (g - 1) & 1; };
@@ -780,7 +780,10 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
         for (int kc = 0; kc < K / FK; ++kc)
             umma::bulk_g2s(dst + kc * ns * FK * 2, src + (size_t)kc * N * FK, (uint32_t)(ns * FK * 2), bar);
     };
-    const auto product = [&](int g) {   // thread 0: issue the operation's MMAs; operand g & 1
+    // warp 0: issues the operation's MMAs, one elected lane of uniform control
+    // flow (from a divergent branch a product took 0.35 us more); operand
+    // g & 1
+    const auto product = [&](int g) {
         const int l = op_layer(g);
         const bool fwd = g < nl - 1;
         const int ns = (fwd ? pm.outp(l) : 256) / CS, K = fwd ? 256 : pm.outp(l), cur = a_buf(g);
@@ -788,21 +791,24 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
         // CTA may leave before those into it have landed
         if (!umma::mbar_wait(&arr[cur], arr_par >> cur & 1u, GEMM_WAIT_NS)) bad = true;
         arr_par ^= 1u << cur;
+        bad = __any_sync(0xffffffffu, bad);
         if (bad) return;
-        if (!umma::mbar_wait(&full[g % S::NBUF], (g / S::NBUF) & 1, GEMM_WAIT_NS)) {
-            bad = true;
-            return;
-        }
+        bad = __any_sync(0xffffffffu, !umma::mbar_wait(&full[g % S::NBUF], (g / S::NBUF) & 1, GEMM_WAIT_NS));
+        if (bad) return;
         umma::fence_after();
         const uint32_t idesc = umma::idesc_bf16(128, ns);
         const uint64_t ad = umma::desc(act0 + cur * F_ACT_BYTES, 128, F_SBO_B);
         const uint64_t bd = umma::desc(umma::saddr(wbuf + (g % S::NBUF) * S::WBYTES), 128, F_SBO_B);
-        for (int kc = 0; kc < K / FK; ++kc)
+        if (umma::elect_one()) {
+            for (int kc = 0; kc < K / FK; ++kc)
 #pragma unroll
-            for (int k4 = 0; k4 < FK / 16; ++k4)
-                umma::mma(tmem, ad + (uint64_t)((kc * T_SLAB) >> 4) + (uint64_t)(k4 * 16),
-                          bd + (uint64_t)((kc * ns * FK * 2) >> 4) + (uint64_t)(k4 * 16), idesc, (kc | k4) ? 1u : 0u);
-        umma::commit(done);
+                for (int k4 = 0; k4 < FK / 16; ++k4)
+                    umma::mma(tmem, ad + (uint64_t)((kc * T_SLAB) >> 4) + (uint64_t)(k4 * 16),
+                              bd + (uint64_t)((kc * ns * FK * 2) >> 4) + (uint64_t)(k4 * 16), idesc,
+                              (kc | k4) ? 1u : 0u);
+            umma::commit(done);
+        }
+        __syncwarp();
     };
     // every thread: the operation's accumulator is complete; its weight buffer is free again
     const auto finish = [&](int g) {
@@ -881,7 +887,7 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
     send(0, my_slab, 1, 0, SLABS);
     // ---- hidden layers
     for (int g = 0; g < nl - 2; ++g) {
-        if (tid == 0) product(g);
+        if (warp == 0) product(g);
         const float *b = a.w + pm.b(g + 1) + rank * S::NS + grp * CH;
         float *Z = a.Z + (size_t)(g + 1) * 256 * B;
         bf16 *H = a.H + (size_t)(g + 1) * 256 * B;
@@ -926,7 +932,7 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
     bf16 *dl = reinterpret_cast<bf16 *>(logits + S::RP * T_LOGIT_LD);                 // [RP][T_DLOG_LD]
     {
         const int g = nl - 2;
-        if (tid == 0) product(g);
+        if (warp == 0) product(g);
         const float *b = a.w + pm.b(nl - 1);
         float bias[CO];
 #pragma unroll
@@ -1006,7 +1012,7 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
     // ---- backward: dZ_{l-1} = (dZ_l W_l) silu'(Z_{l-1})
     for (int l = nl - 1; l >= 1; --l) {
         const int g = 2 * (nl - 1) - l;
-        if (tid == 0) product(g);
+        if (warp == 0) product(g);
         const float *Z = a.Z + (size_t)(l - 1) * 256 * B;
         dZ = a.dZ + (size_t)(l - 1) * 256 * B;
         float z[CH];   // requested while the product runs
@@ -1030,10 +1036,11 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
         if (l > 1) send(a_buf(g + 1), my_slab, 1, 0, SLABS);
     }
     cluster_sync();   // no CTA leaves while another may read or write its shared memory
+    if (warp == 0) bad = __any_sync(0xffffffffu, bad);
     if (bad) {
         // a wait gave up: products may still run; wait (with a limit) before
         // their TMEM is freed, and flag it
-        if (tid == 0) {
+        if (warp == 0 && umma::elect_one()) {   // the lane that issued
             umma::commit(done);
             umma::mbar_wait(done, nops & 1, GEMM_WAIT_NS);
         }
@@ -1071,7 +1078,7 @@ __host__ __device__ inline int grad_sums(const ParamMap &pm) { return pm.nl * 25
 
 __global__ void __launch_bounds__(128) k_train_grads(const __grid_constant__ GradArgs a) {
     extern __shared__ __align__(1024) unsigned char sm[];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, B = a.B;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31, B = a.B;
     const int tiles = grad_tiles(a.pm);
     if ((int)blockIdx.x >= tiles * a.ks) {
         const int per = grad_sums(a.pm) / 128, e = (int)blockIdx.x - tiles * a.ks;
@@ -1148,7 +1155,7 @@ __global__ void __launch_bounds__(128) k_train_grads(const __grid_constant__ Gra
         umma::fence_proxy_smem();
         __syncthreads();
         const int s = kt % G_STAGES;
-        if (tid == 0) {
+        if (warp == 0 && umma::elect_one()) {
             umma::fence_after();
             const uint32_t a0 = umma::saddr(sm + s * G_STAGE_BYTES), b0 = a0 + G_STAGE_BYTES / 2;
 #pragma unroll
@@ -1169,7 +1176,8 @@ __global__ void __launch_bounds__(128) k_train_grads(const __grid_constant__ Gra
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     if (s_ok && !umma::mbar_wait(&mbar[(nk - 1) % G_STAGES], ((nk - 1) / G_STAGES) & 1, GEMM_WAIT_NS)) s_ok = 0;
-    if (!s_ok && tid == 0) {
+    __syncthreads();
+    if (!s_ok && warp == 0 && umma::elect_one()) {
         umma::commit(&mbar[G_STAGES]);
         umma::mbar_wait(&mbar[G_STAGES], 0, GEMM_WAIT_NS);
     }
