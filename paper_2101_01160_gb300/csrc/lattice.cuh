@@ -70,12 +70,9 @@ __device__ __forceinline__ int lattice_floor_f32(int c, T off, double h, float h
     return lattice_cell_slow(c, (double)off, h, dxl, lx);
 }
 
-template <typename T>
-__device__ __forceinline__ int lattice_cell_f32(int c, T off, double h, float hf, double dxl, float invf,
-                                                int lx) {
-    int l = lattice_floor_f32<T>(c, off, h, hf, dxl, invf, lx);
-    // positions within a box edge of the box need one wrap; others the
-    // general reduction
+// l modulo lx: positions within a box edge of the box need one wrap; others
+// the general reduction.
+__device__ __forceinline__ int lattice_wrap(int l, int lx) {
     if (l < 0) l += lx;
     else if (l >= lx) l -= lx;
     if (l < 0 || l >= lx) {
@@ -83,6 +80,12 @@ __device__ __forceinline__ int lattice_cell_f32(int c, T off, double h, float hf
         if (l < 0) l += lx;
     }
     return l;
+}
+
+template <typename T>
+__device__ __forceinline__ int lattice_cell_f32(int c, T off, double h, float hf, double dxl, float invf,
+                                                int lx) {
+    return lattice_wrap(lattice_floor_f32<T>(c, off, h, hf, dxl, invf, lx), lx);
 }
 
 // Division of 0 <= c < 2^31 by an invariant ncell >= 1 as one high product

@@ -41,10 +41,12 @@ __device__ __forceinline__ int occ_index(const OccParams &P, int c0, T ox0, T oy
     int cx0, cy0, cx1, cy1;
     split_cell(c0, P.ncell, P.div, cx0, cy0);
     split_cell(c1, P.ncell, P.div, cx1, cy1);
-    const int sx1 = lattice_cell_f32<T>(cx1, ox1, P.h, P.hf, P.dxl, P.invf, P.lx);
-    const int sy1 = lattice_cell_f32<T>(cy1, oy1, P.h, P.hf, P.dxl, P.invf, P.lx);
-    const int vx = lattice_shift_near(sx1 - lattice_cell_f32<T>(cx0, ox0, P.h, P.hf, P.dxl, P.invf, P.lx), P.lx);
-    const int vy = lattice_shift_near(sy1 - lattice_cell_f32<T>(cy0, oy0, P.h, P.hf, P.dxl, P.invf, P.lx), P.lx);
+    // only the arrival cells are needed reduced modulo lx
+    const int fx1 = lattice_floor_f32<T>(cx1, ox1, P.h, P.hf, P.dxl, P.invf, P.lx);
+    const int fy1 = lattice_floor_f32<T>(cy1, oy1, P.h, P.hf, P.dxl, P.invf, P.lx);
+    const int vx = lattice_shift_floors(fx1 - lattice_floor_f32<T>(cx0, ox0, P.h, P.hf, P.dxl, P.invf, P.lx), P.lx);
+    const int vy = lattice_shift_floors(fy1 - lattice_floor_f32<T>(cy0, oy0, P.h, P.hf, P.dxl, P.invf, P.lx), P.lx);
+    const int sx1 = lattice_wrap(fx1, P.lx), sy1 = lattice_wrap(fy1, P.lx);
     const int site = sy1 * P.lx + sx1;
     oi = -1;
     if (vx >= -P.W && vx <= P.W && vy >= -P.W && vy <= P.W)
