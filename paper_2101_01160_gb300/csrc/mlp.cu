@@ -627,7 +627,7 @@ __global__ void k_pack_t(const float *W, int rows, int N, bf16 *out) {
 // a GEMM, two transposes, column sums, sums of partials, two Adam kernels),
 // 466 us at B = 512 for 0.7 GFLOP: launches, and epilogues that read and
 // wrote one row per lane.  It is three launches now; of 5 layers at B = 512:
-// k_train_chain 41 us, k_train_grads 7.1 us, k_train_update 4.2 us.
+// k_train_chain 38 us, k_train_grads 7.1 us, k_train_update 4.1 us.
 //
 // k_train_chain: one thread-block cluster of CS CTAs per 128-row tile runs the
 // whole forward pass, the softmax and loss, and the backward pass down to the
@@ -638,7 +638,7 @@ __global__ void k_pack_t(const float *W, int rows, int N, bf16 *out) {
 // from there, as contiguous 64-column slabs, to the other CTAs' by bulk copies
 // through distributed shared memory that signal the receiver's mbarrier: no
 // cluster barrier per layer.  (Storing every 16 bytes into all CTAs and
-// meeting at a cluster barrier took 44 us per step in place of 41.)  What it leaves in global memory is transposed, [column][batch], so
+// meeting at a cluster barrier took 44 us per step when this took 41.)  What it leaves in global memory is transposed, [column][batch], so
 // that a warp's 32 rows are contiguous and the weight gradients' operands are
 // K-major.  The tile is one row block of 128 (the M of the instruction); the
 // columns are what is split, because a batch of 512 has only four row blocks.
