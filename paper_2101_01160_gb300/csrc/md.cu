@@ -909,6 +909,7 @@ int launch_resident(md_system *s, long long nsteps) {
         done += n;
     }
     s->needs_sort = true;
+    s->slab_last = false;   // the slots are in this engine's order now
     return MD_OK;
 }
 

@@ -852,6 +852,7 @@ __global__ void __launch_bounds__(RES_THREADS, RES_CTAS_PER_SM) k_md_resident(Sy
 __global__ void k_res_flip(Control *C) {
     C->set ^= 1;
     C->cur = 0;
+    C->slab_order = 0;
 }
 
 }  // namespace mdlg

@@ -247,7 +247,9 @@ __device__ __forceinline__ int slab_before(const SlabDev &D, const SlabCta &X) {
 
 // ---------------------------------------------------------------- halo
 // Publishes the first and the last row of the slab (cells, ids, offsets).
-// Returns whether they fit.
+// Returns whether they fit, and whether every particle lies in the slab's rows
+// (the lists index cells by row; slots in another order than the slabs' leave
+// all steps to the global engine, which sorts).
 template <typename T>
 __device__ bool slab_publish_rows(const SlabDev &D, const SlabMem<T> &M, const SlabCta &X) {
     using V = typename V2<T>::type;
@@ -262,6 +264,7 @@ __device__ bool slab_publish_rows(const SlabDev &D, const SlabMem<T> &M, const S
         // (a slab of one row publishes it once, as its first, for both neighbours)
         const int side = cy == X.r0 ? 0 : (cy == X.r1 - 1 ? 1 : -1);
         uint16_t b = RES_NOB;
+        if (cy < X.r0 || cy >= X.r1) atomicAdd(&s_n[0], D.h_cap + 1);   // a stranger: does not fit
         if (side >= 0) {
             const int at = atomicAdd(&s_n[side], 1);   // the order of a halo changes no result
             if (at < D.h_cap) {

@@ -1,0 +1,53 @@
+"""One replica handed from engine to engine: the slots' order, the step's
+velocity bound and the rebuild count belong to the system, whichever engine ran
+last.  Every walk gives the bits of the global engine alone."""
+
+import itertools
+
+import numpy as np
+import pytest
+
+from paper_2101_01160_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+SLAB, GLOBAL, RESIDENT = (256, 1, 0), (256, 1, 2), (0, 0, 4)
+
+
+def _make(mdlg, n, prec, phi=0.1, T=12.0, skin=0.3):
+    L = inputs.box_length(n, phi)
+    st = inputs.lattice_gas_state(n, L, T, seed=n)
+    p = mdlg.make_params(n, L, precision=prec, skin=skin, lg_every=(20, 50), lx=(int(L), 31))
+    return mdlg.System(p, st.x, st.y, st.vx, st.vy)
+
+
+def _observe(s):
+    out = [np.array(v) for v in s.get_state()] + [t.cpu().numpy() for t in s.get_snapshot(1)]
+    return out + [s.hist_raw(0, k, d)[0] for k in range(2) for d in range(2)]
+
+
+@pytest.mark.parametrize("n", [4000, 12_000])   # slabs as one cluster, slabs as a grid; one and several resident slabs
+def test_walks_over_the_engines(mdlg, n):
+    """All orders of three of slab, resident, global and readout, each step a
+    call of 20 steps, then the slab engine."""
+    ref = {}
+    for k in range(1, 5):
+        s = _make(mdlg, n, mdlg.MD_FP32_CELLOFF)
+        s.tune(*GLOBAL)
+        s.step(20 * k)
+        ref[k] = _observe(s)
+        s.close()
+    for walk in itertools.product("SRGO", repeat=3):
+        s = _make(mdlg, n, mdlg.MD_FP32_CELLOFF)
+        k = 1
+        for op in walk + ("S",):
+            if op == "O":
+                s.get_raw()
+                continue
+            s.tune(*{"S": SLAB, "R": RESIDENT, "G": GLOBAL}[op])
+            s.step(20)
+            k += 1
+        for u, v in zip(_observe(s), ref[k - 1]):
+            assert np.array_equal(u, v), walk
+        s.close()
