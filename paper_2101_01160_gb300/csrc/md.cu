@@ -634,6 +634,11 @@ struct md_system {
     // order; global: sorted within each chunk of the chunk table), so a new
     // shape's first launch rebuilds them (sort only)
     bool lists_valid = false;
+    // The rebuild count does not depend on the engine: it includes the sort of
+    // a new launch shape's first step (shape_new) and the sort behind a
+    // resident launch or a loaded checkpoint (sort_counts), and no sort that
+    // is made only because the slab engine ran
+    bool shape_new = false, sort_counts = false;
     // slab engine (a single replica): its plan and buffers (slab_ok: it has
     // one), whether md_step may take it, and whether the state is as its last
     // launch left it
@@ -908,7 +913,7 @@ int launch_resident(md_system *s, long long nsteps) {
         MD_CUDA_TRY(cudaGetLastError());
         done += n;
     }
-    s->needs_sort = true;
+    s->needs_sort = s->sort_counts = true;
     s->slab_last = false;   // the slots are in this engine's order now
     return MD_OK;
 }
@@ -995,6 +1000,7 @@ int configure_launch(md_system *s, int block, int ppt, int stage) {
     s->stage = stage;
     s->engine = 0;
     s->lists_valid = false;   // chunk table and list layout change with the shape
+    s->shape_new = true;
     return MD_OK;
 }
 
@@ -1015,6 +1021,9 @@ int launch_persistent(md_system *s, long long nsteps, int force_rebuild, const l
     if (force_rebuild != RB_ALL && force_rebuild != RB_SORT && (s->needs_sort || !s->lists_valid)) force_rebuild = RB_NONE;
     s->needs_sort = false;
     s->lists_valid = force_rebuild != RB_SORT;
+    if (force_rebuild == RB_NONE && !s->sort_counts && !s->shape_new) force_rebuild |= RB_QUIET;
+    s->sort_counts = false;
+    if (s->lists_valid) s->shape_new = false;
     const void *fn = persistent_fn(s->prec, s->block, s->stage);
     long long step0 = s->step;
     int phase = s->phase_half;
@@ -1166,6 +1175,8 @@ int launch_slab(md_system *s, long long nsteps) {
     }
     long long step0 = s->step;
     int phase = s->phase_half;
+    s->sl.counted = s->shape_new;
+    s->shape_new = false;
     void *args[] = {&s->sd, &s->sl, &step0, &nsteps, &phase};
     if (!s->sl.cluster)
         MD_CUDA_TRY(cudaMemsetAsync(s->sl.word, 0, sizeof(unsigned long long) * 2 * s->sl.g * s->sl.g, s->st));
@@ -1643,7 +1654,8 @@ int md_checkpoint_load(md_system *s, const void *buf) {
     MD_CUDA_TRY(cudaMemset(s->sd.vmax_rep, 0, sizeof(unsigned) * 3 * (size_t)s->nrep));
     s->step = h.step;
     s->phase_half = h.phase_half;
-    s->needs_sort = true;
+    s->needs_sort = s->sort_counts = true;
+    s->slab_last = false;
     rc = ensure_sorted(s);
     if (rc) return rc;
     return sync_status(s);

@@ -668,13 +668,14 @@ __device__ __forceinline__ void chunk_lists_sorted(const SysDev &S, int set, con
 // offset now lies in, the offset re-expressed from that cell's corner); with
 // RB_NONE every particle keeps its cell (a sort of a state written in
 // another order), and RB_SORT stops before the lists (a sort for a readout,
-// which walks the cells).  Then a counting sort of all particles by cell, particles
+// which walks the cells; never counted).  RB_QUIET, with RB_NONE, leaves the
+// rebuild count alone: a sort that only undoes the slab engine's order.  Then a counting sort of all particles by cell, particles
 // inside one cell ordered by id, so the order -- and therefore every force
 // sum -- is reproducible and independent of the launch shape; then the
 // neighbour lists.  Six grid barriers (seven in the global-memory shapes,
 // whose lists other CTAs read next).  Padding slots keep perm = -1 (set at
 // creation).
-enum RebuildMode { RB_ALL = 1, RB_NONE = 2, RB_SORT = 4 };
+enum RebuildMode { RB_ALL = 1, RB_NONE = 2, RB_SORT = 4, RB_QUIET = 8 };
 
 template <typename T, int BLOCK>
 __device__ bool rebuild(const SysDev &S, int &set, int &cur, unsigned &gen, int nloc,
@@ -831,11 +832,8 @@ __device__ bool rebuild(const SysDev &S, int &set, int &cur, unsigned &gen, int 
     if (!grid_sync(bar, gen, S.timeout_ns)) return false;
     set ^= 1;
     cur = 0;
-    if (mode == RB_SORT) {
-        if (blockIdx.x == 0 && tid == 0) {
-            C->n_rebuilds += 1;
-            C->slab_order = 0;
-        }
+    if (mode & RB_SORT) {
+        if (blockIdx.x == 0 && tid == 0) C->slab_order = 0;
         return true;
     }
     // R7: neighbour lists.  Staged shapes: the chunk windows and lists of
@@ -866,7 +864,7 @@ __device__ bool rebuild(const SysDev &S, int &set, int &cur, unsigned &gen, int 
         if (__syncthreads_or(over) && tid == 0) atomicOr(&C->status, (int)DS_NBR_OVERFLOW);
     }
     if (blockIdx.x == 0 && tid == 0) {
-        C->n_rebuilds += 1;
+        C->n_rebuilds += mode & RB_QUIET ? 0 : 1;
         C->slab_order = 0;
     }
     if (!S.stage && !grid_sync(bar, gen, S.timeout_ns)) return false;

@@ -75,6 +75,7 @@ struct SlabDev {
     int32_t *slab_n;            // [g]: particles of each slab in the state written back
     long long *left;            // steps that the launch leaves to the global engine
     int32_t g, p_cap, h_cap, e_cap, ncells, threads, cluster;   // ncells: MD cells of the largest slab with its halo rows
+    int32_t counted;            // rebuilds that this launch adds to the count besides its own (0 or 1)
 };
 
 // Byte offsets of a slab's arrays in dynamic shared memory (after the
@@ -741,6 +742,7 @@ __global__ void __launch_bounds__(SLAB_THREADS<T, CL>, 1)
         s_next[tid] = S.n_equil + (t <= 0 ? 0 : (t + v - 1) / v * v);
     }
     double disp = S.disp_rep[0];
+    if (X.k == 0 && tid == 0) C->n_rebuilds += D.counted;
     bool ok = true;
     // ---- load: the slab's slots are contiguous, in the order of the cells'
     // sort or as a slab launch left them

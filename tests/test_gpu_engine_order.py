@@ -51,3 +51,48 @@ def test_walks_over_the_engines(mdlg, n):
         for u, v in zip(_observe(s), ref[k - 1]):
             assert np.array_equal(u, v), walk
         s.close()
+
+
+def _count(s):
+    return s.info().n_rebuilds
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_rebuild_count_does_not_depend_on_the_engine(mdlg, prec):
+    """Readouts, short calls, a changed shape, a checkpoint and a new state
+    between slab calls: the count after each is the global engine's."""
+    runs = []
+    for shape in (GLOBAL, SLAB):
+        s = _make(mdlg, 5000, prec)
+        c = [_count(s)]
+        s.tune(*shape)
+        for n in (40, 3, 60, 17, 1, 1, 90):
+            s.step(n)
+            c.append(_count(s))
+            s.get_raw()
+            c.append(_count(s))
+        s.step(50)
+        s.energy()
+        s.forces()
+        s.step(5)
+        c.append(_count(s))
+        s.tune(128, 1, shape[2])
+        s.get_raw()
+        s.step(30)
+        c.append(_count(s))
+        ck = s.checkpoint()
+        c.append(_count(s))
+        s.step(70)
+        s.restore(ck)
+        s.step(20)
+        c.append(_count(s))
+        st = s.get_state()
+        s.set_state(*st)
+        s.step(64)
+        c.append(_count(s))
+        runs.append((c, _observe(s)))
+        s.close()
+    assert runs[0][0] == runs[1][0]
+    assert runs[0][0][-1] > 10
+    for u, v in zip(runs[0][1], runs[1][1]):
+        assert np.array_equal(u, v)
