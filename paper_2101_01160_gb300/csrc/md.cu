@@ -6,6 +6,7 @@
 // returns to the host only at md_sync or at a readout.
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -1028,7 +1029,10 @@ int launch_persistent(md_system *s, long long nsteps, int force_rebuild, const l
     long long step0 = s->step;
     int phase = s->phase_half;
     void *args[] = {&s->sd, &step0, &nsteps, &phase, &force_rebuild, &left};
-    MD_CUDA_TRY(cudaMemsetAsync(&s->d_ctl->claims, 0, sizeof(unsigned long long), s->st));
+    // the steps' maxima and the chunk claims start from zero: the slot of the
+    // first step may hold a maximum from before another engine's steps
+    constexpr size_t from = offsetof(Control, vmax), to = offsetof(Control, claims) + sizeof(Control::claims);
+    MD_CUDA_TRY(cudaMemsetAsync(s->d_ctl->vmax, 0, to - from, s->st));
     MD_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3(s->grid), dim3(s->block), args, s->smem, s->st));
     return MD_OK;
 }
@@ -1650,7 +1654,6 @@ int md_checkpoint_load(md_system *s, const void *buf) {
         o += p.bytes;
     }
     MD_CUDA_TRY(cudaMemcpy(&s->d_ctl->n_rebuilds, &h.n_rebuilds, sizeof(long long), cudaMemcpyHostToDevice));
-    MD_CUDA_TRY(cudaMemset(s->d_ctl->vmax, 0, sizeof(s->d_ctl->vmax)));
     MD_CUDA_TRY(cudaMemset(s->sd.vmax_rep, 0, sizeof(unsigned) * 3 * (size_t)s->nrep));
     s->step = h.step;
     s->phase_half = h.phase_half;

@@ -67,9 +67,9 @@ struct Control {
     int set, cur;
     int slab_order;       // the state is in the order a slab launch left it in (SlabDev::slab_n), not sorted
     long long n_rebuilds;
-    unsigned vmax[3];     // global engine: per-step max |v| dt / half_skin (float bits), by step mod 3
+    unsigned vmax[3];     // global engine: per-step max |v| dt / half_skin (float bits), by step mod 3 (zeroed before a launch)
     unsigned pad1;
-    unsigned long long claims;   // global engine: chunk claims of this launch (zeroed before it)
+    unsigned long long claims;   // global engine: chunk claims of this launch (zeroed with vmax)
 };
 
 // Everything the kernels need, passed by value.

@@ -96,3 +96,30 @@ def test_rebuild_count_does_not_depend_on_the_engine(mdlg, prec):
     assert runs[0][0][-1] > 10
     for u, v in zip(runs[0][1], runs[1][1]):
         assert np.array_equal(u, v)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("between", [16, 17, 18])
+def test_velocity_bound_of_earlier_steps_is_not_used(mdlg, prec, between):
+    """Hot steps on the global engine, slab steps, then a cold state: the
+    maxima of the hot steps (each above half the skin) must not make the cold
+    steps rebuild, whichever slot of three they were left in."""
+    n, L = 4000, inputs.box_length(4000, 0.05)
+    hot, cold = inputs.lattice_gas_state(n, L, 20.0, seed=1), inputs.lattice_gas_state(n, L, 0.05, seed=1)
+    p = mdlg.make_params(n, L, precision=prec, skin=0.008, lg_every=(20,), lx=(int(L),))
+    runs = []
+    for shape in (GLOBAL, SLAB):
+        s = mdlg.System(p, hot.x, hot.y, hot.vx, hot.vy)
+        s.tune(*shape)
+        s.step(4)
+        s.step(between)
+        s.set_state(cold.x, cold.y, cold.vx, cold.vy)
+        c = _count(s)
+        s.step(1)
+        c = (c, _count(s))
+        s.step(5)
+        runs.append((c, _count(s), s.get_state()))
+        s.close()
+    assert runs[0][:2] == runs[1][:2] and runs[1][0][0] == runs[1][0][1]
+    for u, v in zip(runs[0][2], runs[1][2]):
+        assert np.array_equal(u, v)
