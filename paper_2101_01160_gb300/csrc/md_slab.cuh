@@ -47,7 +47,9 @@
 // room ends the launch for all slabs at that point, which is always one where
 // the state is consistent: the slabs write it back and *left says how many
 // steps remain; the global engine, launched behind every slab launch, runs
-// them (none as a rule: it then returns at once).
+// them (none as a rule: it then returns at once).  So does one whose list grows
+// beyond the caller's nbr_max at a rebuild: the global engine builds the lists
+// of that state again and reports it.
 #pragma once
 
 #include "md_kernels.cuh"
@@ -340,9 +342,9 @@ __device__ __forceinline__ int slab_member(const uint16_t *mem, const int32_t *c
 // inside a cell, then one run over the three cells of each stencil row whose
 // hits are kept as bits, so the entries are written as soon as the counts
 // before them are known.  FP32 distances; with T = double the radius is widened by
-// the bound of their rounding.  Returns whether they fit.
+// the bound of their rounding.  Returns whether they fit, none longer than kmax.
 template <typename T>
-__device__ bool slab_lists(const RepDev &R, const SlabDev &D, const SlabMem<T> &M, const SlabCta &X, int *s_w) {
+__device__ bool slab_lists(const RepDev &R, const SlabDev &D, const SlabMem<T> &M, const SlabCta &X, int kmax, int *s_w) {
     const int nc = R.nc, nt = (int)blockDim.x;
     const int G = X.g == 1 ? nc : (X.r1 - X.r0) + 2, ncells = G * nc;
     uint16_t *mem = M.mem();
@@ -470,7 +472,7 @@ __device__ bool slab_lists(const RepDev &R, const SlabDev &D, const SlabMem<T> &
                 cnt += __popcll(hit[q]);
                 if (q < 2) rows |= (uint32_t)min(cnt, 255) << (8 * q);
             }
-            over |= cnt > RES_MAXLIST;
+            over |= cnt > kmax;
         }
         int tot;
         const int at = e0 + block_excl_scan(cnt, s_w, &tot);
@@ -774,7 +776,8 @@ __global__ void __launch_bounds__(SLAB_THREADS<T, CL>, 1)
     if (!ok) return;
     if (!over) {
         slab_read_rows<T>(D, M, X);
-        over = slab_sync<CL>(S, D, X, !slab_lists<T>(R, D, M, X, s_w), ok);
+        // (lists between two rebuilds: the limit nbr_max is one of rebuilds)
+        over = slab_sync<CL>(S, D, X, !slab_lists<T>(R, D, M, X, RES_MAXLIST, s_w), ok);
         if (!ok) return;
     }
     if (over) {   // nothing was changed: all steps are left
@@ -975,7 +978,7 @@ __global__ void __launch_bounds__(SLAB_THREADS<T, CL>, 1)
             }
             slab_read_rows<T>(D, M, X);
         }
-        over = slab_sync<CL>(S, D, X, !slab_lists<T>(R, D, M, X, s_w), ok);
+        over = slab_sync<CL>(S, D, X, !slab_lists<T>(R, D, M, X, min(S.K, RES_MAXLIST), s_w), ok);
         if (!ok) return;
         if (over) {
             early = true;

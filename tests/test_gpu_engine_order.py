@@ -123,3 +123,34 @@ def test_velocity_bound_of_earlier_steps_is_not_used(mdlg, prec, between):
     assert runs[0][:2] == runs[1][:2] and runs[1][0][0] == runs[1][0][1]
     for u, v in zip(runs[0][2], runs[1][2]):
         assert np.array_equal(u, v)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_list_limit_is_reported_by_every_engine(mdlg, prec):
+    """A hexagonal cluster that contracts: its lists outgrow the default
+    capacity (24 entries here) in flight.  Before that the call succeeds, after
+    it md_sync reports MD_E_LIMIT, whichever engine runs."""
+    n, L = 3000, inputs.box_length(3000, 0.04)
+    a, c = 1.22, L / 2
+    hexes = np.array([(a * (i + 0.5 * (j % 2)), a * np.sqrt(0.75) * j) for i in range(-9, 10) for j in range(-10, 11)])
+    hexes = hexes[np.hypot(*hexes.T) < 5.6]
+    g = np.stack(np.meshgrid(*[(np.arange(70) + 0.5) * (L / 70)] * 2), -1).reshape(-1, 2)
+    g = g[np.hypot(*(g - c).T) > 16.0][:n - len(hexes)]
+    x, y = np.concatenate([hexes + c, g]).T.copy()
+    vx, vy = np.concatenate([-5.0 * hexes, np.zeros_like(g)]).T.copy()
+    p = mdlg.make_params(len(x), L, precision=prec, skin=0.3, lg_every=(20,), lx=(int(L),))
+    codes = []
+    for shape in (GLOBAL, SLAB):
+        s = mdlg.System(p, x, y, vx, vy)
+        s.tune(*shape)
+        for k in range(10):
+            s.step(16)
+            try:
+                s.sync()
+                codes.append(0)
+            except mdlg.MDError as e:
+                codes.append(e.code)
+                break
+        s.close()
+    half = len(codes) // 2
+    assert codes[:half] == codes[half:] and codes[-1] == mdlg.MD_E_LIMIT and half >= 3, codes
