@@ -2009,7 +2009,9 @@ namespace {
 std::mutex g_tune_mu;
 std::map<std::tuple<int, int, int, int>, std::tuple<int, int, int>> g_tune_cache;
 std::map<std::tuple<int, int, int, int>, std::vector<double>> g_tune_costs;   // resident slab times
-std::map<std::tuple<int, int, int, int>, bool> g_tune_slab;   // the slab engine was the fastest
+// whether the slab engine was the fastest, kept by a system that has a plan for
+// it (of the systems under one key some have none)
+std::map<std::tuple<int, int, int, int>, bool> g_tune_slab;
 }
 
 int md_autotune(md_system *s, int64_t steps_per_trial, int32_t *best3) {
@@ -2029,7 +2031,8 @@ int md_autotune(md_system *s, int64_t steps_per_trial, int32_t *best3) {
                          : configure_launch(s, std::get<0>(it->second), std::get<1>(it->second),
                                             std::get<2>(it->second));
             if (rc) return rc;
-            s->slab_on = g_tune_slab[key];
+            const auto is = g_tune_slab.find(key);   // none: the library's choice, as without a tuner
+            s->slab_on = is == g_tune_slab.end() || is->second;
             if (best3) {
                 best3[0] = std::get<0>(it->second);
                 best3[1] = std::get<1>(it->second);
@@ -2128,7 +2131,7 @@ int md_autotune(md_system *s, int64_t steps_per_trial, int32_t *best3) {
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         g_tune_cache[key] = std::make_tuple(bb, bp, bs);
-        g_tune_slab[key] = slab;
+        if (s->slab_ok) g_tune_slab[key] = slab;
         g_tune_costs[key] = res_cost;
     }
     if (best3) {

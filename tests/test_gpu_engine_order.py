@@ -154,3 +154,30 @@ def test_list_limit_is_reported_by_every_engine(mdlg, prec):
         s.close()
     half = len(codes) // 2
     assert codes[:half] == codes[half:] and codes[-1] == mdlg.MD_E_LIMIT and half >= 3, codes
+
+
+def _slab_runs(s, n=50):
+    """Whether a call of n steps runs the slab engine."""
+    from torch.profiler import ProfilerActivity, profile
+
+    for _ in range(2):   # (the first profile of a process may record nothing)
+        s.sync()
+        with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            s.step(n)
+            s.sync()
+            torch.cuda.synchronize()
+        names = [e.name for e in prof.events() if "k_md_" in e.name]
+    assert names
+    return any("k_md_slab" in v for v in names)
+
+
+def test_tuner_cache_of_a_system_without_a_slab_plan(mdlg):
+    """520,000 particles have no slab plan, 270,000 have one and share the
+    tuner's key: the second system, tuned without trials, keeps the slab engine."""
+    big, small = (_make(mdlg, n, mdlg.MD_FP32_CELLOFF, 0.0784, 20.0, 0.5) for n in (520_000, 270_000))
+    best = big.autotune(16)
+    assert not _slab_runs(big)
+    assert small.autotune(16) == best and small.info().step == 0
+    assert _slab_runs(small)
+    big.close()
+    small.close()
