@@ -1556,8 +1556,9 @@ int md_tune(md_system *s, int32_t block_threads, int32_t per_thread, int32_t sta
     if (per_thread == 0) per_thread = default_ppt(s);
     const bool slab = staging == 0;   // the default: the slab engine where a single replica has a plan
     if (staging == 0) staging = 1;
-    if (staging >= 1 && staging <= 3) s->slab_on = slab;
-    return configure_launch(s, block_threads, per_thread, staging);
+    const int rc = configure_launch(s, block_threads, per_thread, staging);
+    if (rc == MD_OK && staging <= 3) s->slab_on = slab;   // (a refused call changes nothing)
+    return rc;
 }
 
 // ---- checkpoint ---------------------------------------------------------------

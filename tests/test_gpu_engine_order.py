@@ -181,3 +181,17 @@ def test_tuner_cache_of_a_system_without_a_slab_plan(mdlg):
     assert _slab_runs(small)
     big.close()
     small.close()
+
+
+def test_refused_tune_changes_nothing(mdlg):
+    s = _make(mdlg, 5000, mdlg.MD_FP32_CELLOFF)
+    for bad in ((100, 1, 1), (256, 9, 2), (256, 1, 5)):
+        with pytest.raises(mdlg.MDError):
+            s.tune(*bad)
+        assert _slab_runs(s)
+    s.tune(*GLOBAL)
+    for bad in ((100, 1, 0), (256, 9, 0)):
+        with pytest.raises(mdlg.MDError):
+            s.tune(*bad)
+        assert not _slab_runs(s)
+    s.close()
