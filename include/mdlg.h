@@ -242,6 +242,14 @@ int md_sync(md_system *s);
  * launch of at least 2 CTAs.  Synchronises. */
 int md_barrier_selftest(md_system *s, double limit_s);
 
+/* The same for the slab engine's exchange: one CTA leaves before it posts its
+ * word, the others' wait for it is limited to limit_s seconds, and the call
+ * returns MD_E_TIMEOUT.  No step is made: the state and the step count are as
+ * before, and the system stays usable.  MD_E_ARG for a system without a slab
+ * plan, or with one whose slabs are a single cluster (their barrier is the
+ * hardware's).  Synchronises. */
+int md_slab_selftest(md_system *s, double limit_s);
+
 int md_info(md_system *s, md_info_t *out);
 int md_rep_info(md_system *s, int32_t rep, md_rep_info_t *out);
 

@@ -1682,6 +1682,23 @@ int md_barrier_selftest(md_system *s, double limit_s) {
     return sync_status(s);
 }
 
+int md_slab_selftest(md_system *s, double limit_s) {
+    if (!s || !(limit_s > 0.0) || !(limit_s <= 4.0)) return fail(MD_E_ARG, "md_slab_selftest: bad arguments");
+    if (!s->slab_ok || s->sl.cluster || s->sl.g < 2)
+        return fail(MD_E_ARG, "md_slab_selftest: needs a system whose slabs meet through mailboxes");
+    int rc = sync_status(s);
+    if (rc) return rc;
+    if ((rc = ensure_sorted(s))) return rc;
+    const uint64_t keep = s->sd.timeout_ns;
+    s->sd.timeout_ns = (uint64_t)(limit_s * 1e9);
+    s->sd.dbg_leave_cta = 0;
+    rc = launch_slab(s, 1);
+    s->sd.dbg_leave_cta = -1;
+    s->sd.timeout_ns = keep;
+    if (rc) return rc;
+    return sync_status(s);
+}
+
 int md_sync(md_system *s) {
     if (!s) return fail(MD_E_ARG, "md_sync: NULL system");
     return sync_status(s);

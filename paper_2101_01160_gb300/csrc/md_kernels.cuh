@@ -114,8 +114,9 @@ struct SysDev {
     // force of the last step's force pass by particle id (md_step_forces), or
     // NULL in ordinary steps
     double *dbg_fx, *dbg_fy;
-    // md_barrier_selftest: this CTA leaves the kernel instead of arriving at
-    // the first step's grid barrier (-1 in every other launch)
+    // md_barrier_selftest, md_slab_selftest: this CTA leaves the kernel instead
+    // of arriving at the first step's grid barrier, or of posting its word at
+    // the first exchange (-1 in every other launch)
     int32_t dbg_leave_cta;
 };
 
@@ -1052,12 +1053,13 @@ __global__ void __launch_bounds__(BLOCK, md_min_ctas(BLOCK, DENSE)) k_md_persist
     __shared__ double s_dmax[BLOCK / 32];
     Control *C = S.ctl;
     // Behind a slab launch: the last *left steps, after a sort (an early end
-    // leaves the state unsorted); as a rule there are none.  (The kernel's
+    // leaves the state unsorted); as a rule there are none, and none after a
+    // wait that gave up (*left is then not written).  (The kernel's
     // parameters stay as they are, in constant memory: copies of them would
     // take registers of the 32-register budget.)
     long long it = 0;
     if (left) {
-        if (*left == 0 && C->slab_order) return;
+        if ((C->status & DS_TIMEOUT) || (*left == 0 && C->slab_order)) return;
         it = nsteps - *left;
     }
     const GridBarrier bar{&C->bar_count, &C->bar_gen, &C->status};

@@ -161,7 +161,9 @@ __device__ __forceinline__ unsigned long long *slab_mail(const SlabDev &D, const
 // next-but-one exchange's, of the same parity, is posted only after the next,
 // which a CTA posts after reading its mailbox of this one.  The wait is
 // bounded (S.timeout_ns): a CTA that waits longer flags DS_TIMEOUT, and every
-// CTA leaves the kernel at its next exchange (ok = false).
+// CTA leaves the kernel at its next exchange (ok = false).  A cluster meets at
+// the hardware's barrier instead: its CTAs run at the same time, and every one
+// makes the same exchanges (what they branch on is exchanged).
 template <bool CL>
 __device__ __forceinline__ unsigned slab_sync(const SysDev &S, const SlabDev &D, SlabCta &X, unsigned payload,
                                               bool &ok) {
@@ -771,6 +773,7 @@ __global__ void __launch_bounds__(SLAB_THREADS<T, CL>, 1)
         }
     }
     __syncthreads();
+    if (!CL && S.dbg_leave_cta == X.k) return;   // the self-test: one CTA never posts
     fits = slab_publish_rows<T>(D, M, X) && fits;
     unsigned over = slab_sync<CL>(S, D, X, !fits, ok);
     if (!ok) return;

@@ -73,6 +73,7 @@ _SIGS = {
     "md_step": ([P, C.c_int64], C.c_int),
     "md_sync": ([P], C.c_int),
     "md_barrier_selftest": ([P, C.c_double], C.c_int),
+    "md_slab_selftest": ([P, C.c_double], C.c_int),
     "md_resident_plan": ([C.POINTER(md_params), C.c_int32, C.c_int32, C.c_int64, P, C.c_int32, P, P], C.c_int),
     "md_tune": ([P, C.c_int32, C.c_int32, C.c_int32], C.c_int),
     "md_autotune": ([P, C.c_int64, P], C.c_int),
@@ -225,6 +226,11 @@ class System:
         """Return code of md_barrier_selftest (MD_E_TIMEOUT when the bounded
         barrier wait works); the system must be closed afterwards."""
         return int(load().md_barrier_selftest(self.h, float(limit_s)))
+
+    def slab_selftest(self, limit_s=0.02):
+        """Return code of md_slab_selftest (MD_E_TIMEOUT when the bounded wait
+        of the slab engine's exchange works); the system stays usable."""
+        return int(load().md_slab_selftest(self.h, float(limit_s)))
 
     def tune(self, block_threads=0, per_thread=0, staging=0):
         _check(load().md_tune(self.h, block_threads, per_thread, staging))
