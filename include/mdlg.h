@@ -579,6 +579,17 @@ int bf16_gemm_tn(const void *A, const void *B, float *C, int32_t M, int32_t N, i
 int bf16_gemm_selftest(const void *A, const void *B, float *C, int32_t M, int32_t N, int32_t K,
                        int32_t *status, double limit_s, void *stream);
 
+/* The same for the training kernels: the launches of mlp_grad on the batch
+ * (arguments as there) up to the one in which CTA 0 withholds a signal, its
+ * mbarrier waits limited to limit_s seconds (0 < limit_s <= 2).
+ * where in [1, 2 n_hidden]: the forward and backward chain, its where-th
+ * product; where -1: the weight gradients.  The CTA's waits run out, it waits
+ * (with the same limit) for the products and copies it issued, and the call
+ * returns MD_E_TIMEOUT (MD_OK would mean the limit failed).  Parameters and
+ * optimiser state are untouched, the model stays usable.  Synchronises. */
+int mlp_train_selftest(mlp_model *m, const float *X, const float *T, int32_t B, int32_t where, double limit_s,
+                       void *stream);
+
 /* Message of the calling thread's last failure ("" if none). */
 const char *md_last_error(void);
 

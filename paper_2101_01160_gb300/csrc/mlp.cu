@@ -674,6 +674,8 @@ struct TrainArgs {
     float *rowloss;                // [B]
     float inv_batch;
     int *status;
+    int dbg_skip;                  // mlp_train_selftest: CTA 0 does not signal product dbg_skip - 1
+    uint64_t dbg_wait_ns;          // and waits no longer than this; the others' limit stays, so they find its columns
 };
 
 constexpr int T_THREADS = 512;
@@ -731,7 +733,8 @@ __device__ __forceinline__ void cluster_sync() {
     asm volatile("fence.proxy.async;" ::: "memory");
 }
 
-template <int CS>
+// TEST: the kernel of mlp_train_selftest; the other has none of its checks.
+template <int CS, bool TEST>
 __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_constant__ TrainArgs a) {
     using S = TrainShape<CS>;
     extern __shared__ __align__(1024) unsigned char sm[];
@@ -739,7 +742,9 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
     uint64_t *full = reinterpret_cast<uint64_t *>(wbuf + S::NBUF * S::WBYTES);   // [NBUF]
     uint64_t *done = full + S::NBUF;                                            // accumulator complete
     uint64_t *arr = done + 1;                                                   // [2] the other CTAs' columns of an A operand are here
-    uint32_t *s_tmem = reinterpret_cast<uint32_t *>(arr + 2);
+    uint64_t *drain = arr + 2;                                                  // after a failed wait: what was issued is complete
+    uint32_t *s_tmem = reinterpret_cast<uint32_t *>(drain + 1);
+    uint32_t *s_bad = s_tmem + 1;                                               // a wait of some CTA gave up
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int rank = (int)cluster_rank(), m0 = (int)(blockIdx.x / CS) * 128;
     const ParamMap pm = a.pm;
@@ -754,7 +759,9 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
         umma::mbar_init(done, 1);
         umma::mbar_init(&arr[0], 1);
         umma::mbar_init(&arr[1], 1);
+        umma::mbar_init(drain, 1);
         umma::mbar_fence_init();
+        *s_bad = 0;
     }
     umma::fence_before();
     __syncthreads();
@@ -762,7 +769,12 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
     const uint32_t tmem = *s_tmem, trow = tmem + ((uint32_t)(quad * 32) << 16);
     const uint32_t act0 = umma::saddr(sm);
     bool bad = false;
-    uint32_t arr_par = 0;   // warp 0: parity of the next phase of arr[0], arr[1]
+    int loads = nops;       // weight slices that are requested (fewer after a failure)
+    uint32_t got = 0;       // warp 0: phases of arr[0] (low half) and arr[1] that have completed
+    const bool test = TEST && blockIdx.x == 0;
+    const auto wait = [&](uint64_t *bar, uint32_t parity) {
+        return umma::mbar_wait(bar, parity, test ? a.dbg_wait_ns : GEMM_WAIT_NS);
+    };
     // operation g reads operand g & 1 up to the output layer; the backward
     // pass starts over from the output layer's
     const auto a_buf = [&](int g) { return g < nl - 1 ? g & 1 : (g - 1) & 1; };
@@ -789,11 +801,11 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
         const int ns = (fwd ? pm.outp(l) : 256) / CS, K = fwd ? 256 : pm.outp(l), cur = a_buf(g);
         // waited for also after a failure: the copies always come, and no
         // CTA may leave before those into it have landed
-        if (!umma::mbar_wait(&arr[cur], arr_par >> cur & 1u, GEMM_WAIT_NS)) bad = true;
-        arr_par ^= 1u << cur;
-        bad = __any_sync(0xffffffffu, bad);
+        const bool here = __all_sync(0xffffffffu, wait(&arr[cur], got >> (16 * cur) & 1u));
+        got += here ? 1u << (16 * cur) : 0u;
+        bad = __any_sync(0xffffffffu, bad || !here);
         if (bad) return;
-        bad = __any_sync(0xffffffffu, !umma::mbar_wait(&full[g % S::NBUF], (g / S::NBUF) & 1, GEMM_WAIT_NS));
+        bad = __any_sync(0xffffffffu, !wait(&full[g % S::NBUF], (g / S::NBUF) & 1));
         if (bad) return;
         umma::fence_after();
         const uint32_t idesc = umma::idesc_bf16(128, ns);
@@ -806,15 +818,18 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
                     umma::mma(tmem, ad + (uint64_t)((kc * T_SLAB) >> 4) + (uint64_t)(k4 * 16),
                               bd + (uint64_t)((kc * ns * FK * 2) >> 4) + (uint64_t)(k4 * 16), idesc,
                               (kc | k4) ? 1u : 0u);
-            umma::commit(done);
+            if (!(test && a.dbg_skip == g + 1)) umma::commit(done);   // the self-test withholds one signal
         }
         __syncwarp();
     };
     // every thread: the operation's accumulator is complete; its weight buffer is free again
     const auto finish = [&](int g) {
-        if (!bad && !umma::mbar_wait(done, g & 1, GEMM_WAIT_NS)) bad = true;
+        if (!bad && !wait(done, g & 1)) bad = true;
         umma::fence_after();
-        if (tid == 0 && !bad) load(g + S::NBUF);
+        if (tid == 0) {
+            if (!bad) load(g + S::NBUF);
+            else loads = min(loads, g + S::NBUF);
+        }
     };
     // 16 BF16 values of row r, columns c .. c + 15 of the layer, into this CTA's operand `buf`
     const auto put = [&](int buf, int c, const uint32_t (&h)[8]) {
@@ -1035,15 +1050,32 @@ __global__ void __launch_bounds__(T_THREADS, 1) k_train_chain(const __grid_const
         }
         if (l > 1) send(a_buf(g + 1), my_slab, 1, 0, SLABS);
     }
-    cluster_sync();   // no CTA leaves while another may read or write its shared memory
     if (warp == 0) bad = __any_sync(0xffffffffu, bad);
+    if (bad)
+        for (int q = 0; q < CS; ++q) st_cluster(cluster_addr(umma::saddr(s_bad), q), 1.0f);
+    cluster_sync();   // no CTA leaves while another may read or write its shared memory
+    if (*reinterpret_cast<volatile uint32_t *>(s_bad)) {
+        // a CTA that gave up may have stopped waiting for columns: all are on
+        // their way now, and no CTA leaves before they have landed
+        if (warp == 0)
+            for (int b = 0; b < 2; ++b) {
+                int n = 0;
+                for (int g = 0; g < nops; ++g) n += a_buf(g) == b;
+                for (int i = (int)(got >> (16 * b) & 0xffffu); i < n; ++i)
+                    if (!wait(&arr[b], i & 1)) break;
+            }
+        cluster_sync();
+    }
     if (bad) {
-        // a wait gave up: products may still run; wait (with a limit) before
-        // their TMEM is freed, and flag it
+        // a wait gave up: products and weight copies may still run; wait (with
+        // a limit) before their TMEM and shared memory are given up, and flag it
         if (warp == 0 && umma::elect_one()) {   // the lane that issued
-            umma::commit(done);
-            umma::mbar_wait(done, nops & 1, GEMM_WAIT_NS);
+            umma::commit(drain);
+            wait(drain, 0);
         }
+        if (tid == 0)   // the last request of each buffer
+            for (int g = max(0, loads - S::NBUF); g < loads; ++g)
+                wait(&full[g % S::NBUF], (g / S::NBUF) & 1);
         atomicOr(a.status, 1);
     }
     umma::fence_before();
@@ -1066,6 +1098,8 @@ struct GradArgs {
     float *bpart;     // [chunk][layer * 256 + column]
     float *wpart;     // [chunk][256 * 4] first layer
     int *status;
+    uint64_t wait_ns; // limit of every mbarrier wait
+    int dbg_skip;     // mlp_train_selftest: CTA 0 does not signal stage dbg_skip - 1 (0: never)
 };
 constexpr int G_STAGES = 3;
 constexpr int G_STAGE_BYTES = 2 * 128 * GBK * 2;
@@ -1162,12 +1196,13 @@ __global__ void __launch_bounds__(128) k_train_grads(const __grid_constant__ Gra
             for (int k4 = 0; k4 < GBK / 16; ++k4)
                 umma::mma(tmem, umma::desc(a0 + k4 * 256, 128, 1024), umma::desc(b0 + k4 * 256, 128, 1024), idesc,
                           (kt | k4) ? 1u : 0u);
-            umma::commit(&mbar[s]);
+            // (the self-test withholds one signal)
+            if (!(a.dbg_skip == kt + 1 && blockIdx.x == 0)) umma::commit(&mbar[s]);
         }
         // the stage fetched next was last read by the products of stage kt - 1
         const int nx = kt + G_STAGES - 1;
         if (nx < nk) {
-            if (nx >= G_STAGES && !umma::mbar_wait(&mbar[nx % G_STAGES], (nx / G_STAGES - 1) & 1, GEMM_WAIT_NS)) s_ok = 0;
+            if (nx >= G_STAGES && !umma::mbar_wait(&mbar[nx % G_STAGES], (nx / G_STAGES - 1) & 1, a.wait_ns)) s_ok = 0;
             __syncthreads();
             if (!s_ok) break;
             fetch(nx);
@@ -1175,11 +1210,11 @@ __global__ void __launch_bounds__(128) k_train_grads(const __grid_constant__ Gra
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-    if (s_ok && !umma::mbar_wait(&mbar[(nk - 1) % G_STAGES], ((nk - 1) / G_STAGES) & 1, GEMM_WAIT_NS)) s_ok = 0;
+    if (s_ok && !umma::mbar_wait(&mbar[(nk - 1) % G_STAGES], ((nk - 1) / G_STAGES) & 1, a.wait_ns)) s_ok = 0;
     __syncthreads();
     if (!s_ok && warp == 0 && umma::elect_one()) {
         umma::commit(&mbar[G_STAGES]);
-        umma::mbar_wait(&mbar[G_STAGES], 0, GEMM_WAIT_NS);
+        umma::mbar_wait(&mbar[G_STAGES], 0, a.wait_ns);
     }
     __syncthreads();
     umma::fence_after();
@@ -1358,9 +1393,9 @@ int refresh_bf16(mlp_model *m, cudaStream_t st) {
     return MD_OK;
 }
 
-template <int CS>
+template <int CS, bool TEST>
 int chain_launch(const TrainArgs &a, cudaStream_t st) {
-    MD_CUDA_TRY(cudaFuncSetAttribute(k_train_chain<CS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    MD_CUDA_TRY(cudaFuncSetAttribute(k_train_chain<CS, TEST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)TrainShape<CS>::smem));
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeClusterDimension;
@@ -1373,12 +1408,15 @@ int chain_launch(const TrainArgs &a, cudaStream_t st) {
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    MD_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_train_chain<CS>, a));
+    MD_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_train_chain<CS, TEST>, a));
     return MD_OK;
 }
 
-// The three launches of a training step on B rows (B % 128 == 0).
-int train_launch(mlp_model *m, const float *X, const float *T, int B, float *loss, const AdamArgs &ad, cudaStream_t st) {
+// The three launches of a training step on B rows (B % 128 == 0).  The
+// self-test (dbg != 0) ends with the launch that withholds a signal: dbg > 0:
+// the chain, its product dbg - 1; dbg < 0: the gradients, a stage that is waited for.
+int train_launch(mlp_model *m, const float *X, const float *T, int B, float *loss, const AdamArgs &ad, cudaStream_t st,
+                 int dbg = 0, uint64_t wait_ns = GEMM_WAIT_NS) {
     int dev = 0, nsm = 0;
     MD_CUDA_TRY(cudaGetDevice(&dev));
     MD_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -1401,10 +1439,14 @@ int train_launch(mlp_model *m, const float *X, const float *T, int B, float *los
     t.rowloss = m->rowloss;
     t.inv_batch = 1.0f / (float)B;
     t.status = m->status;
+    t.dbg_skip = dbg;
+    t.dbg_wait_ns = wait_ns;
     // four CTAs per row block while the device has SMs for them, else two
     // (CTAs beyond the device then queue)
-    int rc = B / 128 * 4 <= nsm ? chain_launch<4>(t, st) : chain_launch<2>(t, st);
-    if (rc) return rc;
+    const bool four = B / 128 * 4 <= nsm;
+    int rc = dbg > 0 ? (four ? chain_launch<4, true>(t, st) : chain_launch<2, true>(t, st))
+                     : (four ? chain_launch<4, false>(t, st) : chain_launch<2, false>(t, st));
+    if (rc || dbg > 0) return rc;
     GradArgs g{};
     g.H = m->H;
     g.dZ = m->dZ;
@@ -1416,10 +1458,14 @@ int train_launch(mlp_model *m, const float *X, const float *T, int B, float *los
     g.bpart = m->bpart;
     g.wpart = m->wpart;
     g.status = m->status;
+    g.wait_ns = dbg < 0 ? wait_ns : GEMM_WAIT_NS;
+    const int nk = B / g.ks / GBK;
+    g.dbg_skip = dbg < 0 ? (nk > G_STAGES ? 1 : nk) : 0;
     const int nch = B / GRAD_ROWS;
     MD_CUDA_TRY(cudaFuncSetAttribute(k_train_grads, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GRADS_SMEM));
     k_train_grads<<<grad_tiles(g.pm) * g.ks + grad_sums(g.pm) / 128 * nch, 128, GRADS_SMEM, st>>>(g);
     MD_CUDA_TRY(cudaGetLastError());
+    if (dbg < 0) return MD_OK;
     UpdateArgs u{};
     u.pm = t.pm;
     u.part = m->part;
@@ -1608,6 +1654,19 @@ int mlp_status(mlp_model *m) {
         return fail(MD_E_TIMEOUT, "tensor-core GEMM wait timed out");
     }
     return MD_OK;
+}
+
+int mlp_train_selftest(mlp_model *m, const float *X, const float *T, int32_t B, int32_t where, double limit_s,
+                       void *stream) {
+    if (!m || !X || !T || B < 128 || B % 128 || where < -1 || where == 0 || where > 2 * (m->nl - 1) ||
+        !(limit_s > 0.0) || !(limit_s <= 2.0))
+        return fail(MD_E_ARG, "mlp_train_selftest: bad arguments");
+    int rc = ensure_ws(m, B);
+    if (rc) return rc;
+    AdamArgs ad{};
+    ad.g = m->g;
+    if ((rc = train_launch(m, X, T, B, nullptr, ad, (cudaStream_t)stream, where, (uint64_t)(limit_s * 1e9)))) return rc;
+    return mlp_status(m);
 }
 
 int bf16_gemm_selftest(const void *A, const void *B, float *C, int32_t M, int32_t N, int32_t K,

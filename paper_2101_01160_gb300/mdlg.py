@@ -122,6 +122,7 @@ _SIGS = {
     "mlp_grad": ([P, P, P, C.c_int32, P, P, P], C.c_int),
     "mlp_train_step": ([P, P, P, C.c_int32, C.c_float, P, P], C.c_int),
     "mlp_status": ([P], C.c_int),
+    "mlp_train_selftest": ([P, P, P, C.c_int32, C.c_int32, C.c_double, P], C.c_int),
     "bf16_gemm_tn": ([P, P, P, C.c_int32, C.c_int32, C.c_int32, P, P], C.c_int),
     "bf16_gemm_selftest": ([P, P, P, C.c_int32, C.c_int32, C.c_int32, P, C.c_double, P], C.c_int),
 }
@@ -637,6 +638,12 @@ class MLP:
 
     def status(self):
         _check(load().mlp_status(self.h))
+
+    def train_selftest(self, X, T, where, limit_s=0.02, stream=None):
+        """Return code of mlp_train_selftest (MD_E_TIMEOUT when the bounded
+        waits of the training kernels work); the model stays usable."""
+        return int(load().mlp_train_selftest(self.h, _ptr(X), _ptr(T), X.shape[0], int(where), float(limit_s),
+                                             _stream(stream)))
 
 
 def bf16_gemm_tn(A, B, stream=None):
