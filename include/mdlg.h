@@ -169,8 +169,8 @@ int md_init_batch(const md_params *p, int32_t n_rep, const double *x, const doub
 void md_destroy(md_system *s);
 
 /* Advances every replica by nsteps velocity-Verlet steps (Sec. 4) in one
- * persistent cooperative kernel (a single replica that fits the SMs' shared
- * memory, from 16 steps on: the slab engine, see md_tune), sampling the MDLG histograms (Sec. 2) on
+ * persistent cooperative kernel (longer calls of a single replica that fits the
+ * SMs' shared memory: the slab engine, see md_tune), sampling the MDLG histograms (Sec. 2) on
  * every step t = n_equil + m*lg_every[k] and rebuilding cell lists as
  * needed.  Asynchronous on the system's stream; device-side failures
  * (MD_E_TIMEOUT, MD_E_SKIN, MD_E_NONFINITE) are reported by md_sync. */
@@ -191,10 +191,11 @@ int md_step(md_system *s, int64_t nsteps);
  * per_thread are ignored; MD_E_LIMIT if a replica fits no slab plan.
  * staging 0 (and no md_tune at all) leaves the choice to the library: a
  * system of a single replica whose state fits the SMs' shared memory (about
- * 500,000 FP32 or 270,000 FP64 particles at phi = 0.08) runs calls of 16 steps
- * or more in the slab engine, which holds one slab of cell rows per SM in
- * shared memory for the whole call, in FP32 or FP64; everything else runs as
- * with staging 1.  Staging 1, 2 and 3 keep to the global engine.
+ * 500,000 FP32 or 270,000 FP64 particles at phi = 0.08) runs longer calls in
+ * the slab engine, which holds one slab of cell rows per SM in shared memory
+ * for the whole call, in FP32 or FP64: calls of 16 steps or more (FP32 above
+ * about 8,000 particles: 32), or of 8 (20) behind another slab call with no
+ * readout in between; everything else runs as with staging 1.  Staging 1, 2 and 3 keep to the global engine.
  * Results do not depend on the shape or the engine: particle order, force
  * summation order, every reduction order and the rebuild schedule (per
  * replica) are fixed by the data, not by the launch; only the FP64 moment
@@ -280,8 +281,8 @@ int md_set_state(md_system *s, const double *x, const double *y, const double *v
  * every engine, the FP64 moment sums too on the global engine (the resident
  * engine sums a slab's moment terms in its slot order, which a load resets,
  * so their last bits may differ; the slab engine's sums do not depend on the
- * order, but md_step calls must be split alike, since calls below 16 steps
- * run on the global engine).  The buffer format is that
+ * order, but md_step calls must be split alike, since short calls run on the
+ * global engine, see md_tune).  The buffer format is that
  * of this library build only. */
 int md_checkpoint_bytes(md_system *s, int64_t *bytes);
 int md_checkpoint_save(md_system *s, void *buf);

@@ -1195,13 +1195,19 @@ int launch_slab(md_system *s, long long nsteps) {
 }
 
 // A slab launch loads, builds its lists, writes back and is followed by the
-// (empty) global launch, about 25 us, and a readout after it has to sort; it
-// gains 2 to 30 us per step.  From this many steps on it is taken (and always
-// from a state that it left itself).
-constexpr int64_t SLAB_MIN_STEPS = 16;
+// (empty) global launch: 15 to 70 us more than a global launch costs.  A readout
+// or a short call after it has to sort: 20 to 90 us.  It gains 3 to 25 us per
+// step.  `enter`: steps from which a call pays for itself and the sort behind it,
+// from a sorted state; `stay`: steps from which a call pays for itself on a state
+// that the slab engine left.  Measured break-evens (1,024 to 262,144 particles, phi
+// 0.08 to 0.3): FP64 and clusters enter 8 to 16 (one case of 24), stay 4 to 8; the
+// FP32 grid enters 12 to 32 (one case of 40), stays 11 to 28.  Single steps behind a slab call,
+// FP32, 99,856 particles: 71 us each while they stayed, 20 now.
+int64_t slab_enter(const md_system *s) { return s->prec == MD_FP64 || s->sl.cluster ? 16 : 32; }
+int64_t slab_stay(const md_system *s) { return s->prec == MD_FP64 || s->sl.cluster ? 8 : 20; }
 
 bool takes_slab(const md_system *s, int64_t nsteps) {
-    return s->engine == 0 && s->slab_ok && s->slab_on && (s->slab_last || nsteps >= SLAB_MIN_STEPS);
+    return s->engine == 0 && s->slab_ok && s->slab_on && nsteps >= (s->slab_last ? slab_stay(s) : slab_enter(s));
 }
 
 int status_to_code(int ds) {
@@ -2101,7 +2107,7 @@ int md_autotune(md_system *s, int64_t steps_per_trial, int32_t *best3) {
         cudaEventElapsedTime(&ms, e0, e1);
         slab = ms < best_ms;
     }
-    if (steps_per_trial < SLAB_MIN_STEPS) slab = s->slab_ok;   // too short to have run there
+    if (steps_per_trial < slab_enter(s)) slab = s->slab_ok;   // too short to have run there
     s->slab_on = slab;
     // the shared-memory-resident engine (batched FP32 ensembles): a trial
     // with the modelled slab costs, then one with the schedule re-planned

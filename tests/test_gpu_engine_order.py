@@ -30,12 +30,12 @@ def _observe(s):
 @pytest.mark.parametrize("n", [4000, 12_000])   # slabs as one cluster, slabs as a grid; one and several resident slabs
 def test_walks_over_the_engines(mdlg, n):
     """All orders of three of slab, resident, global and readout, each step a
-    call of 20 steps, then the slab engine."""
+    call of 40 steps, then the slab engine."""
     ref = {}
     for k in range(1, 5):
         s = _make(mdlg, n, mdlg.MD_FP32_CELLOFF)
         s.tune(*GLOBAL)
-        s.step(20 * k)
+        s.step(40 * k)
         ref[k] = _observe(s)
         s.close()
     for walk in itertools.product("SRGO", repeat=3):
@@ -46,7 +46,7 @@ def test_walks_over_the_engines(mdlg, n):
                 s.get_raw()
                 continue
             s.tune(*{"S": SLAB, "R": RESIDENT, "G": GLOBAL}[op])
-            s.step(20)
+            s.step(40)
             k += 1
         for u, v in zip(_observe(s), ref[k - 1]):
             assert np.array_equal(u, v), walk
@@ -195,3 +195,24 @@ def test_refused_tune_changes_nothing(mdlg):
             s.tune(*bad)
         assert not _slab_runs(s)
     s.close()
+
+
+@pytest.mark.parametrize("n,prec,enter,stay", [(4000, 1, 16, 8), (20_000, 1, 32, 20), (20_000, 0, 16, 8)])
+def test_short_calls_leave_the_slab_engine(mdlg, n, prec, enter, stay):
+    """Calls too short to pay for a slab launch run on the global engine, also
+    behind a slab call, with the bits of the global engine alone."""
+    runs = []
+    for shape in (GLOBAL, SLAB):
+        s = _make(mdlg, n, prec)
+        s.tune(*shape)
+        ran = []
+        for k in (enter - 1, enter, stay, stay - 1, stay, 1, 1, 100, 1):
+            ran.append(_slab_runs(s, k))
+        runs.append((ran, _count(s), _observe(s)))
+        s.close()
+    assert not any(runs[0][0])
+    # (_slab_runs makes two calls of each)
+    assert runs[1][0] == [False, True, True, False, False, False, False, True, False]
+    assert runs[0][1] == runs[1][1]
+    for u, v in zip(runs[0][2], runs[1][2]):
+        assert np.array_equal(u, v)
