@@ -195,7 +195,9 @@ int md_step(md_system *s, int64_t nsteps);
  * the slab engine, which holds one slab of cell rows per SM in shared memory
  * for the whole call, in FP32 or FP64: calls of 16 steps or more (FP32 above
  * about 8,000 particles: 32), or of 8 (20) behind another slab call with no
- * readout in between; everything else runs as with staging 1.  Staging 1, 2 and 3 keep to the global engine.
+ * readout in between; not those of a state that has outgrown the slabs' room
+ * (found at the next synchronisation; tried again after 32 calls, then after
+ * twice as many each time); everything else runs as with staging 1.  Staging 1, 2 and 3 keep to the global engine.
  * Results do not depend on the shape or the engine: particle order, force
  * summation order, every reduction order and the rebuild schedule (per
  * replica) are fixed by the data, not by the launch; only the FP64 moment

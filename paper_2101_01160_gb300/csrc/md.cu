@@ -622,7 +622,7 @@ struct md_system {
     RepDev *d_reps = nullptr;
     int32_t *d_gran = nullptr;
     Control *d_ctl = nullptr;
-    int *h_status = nullptr;     // pinned: the status word's landing place
+    int *h_status = nullptr;     // pinned: the landing place of Control::status .. slab_ends
     double *d_epart = nullptr;
     double *d_small = nullptr;   // readout scratch (2*nb + 8 doubles, 4 energy)
     long long *d_hist64 = nullptr;
@@ -646,6 +646,11 @@ struct md_system {
     SlabDev sl{};
     size_t slab_smem = 0;
     bool slab_ok = false, slab_on = true, slab_last = false;
+    // A state that outgrows the slabs' room makes every slab launch a detour: after
+    // a synchronisation that finds one ended early, the next slab_wait calls that
+    // would take the engine run globally; twice as many after each such try
+    int slab_ends = 0, slab_wait = 0, slab_backoff = 0;
+    bool slab_tried = false;     // a slab launch since the last synchronisation
     std::vector<void *> res_allocs;
     ResDev rd{};
     int res_grid = 0;
@@ -1191,6 +1196,7 @@ int launch_slab(md_system *s, long long nsteps) {
     if (rc) return rc;
     s->needs_sort = true;
     s->slab_last = true;
+    s->slab_tried = true;
     return MD_OK;
 }
 
@@ -1206,8 +1212,12 @@ int launch_slab(md_system *s, long long nsteps) {
 int64_t slab_enter(const md_system *s) { return s->prec == MD_FP64 || s->sl.cluster ? 16 : 32; }
 int64_t slab_stay(const md_system *s) { return s->prec == MD_FP64 || s->sl.cluster ? 8 : 20; }
 
-bool takes_slab(const md_system *s, int64_t nsteps) {
-    return s->engine == 0 && s->slab_ok && s->slab_on && nsteps >= (s->slab_last ? slab_stay(s) : slab_enter(s));
+bool takes_slab(md_system *s, int64_t nsteps) {
+    if (s->engine != 0 || !s->slab_ok || !s->slab_on || nsteps < (s->slab_last ? slab_stay(s) : slab_enter(s)))
+        return false;
+    if (s->slab_wait == 0) return true;
+    --s->slab_wait;
+    return false;
 }
 
 int status_to_code(int ds) {
@@ -1221,11 +1231,20 @@ int status_to_code(int ds) {
     return MD_OK;
 }
 
+constexpr size_t STATUS_BYTES = offsetof(Control, slab_ends) + sizeof(int) - offsetof(Control, status);
+
 int sync_status(md_system *s) {
     // the status word follows the work into pinned memory: one wait
-    MD_CUDA_TRY(cudaMemcpyAsync(s->h_status, &s->d_ctl->status, sizeof(int), cudaMemcpyDeviceToHost, s->st));
+    MD_CUDA_TRY(cudaMemcpyAsync(s->h_status, &s->d_ctl->status, STATUS_BYTES, cudaMemcpyDeviceToHost, s->st));
     MD_CUDA_TRY(cudaStreamSynchronize(s->st));
-    const int ds = *s->h_status;
+    const int ds = *s->h_status, ends = s->h_status[STATUS_BYTES / sizeof(int) - 1];
+    if (s->slab_tried) {
+        const bool early = ends != s->slab_ends;
+        s->slab_backoff = early ? std::min(std::max(32, 2 * s->slab_backoff), 1 << 20) : 0;
+        s->slab_wait = s->slab_backoff;
+    }
+    s->slab_ends = ends;
+    s->slab_tried = false;
     if (ds) {
         MD_CUDA_TRY(cudaMemset(&s->d_ctl->status, 0, sizeof(int)));
         // a wait that gave up leaves the arrival count behind; no kernel of
@@ -1300,6 +1319,8 @@ int upload_state(md_system *s, const double *x, const double *y, const double *v
     scratch_free(tmp, s->st);
     if (rc) return rc;
     s->phase_half = 0;
+    s->slab_wait = s->slab_backoff = 0;   // another state, another chance
+    s->slab_tried = false;
     // a state placed on a sampling boundary starts the next window there
     unsigned mask = 0;
     for (int k = 0; k < s->n_lg; ++k)
@@ -1441,7 +1462,7 @@ int md_init_batch(const md_params *p, int32_t n_rep, const double *x, const doub
     ALLOC(s->d_hist64, sizeof(long long) * s->nb);
     ALLOC(s->d_nc_of_id, sizeof(int32_t) * s->ntot);
 #undef ALLOC
-    if (rc == MD_OK && cudaMallocHost((void **)&s->h_status, sizeof(int)) != cudaSuccess) {
+    if (rc == MD_OK && cudaMallocHost((void **)&s->h_status, STATUS_BYTES) != cudaSuccess) {
         s->h_status = nullptr;
         rc = fail(MD_E_NOMEM, "md_init_batch: pinned memory");
     }
@@ -1666,6 +1687,7 @@ int md_checkpoint_load(md_system *s, const void *buf) {
     s->phase_half = h.phase_half;
     s->needs_sort = s->sort_counts = true;
     s->slab_last = false;
+    s->slab_wait = s->slab_backoff = 0;
     rc = ensure_sorted(s);
     if (rc) return rc;
     return sync_status(s);

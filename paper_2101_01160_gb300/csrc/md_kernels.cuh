@@ -66,6 +66,8 @@ struct Control {
     int status;
     int set, cur;
     int slab_order;       // the state is in the order a slab launch left it in (SlabDev::slab_n), not sorted
+    int slab_ends;        // slab launches that ended early (the host reads status .. slab_ends in one copy)
+    int pad0;
     long long n_rebuilds;
     unsigned vmax[3];     // global engine: per-step max |v| dt / half_skin (float bits), by step mod 3 (zeroed before a launch)
     unsigned pad1;

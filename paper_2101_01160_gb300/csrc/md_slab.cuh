@@ -784,7 +784,10 @@ __global__ void __launch_bounds__(SLAB_THREADS<T, CL>, 1)
         if (!ok) return;
     }
     if (over) {   // nothing was changed: all steps are left
-        if (X.k == 0 && tid == 0) *D.left = nsteps;
+        if (X.k == 0 && tid == 0) {
+            *D.left = nsteps;
+            C->slab_ends += 1;
+        }
         return;
     }
     long long it = 0;
@@ -1025,6 +1028,7 @@ __global__ void __launch_bounds__(SLAB_THREADS<T, CL>, 1)
         // a state left early is sorted by the global engine, which then runs
         // the steps left (possibly none)
         C->slab_order = !early;
+        C->slab_ends += early;
         *D.left = nsteps - it;
         S.disp_rep[0] = disp;
     }

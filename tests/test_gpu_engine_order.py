@@ -216,3 +216,32 @@ def test_short_calls_leave_the_slab_engine(mdlg, n, prec, enter, stay):
     assert runs[0][1] == runs[1][1]
     for u, v in zip(runs[0][2], runs[1][2]):
         assert np.array_equal(u, v)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_state_without_room_leaves_the_slab_engine(mdlg, prec):
+    """All particles in a band of rows that outgrows the slabs' room: found at
+    the first synchronisation, the next 32 calls go to the global engine at once,
+    then one tries again, then 64; a new state gets its chance at once."""
+    n, L = 4000, inputs.box_length(4000, 0.05)
+    st = inputs.lattice_gas_state(n, L, 1.0, seed=4)
+    k = np.arange(n)
+    p = mdlg.make_params(n, L, precision=prec, skin=0.4, lg_every=(50,), lx=(int(L),))
+    p.nbr_max = 200
+    s = mdlg.System(p, (k % 200 + 0.5) * (L / 200), 20.0 + 1.3 * (k // 200), 0.05 * st.vx, 0.05 * st.vy)
+    s.tune(*SLAB)
+    s.step(32)
+    s.sync()
+    assert not _slab_runs(s, 32)              # two calls
+    for _ in range(29):
+        s.step(32)
+    assert not _slab_runs(s, 1)
+    s.step(32)                                # the 32nd
+    s.step(32)                                # the try
+    s.sync()
+    for _ in range(32):
+        s.step(32)
+    assert not _slab_runs(s, 32)
+    s.set_state(st.x, st.y, st.vx, st.vy)
+    assert _slab_runs(s, 32)
+    s.close()
