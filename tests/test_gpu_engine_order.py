@@ -245,3 +245,16 @@ def test_state_without_room_leaves_the_slab_engine(mdlg, prec):
     s.set_state(st.x, st.y, st.vx, st.vy)
     assert _slab_runs(s, 32)
     s.close()
+
+
+def test_tuner_compares_engines_on_one_state(mdlg):
+    """FP64 on a fresh lattice start, where a global step costs half of what it
+    costs later (16,384 particles: 10 us against 19; slab 11): the slab engine,
+    the faster one from then on, is chosen."""
+    L = inputs.box_length(16_384, 0.0784)
+    st = inputs.lattice_gas_state(16_384, L, 20.0, seed=5)
+    p = mdlg.make_params(16_384, L, precision=mdlg.MD_FP64, lg_every=(400,), lx=(int(L),))
+    s = mdlg.System(p, st.x, st.y, st.vx, st.vy)
+    s.autotune(50)
+    assert _slab_runs(s)
+    s.close()
