@@ -9,10 +9,14 @@
 //   * lattice cells are decided in FP32 where that provably gives the FP64
 //     cell (lattice_floor_f32);
 //   * the displacement is taken in the cell frame, wrap(c1 - c0) h + (o1 -
-//     o0), and its powers are formed and summed in pairs of FP32 values
-//     (about 48 bits; h split in three parts, error terms by fused
-//     multiply-adds and Knuth's two-sum), each thread's sums becoming FP64
-//     once at its end.  FP64 offsets, displacements within 1 % of half the
+//     o0), and its powers are formed as pairs of FP32 values (h split in three
+//     parts, error terms by fused multiply-adds): a square is off by at most
+//     3 2^-48 of itself, a fourth power by 9 2^-48.  They are summed in three
+//     FP32 values by Knuth's two-sum, which catches what every addition rounds
+//     off, however many particles a thread takes; each thread's sums become
+//     FP64 once at its end.  (With the low part of the fourth moments added
+//     plainly an addition's error did not average out: 1e-12 after 220 equal
+//     displacements.  Catching it costs 4 us of 96.)  FP64 offsets, displacements within 1 % of half the
 //     box (where the nearest image is a choice), below 2^-20 of the cell
 //     edge (whose fourth power would leave FP32's range) or not finite go
 //     through FP64;
@@ -22,14 +26,14 @@
 //     cluster does everything and its first CTA adds the others' results
 //     through distributed shared memory: no memsets, no scratch, no second
 //     kernel.  Above it, a one-wave grid with per-CTA moment partials that a
-//     one-block kernel sums in CTA order, so results do not depend on
-//     scheduling.
-// What bounds it now is the instruction rate: 317 warp instructions per 32
-// particles before the moments' third terms, issue slots 73 % busy, DRAM at a
-// quarter of its rate.
+//     one-block kernel sums with fixed strides and a fixed tree, so results do
+//     not depend on scheduling.
+// What bounds it now is the instruction rate: more than 317 warp instructions
+// per 32 particles (counted before the moments' third terms), issue slots 73 %
+// busy, DRAM at a quarter of its rate.
 // Measured (6.4M FP32 particles, W = 4): 1016 us per call with FP64 positions,
-// 64-bit remainders and an FP64 division per axis, 92 us now, the moments'
-// error against 64 bits 2.4e-16 -> 1.2e-16; 2047 FP64 particles alone 257 ->
+// 64-bit remainders and an FP64 division per axis, 96 us now, the moments'
+// error against 64 bits at most 1.2e-16 on four inputs; 2047 FP64 particles alone 257 ->
 // 80 us with the host's part (memsets, allocation and a second kernel gone).
 #include <cooperative_groups.h>
 
@@ -128,8 +132,9 @@ __device__ __forceinline__ void bin_moments(const BinParams &P, int c0, float o0
         const float z = __fmaf_rn(x2, eps, __fmul_rn(y, y));   // what q + r lacks
         S.c2 = __fadd_rn(S.c2, __fadd_rn(z, __fadd_rn(f, k)));
         two_sum(S.a4, u, S.a4, e);
-        S.b4 = __fadd_rn(S.b4, __fadd_rn(e, v));
-        S.c4 = __fadd_rn(S.c4, __fmaf_rn(q2, z, __fmul_rn(r, r)));
+        two_sum(e, v, e, f);
+        two_sum(S.b4, e, S.b4, k);
+        S.c4 = __fadd_rn(S.c4, __fadd_rn(__fmaf_rn(q2, z, __fmul_rn(r, r)), __fadd_rn(f, k)));
     } else if (!(x == 0.f && y == 0.f && eps == 0.f)) {
         S.add64(bin_disp64(c1, (double)o1, c0, (double)o0, P.h, P.L));
     }
