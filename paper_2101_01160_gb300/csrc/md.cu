@@ -2120,21 +2120,27 @@ int md_autotune(md_system *s, int64_t steps_per_trial, int32_t *best3) {
     // again: the state has gone on since that shape's trial, and a step's cost
     // with it (the first trial runs on the caller's start, a lattice as a rule,
     // with few pairs in range: FP64, 262,144 particles, 39 us a step there and 71
-    // later, when the slab engine's 55 used to lose)
+    // later, when the slab engine's 55 used to lose).  Twice in turn: a trial of 50
+    // steps holds one rebuild or two.  Near ties go to the slab engine, whose
+    // launch weighs less in a program's longer calls (86,281 FP32 particles: 0.49
+    // and 0.47-0.49 ms for 50 steps, 0.89 and 0.77 for 80 and a readout); short
+    // calls are kept from it by slab_enter.
     bool slab = false;
     if (rc == MD_OK && s->slab_ok && configure_launch(s, bb, bp, bs) == MD_OK) {
         float ms[2] = {0.0f, 0.0f};
         s->slab_wait = 0;
-        for (int k = 0; k < 2 && rc == MD_OK; ++k) {
-            s->slab_on = k == 1;
+        for (int k = 0; k < 4 && rc == MD_OK; ++k) {
+            s->slab_on = k & 1;
             rc = md_step(s, steps_per_trial);
             cudaEventRecord(e0, s->st);
             if (rc == MD_OK) rc = md_step(s, steps_per_trial);
             cudaEventRecord(e1, s->st);
             cudaEventSynchronize(e1);
-            cudaEventElapsedTime(&ms[k], e0, e1);
+            float t = 0.0f;
+            cudaEventElapsedTime(&t, e0, e1);
+            ms[k & 1] += t;
         }
-        slab = ms[1] < ms[0];
+        slab = ms[1] < 1.05f * ms[0];
     }
     if (steps_per_trial < slab_enter(s)) slab = s->slab_ok;   // too short to have run there
     s->slab_on = slab;
