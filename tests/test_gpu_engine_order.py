@@ -258,3 +258,23 @@ def test_tuner_compares_engines_on_one_state(mdlg):
     s.autotune(50)
     assert _slab_runs(s)
     s.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_moment_sums_of_the_engines(mdlg, prec):
+    """The engines group the FP64 moment terms differently.  Every grouping adds a
+    term to others at most 5 times inside a warp, once per window, and at most 2 +
+    8 times in the readout (157 warps or fewer slabs over 256 threads), each
+    addition within 2^-53 of its result; all terms are positive."""
+    st = []
+    for shape in (GLOBAL, SLAB):
+        s = _make(mdlg, 5000, prec)
+        s.tune(*shape)
+        s.step(100)
+        s.step(100)
+        st.append([s.feq_measured(0, k, 0)[2] for k in range(2)])
+        s.close()
+    for a, b in zip(*st):
+        assert a.n_windows == b.n_windows > 0
+        bar = 2 * (15 + a.n_windows) * 2.0 ** -53
+        assert abs(a.mu2 - b.mu2) <= bar * a.mu2 and abs(a.mu4 - b.mu4) <= bar * a.mu4
