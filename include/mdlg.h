@@ -119,7 +119,7 @@ typedef struct md_snapshot {
 typedef struct md_info_t {
     int64_t n_total;       /* particles over all replicas                   */
     int64_t step;          /* completed MD steps                            */
-    int64_t n_rebuilds;    /* cell-list rebuilds so far                     */
+    int64_t n_rebuilds;    /* cell-list rebuilds so far, on any engine      */
     int32_t n_rep;
     int32_t precision;
     int32_t grid_blocks;   /* persistent-kernel CTAs                        */
@@ -208,10 +208,15 @@ int md_tune(md_system *s, int32_t block_threads, int32_t per_thread, int32_t sta
 /* Autotuner: times md_step(steps_per_trial) twice for every launch shape
  * (block {256,128} x per_thread {1,2,4} x staging {1,2,3}; 3 skipped in
  * FP64; then the slab engine for a single replica, or staging 4 for FP32
- * batches of >= 2 replicas) and keeps the fastest (best3 names the fastest
- * global shape also where the slab engine was faster still); the choice is cached for the process by (precision, replicas,
- * particle count rounded up to a power of two, list capacity) and reused
- * without trials.  The trial steps are real MD steps: the system advances
+ * batches of >= 2 replicas) and keeps the fastest.  best3 names the fastest
+ * global shape also where the slab engine was faster still, and md_tune with
+ * such a shape keeps to the global engine: a program that wants the same choice
+ * on another system calls md_autotune there (no trials for a cached size), or
+ * md_tune with staging 0, the library's choice.  The slab engine is timed
+ * against the fastest global shape, twice in turn, and kept unless it is more
+ * than 5 % slower.  The choice is cached for the process by (precision,
+ * replicas, particle count rounded up to a power of two, list capacity) and
+ * reused without trials.  The trial steps are real MD steps: the system advances
  * by them (the trajectory itself does not depend on the shape).  best3
  * (host, may be NULL) receives {block_threads, per_thread, staging}.
  * Synchronises. */

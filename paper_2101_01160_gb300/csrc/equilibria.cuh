@@ -46,10 +46,12 @@ __host__ __device__ inline int wsg_cmin(double lam) {
 // cos(2 pi / k))) (the roots-of-unity filter); the factors they multiply vary
 // over c ~ lambda, slower than the weights' width sqrt(lambda), except near
 // c = 0, where the weight is exp(-lambda).  From lambda = 40 on with k =
-// floor(0.45 sqrt(lambda)) the sums agree with the full ones to 6e-20
-// relative for probabilities above 1e-25 and 1e-11 above 1e-50 (40-digit
-// arithmetic, a^2 from 0.003 to 4), and no window holds more than 137 terms,
-// where lambda = 1e5 had 7,631.
+// floor(0.45 sqrt(lambda)) the sums agree with the full ones to 1e-18 relative
+// for probabilities above 1e-25 (40-digit arithmetic, lambda from 40 to 2,000,
+// a^2 from 1e-4 to 20, |v| up to 10), and no window holds more than 137 terms,
+// where lambda = 1e5 had 7,631.  (From about 1e-40 down the sum leans on its last
+// terms and the two part, 1 % at 1e-46; FP64 has nothing there: the differences
+// of error functions that a factor is made of are off by 1e-16.)
 __host__ __device__ inline int wsg_stride(double lam) {
     return lam >= 40.0 ? (int)floor(0.45 * sqrt(lam)) : 1;
 }

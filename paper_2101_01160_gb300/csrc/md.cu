@@ -1118,9 +1118,10 @@ int plan_slab(md_system *s, bool may_cluster = true) {
     // FP64 is bound by its pipe, so the fullest slab counts (whole rows: up to
     // twice the mean), and long lists leave the global engine fewer idle lanes.
     // Microseconds per step of both, fitted to runs from 1,024 to 262,144
-    // particles at phi 0.08 to 0.3 (e.g. 262,144 at 0.08: 44 against 71 us;
-    // 99,856 at 0.2: 57 against 66; 150,000 at 0.3: 139 against 86; 16,384 at
-    // 0.3: 30 against 25).  FP32 slabs were faster at all of them.
+    // particles at phi 0.08 to 0.3 (on starts of few collisions, 262,144 at 0.08:
+    // 44 against 71 us; 99,856 at 0.2: 57 against 66; 150,000 at 0.3: 139 against
+    // 86; 16,384 at 0.3: 30 against 25; both grow with the gas's correlations, 56
+    // and 93 at 262,144).  FP32 slabs were faster at all of them.
     if (s->prec == MD_FP64) {
         const long long chunks = (R.n + 255) / 256, waves = (chunks + 2 * s->nsm - 1) / (2 * s->nsm);
         const double slab = 5.0 + pmax * (0.0091 * cbar - 0.0054);

@@ -3,8 +3,8 @@
 // FP32 and FP64.  Included by md.cu only.
 //
 // The replica is cut into as many horizontal slabs of whole MD-cell rows as
-// there are SMs (at least two rows each), one slab per CTA for the whole
-// launch.  What a step of the global engine spends on a system of up to a few
+// there are SMs (of two rows or more in FP32, of one or more in FP64), one slab
+// per CTA for the whole launch.  What a step of the global engine spends on a system of up to a few
 // hundred thousand particles is latency: list and position gathers through L2
 // and a barrier of 600 CTAs.  Here the gathers are shared-memory reads and the
 // CTAs exchange three things per step, each through one L2 round trip:
@@ -22,11 +22,12 @@
 // particle), then, after a CTA barrier, drift in place, so offsets are held
 // once.
 //
-// Measured per step, against the best global shape (phi 0.0784, T 20): FP32
-// 1,024 particles 6.8 -> 3.2 us, 99,856 10.3 -> 8.0 us, 262,144 16.2 -> 9.9 us;
-// FP64 1,024 13.3 -> 6.3 us, 99,856 39 -> 23 us, 262,144 71 -> 44 us.  Of the
-// 9.9 us of 262,144 FP32 particles the forces take 2.9, the exchange 3.3, halo
-// and drift 2.1, the rebuilds (one in 22 steps) 1.6.
+// Measured per step, best of three global shapes -> slabs (phi 0.0784, T 20,
+// calls of 800 steps after 2,000): FP32 1,024 particles 6.0 -> 3.1 us, 99,856
+// 10.8 -> 7.6 us, 262,144 17.0 -> 10.5 us; FP64 1,024 11.7 -> 6.2 us, 99,856 42
+// -> 29 us, 262,144 93 -> 56 us.  By clock stamps in a run of 9.9 us a step
+// (262,144 FP32 particles) the forces take 2.9, the exchange 3.3, halo and drift
+// 2.1, the rebuilds (one in 22 steps) 1.6.
 //
 // FP64.  GB300 issues one FP64 warp instruction per 15 clocks and SM, so what
 // counts is how many of its lanes work.  A warp first tests its particles'
@@ -59,9 +60,9 @@ namespace mdlg {
 
 constexpr int SLAB_MAX_THREADS = 768;
 // FP64 is bound by its pipe, which 16 warps keep busy with twice the registers,
-// and a cluster's CTAs hold a few hundred particles.  The FP32 grid's step does
-// not spill at 768 threads (80 registers); at 1,024 (64) it did: 262,144
-// particles 13.3 -> 13.1 us, 16,384 at phi 0.3 7.4 -> 6.6 us.
+// and a cluster's CTAs hold a few hundred particles.  The FP32 grid spills two
+// words at 768 threads (80 registers) and many at 1,024 (64): 262,144 particles
+// 13.3 -> 13.1 us, 16,384 at phi 0.3 7.4 -> 6.6 us.
 template <typename T, bool CL> constexpr int SLAB_THREADS = sizeof(T) == 8 || CL ? 512 : 768;
 constexpr int SLAB_CLUSTER = 16;        // most CTAs of a cluster
 constexpr int SLAB_MAX_IDX = 1 << 14;   // list entries: 14-bit index, 2-bit column tag

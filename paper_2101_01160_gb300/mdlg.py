@@ -237,6 +237,10 @@ class System:
         _check(load().md_tune(self.h, block_threads, per_thread, staging))
 
     def autotune(self, steps_per_trial=100):
+        """md_autotune: (block_threads, per_thread, staging) of the fastest
+        global shape (or staging 4).  Replayed by tune(), a shape of staging 1-3
+        keeps to the global engine; for the tuned choice on another system call
+        autotune() there, which makes no trials for a cached size."""
         best = np.zeros(3, np.int32)
         _check(load().md_autotune(self.h, int(steps_per_trial), _ptr(best)))
         return tuple(int(v) for v in best)
