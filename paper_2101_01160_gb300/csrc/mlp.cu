@@ -1318,7 +1318,7 @@ using namespace mdlg;
 // ---------------------------------------------------------------- model
 struct mlp_model {
     int nl = 0;                   // linear layers (hidden + 1)
-    int width = 256, ncls = 81, npad = 128, nin = 4;
+    int ncls = 81;
     float shift[4], scale[4];
     // FP32 master parameters, Adam moments and gradient, packed as `params`
     float *w = nullptr, *mom = nullptr, *var = nullptr, *g = nullptr;
@@ -1499,9 +1499,7 @@ int mlp_create(int32_t n_hidden, int32_t width, int32_t n_classes, const float *
         return fail(MD_E_ARG, "mlp_create: n_hidden in [2,15], width 256, classes in [2,112]");
     mlp_model *m = new mlp_model();
     m->nl = n_hidden + 1;
-    m->width = width;
     m->ncls = n_classes;
-    m->npad = 128;
     std::memcpy(m->shift, shift4, sizeof(m->shift));
     std::memcpy(m->scale, scale4, sizeof(m->scale));
     const ParamMap pm = m->map();
